@@ -40,7 +40,7 @@ def _sources():
 
 
 def _deps():
-    files = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    files = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     files.append(os.path.join(INCLUDE, "bf.h"))
     files.append(os.path.abspath(__file__))
     return files

@@ -173,33 +173,71 @@ static int interleaved_box(int wmax, int nf, int prec)
 
 // -------------------------------------------------------- envelope tables --
 
-static std::mutex g_env_mu;
-static std::map<std::pair<int, int>, std::shared_ptr<EnvTablesDev>> g_env_cache;  // (device, nz)
+// Transform tables are shared by the handles of a device: the twiddles of the
+// powers of two up to 8192 (n = 0: the level twiddles of bf_fft16.cuh), kept,
+// and the envelope factors of the depths and bands used last (at most
+// kEnvTablesKept; frames that use older ones hold them).
+static std::mutex g_tables_mu;
+static std::map<std::pair<int, int>, std::shared_ptr<FftTablesDev>> g_fft_tables;  // (device, n)
 
-static int env_tables(int nz, std::shared_ptr<EnvTablesDev> &out)
+struct EnvTablesKey {
+    int dev, nz, band, lo, hi;
+    bool operator==(const EnvTablesKey &o) const
+    {
+        return dev == o.dev && nz == o.nz && band == o.band && lo == o.lo && hi == o.hi;
+    }
+};
+constexpr size_t kEnvTablesKept = 256;
+static std::vector<std::pair<EnvTablesKey, std::shared_ptr<EnvTablesDev>>> g_env_tables;  // oldest first
+
+static int fft_tables(int n, std::shared_ptr<FftTablesDev> &out)
 {
     int dev = 0;
     cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lk(g_env_mu);
-    auto it = g_env_cache.find({dev, nz});
-    if (it != g_env_cache.end()) {
+    std::lock_guard<std::mutex> lk(g_tables_mu);
+    auto it = g_fft_tables.find({dev, n});
+    if (it != g_fft_tables.end()) {
         out = it->second;
         return BF_OK;
     }
-    EnvHost eh;
-    envelope_tables(nz, eh);
-    auto t = std::make_shared<EnvTablesDev>();
-    t->nz = nz;
-    t->fft_m = eh.fft_m;
-    t->bluestein = eh.bluestein;
-    int rc = t->tw.upload(eh.tw.data(), eh.tw.size() * sizeof(float));
-    if (!rc && eh.bluestein)
-        rc = t->chirp.upload(eh.chirp.data(), eh.chirp.size() * sizeof(float));
-    if (!rc && eh.bluestein)
-        rc = t->bhat.upload(eh.bhat.data(), eh.bhat.size() * sizeof(float));
+    std::vector<float> tw;
+    if (n == 0)
+        fft16_twiddles(tw);
+    else
+        fft_twiddles(n, tw);
+    auto t = std::make_shared<FftTablesDev>();
+    int rc = t->tw.upload(tw.data(), tw.size() * sizeof(float));
     if (rc)
         return rc;
-    g_env_cache[{dev, nz}] = t;
+    g_fft_tables[{dev, n}] = t;
+    out = t;
+    return BF_OK;
+}
+
+static int env_tables(int nz, bool band, int lo, int hi, std::shared_ptr<EnvTablesDev> &out)
+{
+    EnvTablesKey key{0, nz, band ? 1 : 0, band ? lo : 0, band ? hi : 0};
+    cudaGetDevice(&key.dev);
+    std::lock_guard<std::mutex> lk(g_tables_mu);
+    for (size_t i = g_env_tables.size(); i-- > 0;)
+        if (g_env_tables[i].first == key) {
+            out = g_env_tables[i].second;
+            std::rotate(g_env_tables.begin() + i, g_env_tables.begin() + i + 1, g_env_tables.end());
+            return BF_OK;
+        }
+    EnvHost eh;
+    envelope_tables(nz, band, lo, hi, eh);
+    auto t = std::make_shared<EnvTablesDev>();
+    t->lg = eh.lg;
+    t->conv = eh.conv;
+    int rc = t->gh.upload(eh.gh.data(), eh.gh.size() * sizeof(float));
+    if (!rc && band)
+        rc = t->gr.upload(eh.gr.data(), eh.gr.size() * sizeof(float));
+    if (rc)
+        return rc;
+    if (g_env_tables.size() >= kEnvTablesKept)
+        g_env_tables.erase(g_env_tables.begin());
+    g_env_tables.emplace_back(key, t);
     out = t;
     return BF_OK;
 }
@@ -462,12 +500,17 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     fp.map_dirty = s.map_dirty;
     fp.scratch = &s;
     if (stage != BF_OUT_RF && !iq) {
-        rc = env_tables(h->g.nz, fp.et);
+        const bool warp = envelope_warp_ok(h->g.nz);
+        rc = fft_tables(warp ? h->g.nz : 0, fp.ft);
+        if (!rc && !warp && (modes & ~BF_DMAS))
+            rc = env_tables(h->g.nz, false, 0, 0, fp.et[0]);
+        if (!rc && !warp && (modes & BF_DMAS))
+            rc = env_tables(h->g.nz, true, h->kb_lo, h->kb_hi, fp.et[1]);
         if (rc)
             return rc;
     }
     if (iq) {
-        rc = env_tables(ns, fp.dt);  // twiddles of the length-ns transforms
+        rc = fft_tables(ns, fp.dt);  // twiddles of the length-ns transforms
         if (rc)
             return rc;
     }
@@ -721,7 +764,6 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         g.rows = acc;
         hl.igroups.push_back(g);
     }
-    int cols = 0;
     long long blks = 0;
     for (const FramePrep &f : frames) {
         if (f.stage == BF_OUT_RF)
@@ -757,28 +799,25 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
             e.maxbits = f.maxbits + slot;
             e.nx = h->g.nx;
             e.nz = h->g.nz;
-            e.fft_m = f.et->fft_m;
-            e.bluestein = f.et->bluestein;
             e.band = bit == BF_DMAS ? 1 : 0;
             e.kb_lo = h->kb_lo;
             e.kb_hi = h->kb_hi;
-            e.tw = (const float2 *)f.et->tw.p;
-            e.chirp = (const float2 *)f.et->chirp.p;
-            e.bhat = (const float2 *)f.et->bhat.p;
-            e.cols_per_block = e.bluestein ? 1 : envelope_cols_per_block(e.fft_m);
-            e.vec4 = (!e.bluestein && e.nz % 4 == 0 && ((uintptr_t)e.y & 15) == 0 &&
-                      ((uintptr_t)e.env & 15) == 0)
-                         ? 1
-                         : 0;
-            if (envelope_warp_ok(e.nz, e.fft_m, e.bluestein)) {
+            if (envelope_warp_ok(e.nz)) {
+                e.tw = (const float2 *)f.ft->tw.p;
                 hl.envw_prefix.push_back(hl.envw_pairs);
                 hl.envw_pairs += (h->g.nx + 1) / 2;
                 hl.envw.push_back(e);
             } else {
-                hl.env_prefix.push_back(cols);
-                cols += (h->g.nx + e.cols_per_block - 1) / e.cols_per_block;
-                hl.env.push_back(e);
-                hl.env_smem = std::max(hl.env_smem, envelope_smem_bytes(e.fft_m, e.bluestein));
+                const EnvTablesDev &t = *f.et[e.band];
+                e.lg = t.lg;
+                e.conv = t.conv;
+                e.ptw = (const float2 *)f.ft->tw.p;
+                e.gr = (const float *)t.gr.p;
+                e.gh = (const float *)t.gh.p;
+                const int big = e.lg > 12 ? 1 : 0, per = 2 * envelope_pairs_per_block(e.lg);
+                hl.env_prefix[big].push_back(hl.env_blocks[big]);
+                hl.env_blocks[big] += (h->g.nx + per - 1) / per;
+                hl.env[big].push_back(e);
             }
             if (f.stage == BF_OUT_LOGDB) {
                 LogJob l{};
@@ -796,7 +835,6 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
             ++slot;
         }
     }
-    hl.env_blocks = cols;
     hl.log_blocks = (int)blks;
 }
 
@@ -816,8 +854,10 @@ int DeviceLaunch::upload(const HostLaunch &hl, cudaStream_t st, bool async)
     if (!rc) rc = put(tile_prefix, hl.tile_prefix.data(), hl.tile_prefix.size() * sizeof(int));
     if (!rc) rc = put(ingest, hl.ingest.data(), hl.ingest.size() * sizeof(IngestJob));
     if (!rc) rc = put(ingest_prefix, hl.ingest_prefix.data(), hl.ingest_prefix.size() * sizeof(int));
-    if (!rc) rc = put(env, hl.env.data(), hl.env.size() * sizeof(EnvJob));
-    if (!rc) rc = put(env_prefix, hl.env_prefix.data(), hl.env_prefix.size() * sizeof(int));
+    for (int b = 0; b < 2; ++b) {
+        if (!rc) rc = put(env[b], hl.env[b].data(), hl.env[b].size() * sizeof(EnvJob));
+        if (!rc) rc = put(env_prefix[b], hl.env_prefix[b].data(), hl.env_prefix[b].size() * sizeof(int));
+    }
     if (!rc) rc = put(envw, hl.envw.data(), hl.envw.size() * sizeof(EnvJob));
     if (!rc) rc = put(envw_prefix, hl.envw_prefix.data(), hl.envw_prefix.size() * sizeof(int));
     if (!rc) rc = put(log, hl.log.data(), hl.log.size() * sizeof(LogJob));
@@ -855,6 +895,17 @@ int upload_maps(std::vector<FramePrep> &frames, cudaStream_t st, bool async)
         }
     }
     return BF_OK;
+}
+
+// The envelope launches of a set of frames: 512-row images, then the others.
+static cudaError_t launch_envelopes(const HostLaunch &hl, DeviceLaunch &dl, cudaStream_t st)
+{
+    cudaError_t e = launch_envelope_warp((const EnvJob *)dl.envw.p, (const int *)dl.envw_prefix.p,
+                                         (int)hl.envw.size(), hl.envw_pairs, st);
+    for (int b = 1; b >= 0 && e == cudaSuccess; --b)
+        e = launch_envelope((const EnvJob *)dl.env[b].p, (const int *)dl.env_prefix[b].p,
+                            (int)hl.env[b].size(), hl.env_blocks[b], b == 1, st);
+    return e;
 }
 
 // The device work of a set of frames, in stream order: ingest, reset of the
@@ -922,18 +973,9 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     e = mark(2);
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
-    if (!hl.env.empty()) {
-        e = launch_envelope((const EnvJob *)dl.env.p, (const int *)dl.env_prefix.p, (int)hl.env.size(),
-                            hl.env_blocks, hl.env_smem, st);
-        if (e != cudaSuccess)
-            return cuda_fail(e, "envelope launch");
-    }
-    if (!hl.envw.empty()) {
-        e = launch_envelope_warp((const EnvJob *)dl.envw.p, (const int *)dl.envw_prefix.p,
-                                 (int)hl.envw.size(), hl.envw_pairs, st);
-        if (e != cudaSuccess)
-            return cuda_fail(e, "envelope launch");
-    }
+    e = launch_envelopes(hl, dl, st);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "envelope launch");
     if (!hl.log.empty()) {
         e = launch_log((const LogJob *)dl.log.p, (const int *)dl.blk_prefix.p, (int)hl.log.size(),
                        hl.log_blocks, 70.0f, st);
@@ -1240,10 +1282,10 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     std::vector<double> key{(double)n_samples, stolt ? 1.0 : 0.0};
     key.insert(key.end(), angles_rad, angles_rad + n_angles);
     const bool rebuild = key != h->fk_key;
-    std::shared_ptr<EnvTablesDev> tt, tk;
-    int rc = env_tables(nt, tt);
+    std::shared_ptr<FftTablesDev> tt, tk;
+    int rc = fft_tables(nt, tt);
     if (!rc)
-        rc = env_tables(nk, tk);
+        rc = fft_tables(nk, tk);
     const size_t nf = (size_t)nt / 2 + 1, img = (size_t)ne * n_samples;
     if (!rc)
         rc = h->fk_D.ensure((size_t)n_angles * nf * nk * sizeof(float2));
@@ -1367,16 +1409,8 @@ BF_API int bf_beamform_plain(bf_handle *h, const int16_t *rf_dev, int32_t n_samp
         rc = cudaMemsetAsync(frames[0].maxbits, 0, 4 * sizeof(unsigned), h->stream) == cudaSuccess
                  ? BF_OK
                  : fail(BF_ECUDA, "cudaMemsetAsync");
-    if (!rc && !hl.env.empty()) {
-        e = launch_envelope((const EnvJob *)h->launch.env.p, (const int *)h->launch.env_prefix.p,
-                            (int)hl.env.size(), hl.env_blocks, hl.env_smem, h->stream);
-        if (e != cudaSuccess)
-            rc = cuda_fail(e, "envelope launch");
-    }
-    if (!rc && !hl.envw.empty()) {
-        e = launch_envelope_warp((const EnvJob *)h->launch.envw.p,
-                                 (const int *)h->launch.envw_prefix.p, (int)hl.envw.size(),
-                                 hl.envw_pairs, h->stream);
+    if (!rc) {
+        e = launch_envelopes(hl, h->launch, h->stream);
         if (e != cudaSuccess)
             rc = cuda_fail(e, "envelope launch");
     }
@@ -1627,7 +1661,8 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
         if (e == cudaSuccess)
             e = cudaEventCreate(&m);
     b->launches = (int)b->hl.igroups.size() + (b->hl.demod.empty() ? 0 : 1) +
-                  (int)b->hl.groups.size() + (b->hl.env.empty() ? 0 : 1) + (b->hl.envw.empty() ? 0 : 1) +
+                  (int)b->hl.groups.size() + (b->hl.env[0].empty() ? 0 : 1) +
+                  (b->hl.env[1].empty() ? 0 : 1) + (b->hl.envw.empty() ? 0 : 1) +
                   (b->hl.log.empty() ? 0 : 1);
     if (e == cudaSuccess)
         e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);

@@ -85,9 +85,14 @@ struct Plan {
     DevMem maps;  // CUtensorMap[2]: valid rows, dx^2
 };
 
+// Device copies of transform tables: exp(-2 pi i k / n), and the spectral
+// factors of one depth (and band).
+struct FftTablesDev {
+    DevMem tw;
+};
 struct EnvTablesDev {
-    int nz = 0, fft_m = 0, bluestein = 0;
-    DevMem tw, chirp, bhat;
+    int lg = 0, conv = 0;
+    DevMem gr, gh;
 };
 
 // Device scratch of one in-flight frame: staged sample pairs, beamformed
@@ -110,8 +115,9 @@ struct FrameScratch {
 struct FramePrep {
     bf_handle *h = nullptr;
     Plan *plan = nullptr;
-    std::shared_ptr<EnvTablesDev> et;   // envelope transform tables (nz)
-    std::shared_ptr<EnvTablesDev> dt;   // demodulation transform tables (n_samples; IQ only)
+    std::shared_ptr<EnvTablesDev> et[2];  // envelope tables: without band, the DMAS band
+    std::shared_ptr<FftTablesDev> ft;     // level twiddles, or the warp kernel's 512-point table
+    std::shared_ptr<FftTablesDev> dt;     // demodulation transform tables (n_samples; IQ only)
     const int16_t *rf = nullptr;
     int ns = 0, na = 0, modes = 0, stage = 0, prec = 0;
     double pdas_p = 2.0;
@@ -141,10 +147,10 @@ struct HostLaunch {
     std::vector<IngestJob> ingest;
     std::vector<int> ingest_prefix;
     std::vector<IGroup> igroups;
-    std::vector<EnvJob> env;
-    std::vector<int> env_prefix;
-    int env_blocks = 0;
-    size_t env_smem = 0;
+    // envelopes of the other depths: [0] transforms of up to 4096 points, [1] of 8192
+    std::vector<EnvJob> env[2];
+    std::vector<int> env_prefix[2];
+    int env_blocks[2] = {0, 0};
     // 512-row images: the warp-per-column-pair envelope kernel (column pairs)
     std::vector<EnvJob> envw;
     std::vector<int> envw_prefix;
@@ -159,7 +165,7 @@ struct HostLaunch {
 };
 
 struct DeviceLaunch {
-    DevMem jobs, tile_prefix, ingest, ingest_prefix, env, env_prefix, log, blk_prefix, err;
+    DevMem jobs, tile_prefix, ingest, ingest_prefix, env[2], env_prefix[2], log, blk_prefix, err;
     DevMem envw, envw_prefix;
     DevMem demod, demod_prefix;
     int upload(const HostLaunch &hl, cudaStream_t st, bool async);

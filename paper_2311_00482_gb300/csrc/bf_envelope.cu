@@ -1,8 +1,13 @@
-// Warp-per-column-pair envelope kernel for 512-sample depths: the
-// analytic-signal envelope along depth of the B-mode display (Fig. 3), with
-// the DMAS image's [f0, 3 f0] band-pass, without block-wide barriers.
+// Envelope kernels: the analytic-signal envelope along depth of the B-mode
+// display (Fig. 3), with the DMAS image's [f0, 3 f0] band-pass.
 //
-// Two image columns a, b form one complex sequence z[n] = y_a[n] + i y_b[n]
+//   envelope_warp_kernel  512-row images: one warp per column pair, no block-wide
+//                         barriers
+//   envelope_kernel       every other depth: sixteen points per thread
+//                         (bf_fft16.cuh), power-of-two depths transformed as they
+//                         are, others convolved in a power-of-two transform
+//
+// Warp kernel.  Two image columns a, b form one complex sequence z[n] = y_a[n] + i y_b[n]
 // of length N = 512.  A warp transforms it with the four-step decomposition
 // n = 32 n1 + n2, k = k1 + 16 k2 (n1, k1 < 16; n2, k2 < 32):
 //   lane n2 holds z[32 n1 + n2] for all n1 (coalesced column loads),
@@ -26,7 +31,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "bf_fft.cuh"
+#include <type_traits>
+
+#include "bf_fft16.cuh"
 #include "bf_internal.h"
 
 namespace bfi {
@@ -38,165 +45,6 @@ constexpr int kR = 16, kN = 32 * kR;         // registers per lane, transform le
 // the lane pairs' strided accesses (row lane / 2, column 2 j + lane % 2) fall
 // on distinct banks.
 constexpr int kPitch = 34;
-
-// cos, sin of 2 pi e / 32 for e < 16
-__device__ __constant__ float2 kW32[16] = {
-    {1.000000000e+00f, 0.000000000e+00f},  {9.807852804e-01f, 1.950903220e-01f},
-    {9.238795325e-01f, 3.826834324e-01f},  {8.314696123e-01f, 5.555702330e-01f},
-    {7.071067812e-01f, 7.071067812e-01f},  {5.555702330e-01f, 8.314696123e-01f},
-    {3.826834324e-01f, 9.238795325e-01f},  {1.950903220e-01f, 9.807852804e-01f},
-    {0.000000000e+00f, 1.000000000e+00f},  {-1.950903220e-01f, 9.807852804e-01f},
-    {-3.826834324e-01f, 9.238795325e-01f}, {-5.555702330e-01f, 8.314696123e-01f},
-    {-7.071067812e-01f, 7.071067812e-01f}, {-8.314696123e-01f, 5.555702330e-01f},
-    {-9.238795325e-01f, 3.826834324e-01f}, {-9.807852804e-01f, 1.950903220e-01f}};
-
-// Complex add / subtract as one paired FP32 instruction (Blackwell f32x2):
-// the real and imaginary parts of a float2 sit in a register pair.
-__device__ __forceinline__ float2 c_add(float2 a, float2 b)
-{
-    unsigned long long ra, rb, rc;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rc) : "l"(ra), "l"(rb));
-    float2 c;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(rc));
-    return c;
-}
-
-__device__ __forceinline__ float2 c_sub(float2 a, float2 b)
-{
-    unsigned long long ra, rb, rc;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rc) : "l"(ra), "l"(rb));
-    float2 c;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(rc));
-    return c;
-}
-
-// (a.x^2 + b.x^2, a.y^2 + b.y^2): per half b^2 rounded, then one FMA.
-__device__ __forceinline__ float2 c_sqsum(float2 a, float2 b)
-{
-    unsigned long long ra, rb, rc;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-    asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(rc) : "l"(rb));
-    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(rc) : "l"(ra), "l"(rc));
-    float2 c;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(rc));
-    return c;
-}
-
-// Square root on the special-function unit (relative error about one unit in
-// the last place, far inside the envelope's tolerance).
-__device__ __forceinline__ float sqrt_fast(float x)
-{
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// s * a + b with s a scalar (both halves), as one paired FMA.
-__device__ __forceinline__ float2 c_sfma(float s, float2 a, float2 b)
-{
-    unsigned long long rs, ra, rb, rc;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(rs) : "f"(s));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(rc) : "l"(rs), "l"(ra), "l"(rb));
-    float2 c;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(rc));
-    return c;
-}
-
-// b * W_32^e (INV: conjugate), W_32 = exp(-2 pi i / 32), 0 <= e < 32; e is a
-// compile-time constant wherever this is used (quarter turns are swaps).
-template <bool INV>
-__device__ __forceinline__ float2 w32mul(float2 b, int e)
-{
-    if (e >= 16) {  // W_32^16 = -1
-        b = make_float2(-b.x, -b.y);
-        e -= 16;
-    }
-    if (e == 0)
-        return b;
-    if (e == 8)
-        return INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
-    const float2 w = kW32[e];
-    const float s = INV ? w.y : -w.y;
-    return make_float2(b.x * w.x - b.y * s, b.x * s + b.y * w.x);
-}
-
-// 4-point DFT in place: y_k = sum_n x_n W_4^(n k), W_4 = -i (INV: +i).
-template <bool INV>
-__device__ __forceinline__ void dft4(float2 &a, float2 &b, float2 &c, float2 &d)
-{
-    const float2 t0 = c_add(a, c), t1 = c_sub(a, c), t2 = c_add(b, d), u = c_sub(b, d);
-    a = c_add(t0, t2);
-    c = c_sub(t0, t2);
-    // t1 +- u W_4 (W_4 = -i, INV: +i): the swapped halves in scalar operations
-    if (INV) {
-        b = make_float2(t1.x - u.y, t1.y + u.x);
-        d = make_float2(t1.x + u.y, t1.y - u.x);
-    } else {
-        b = make_float2(t1.x + u.y, t1.y - u.x);
-        d = make_float2(t1.x - u.y, t1.y + u.x);
-    }
-}
-
-// In-register 16-point DFT, natural order in and out: x[k] <- sum_n x[n]
-// W_16^(n k) (INV: conjugate exponent, no scaling), as 4 x 4 with n = n1 + 4 n2
-// and k = 4 k1 + k2: DFTs over n2, twiddles W_16^(n1 k2), DFTs over n1, and a
-// transposed read-out (register renaming only).
-template <bool INV>
-__device__ __forceinline__ void dft16(float2 (&x)[16])
-{
-    dft4<INV>(x[0], x[4], x[8], x[12]);  // -> B[n1][k2] at n1 + 4 k2
-    dft4<INV>(x[1], x[5], x[9], x[13]);
-    dft4<INV>(x[2], x[6], x[10], x[14]);
-    dft4<INV>(x[3], x[7], x[11], x[15]);
-    x[5] = w32mul<INV>(x[5], 2);  // W_16^(n1 k2) = W_32^(2 n1 k2)
-    x[9] = w32mul<INV>(x[9], 4);
-    x[13] = w32mul<INV>(x[13], 6);
-    x[6] = w32mul<INV>(x[6], 4);
-    x[10] = w32mul<INV>(x[10], 8);
-    x[14] = w32mul<INV>(x[14], 12);
-    x[7] = w32mul<INV>(x[7], 6);
-    x[11] = w32mul<INV>(x[11], 12);
-    x[15] = w32mul<INV>(x[15], 18);
-    dft4<INV>(x[0], x[1], x[2], x[3]);  // -> X[4 k1 + k2] at 4 k2 + k1
-    dft4<INV>(x[4], x[5], x[6], x[7]);
-    dft4<INV>(x[8], x[9], x[10], x[11]);
-    dft4<INV>(x[12], x[13], x[14], x[15]);
-    float2 t;
-    t = x[1], x[1] = x[4], x[4] = t;
-    t = x[2], x[2] = x[8], x[8] = t;
-    t = x[3], x[3] = x[12], x[12] = t;
-    t = x[6], x[6] = x[9], x[9] = t;
-    t = x[7], x[7] = x[13], x[13] = t;
-    t = x[11], x[11] = x[14], x[14] = t;
-}
-
-// Shared-memory accesses through 32-bit shared-window addresses, and global
-// stores and reductions through explicitly global instructions: generic
-// accesses through pointers the compiler cannot place would keep the
-// transforms' register arrays in local memory.
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ float2 lds2(uint32_t a)
-{
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-    return v;
-}
-
-__device__ __forceinline__ void sts2(uint32_t a, float2 v)
-{
-    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
-}
 
 __device__ __forceinline__ void red_max_global(unsigned *p, unsigned v)
 {
@@ -418,12 +266,182 @@ __global__ void __launch_bounds__(32 * kEnvWarps, 2)
     }
 }
 
+// ------------------------------------------------- other depths (Fft16) ----
+
+// Magnitude where the sum of squares leaves the range it can be formed in.
+__device__ __noinline__ float hypot_far(float a, float b) { return hypotf(a, b); }
+
+__device__ __forceinline__ float magnitude(float q, float a, float b)
+{
+    return (q > 1e-36f && q < 3e38f) ? sqrt_fast(q) : hypot_far(a, b);
+}
+
+// Envelopes of the column pairs pair0, pair0 + 1, ... of one image, one pair per
+// T threads (C = THREADS / T pairs per CTA), as one complex column a + i b.
+// Depths that are a power of two are transformed as they are (M = nz); any other
+// depth nz convolves the column with the mask's impulse response of period nz,
+// unrolled to 2 nz - 1 lags, in a transform of length M >= 2 nz - 1.  Either
+// way the spectrum is multiplied by real tables (gr: the band-passed column, a
+// real even response; gh: i gh its Hilbert transform, a real odd one), with the
+// inverse's 1 / M in them: one forward transform and one inverse, or two for the
+// band-passed image, serve two columns.  (Bluestein's four transforms per single
+// column, which this replaced: 39.4 us of a 64 x 1750 image's pass, 732 us of the
+// pass of 32 uneven images of 64-1024 rows; measured now by the whole passes,
+// 47.7 -> 30.7 us and 3345 -> 2712 us.)  Bound: latency of the exchanges at small
+// image counts, shared-memory traffic and FP32 issue about equally at large ones.
+template <int LG, bool CONV, int THREADS>
+__device__ __forceinline__ float envelope_pairs(const EnvJob &J, int pair0, uint32_t bufs,
+                                                uint32_t hold)
+{
+    using F = Fft16<LG>;
+    constexpr int T = F::T;
+    const int grp = threadIdx.x / T;
+    const F f{bufs + (uint32_t)(grp * fft16_buf_bytes(LG)), J.ptw, (int)threadIdx.x % T, 1 + grp};
+    const uint32_t slot = hold + 8u * threadIdx.x;  // value r at slot + 8 THREADS r
+    const int nz = CONV ? J.nz : F::M;
+    const int ca = 2 * (pair0 + grp), cb = ca + 1;
+    const bool has_a = ca < J.nx, has_b = cb < J.nx;
+    const float *__restrict__ ya = J.y + (size_t)ca * nz;
+    const float *__restrict__ yb = ya + nz;
+    float2 v[16];
+    constexpr int JN = CONV ? 8 : 16;  // M >= 2 nz - 1: nothing from M / 2 on
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        v[j] = make_float2(0.f, 0.f);
+        if (j < JN) {
+            const int n = f.u + j * T;
+            const bool in = !CONV || n < nz;
+            if (in && has_a)
+                v[j].x = __ldcs(ya + n);
+            if (in && has_b)
+                v[j].y = __ldcs(yb + n);
+        }
+    }
+    const bool band = J.band != 0;
+    if (!band) {
+#pragma unroll
+        for (int j = 0; j < JN; ++j)
+            sts2(slot + 8u * THREADS * j, v[j]);  // the columns themselves
+    }
+    f.template forward<CONV>(v);
+    const float *__restrict__ gr = J.gr + f.u, *__restrict__ gh = J.gh + f.u;
+#pragma unroll 1
+    for (int it = band ? 0 : 1; it < 2; ++it) {
+        if (it == 0) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float r = __ldg(gr + q * T), h = __ldg(gh + q * T);
+                sts2(slot + 8u * THREADS * q, make_float2(-v[q].y * h, v[q].x * h));
+                v[q] = make_float2(v[q].x * r, v[q].y * r);
+            }
+        } else if (!band) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float h = __ldg(gh + q * T);
+                v[q] = make_float2(-v[q].y * h, v[q].x * h);
+            }
+        }
+        f.inverse(v);
+        if (it == 0) {  // the band-passed columns kept, their Hilbert spectrum next
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float2 t = lds2(slot + 8u * THREADS * q);
+                sts2(slot + 8u * THREADS * q, v[q]);
+                v[q] = t;
+            }
+        }
+    }
+    float lmax = 0.f;
+    float *__restrict__ oa = J.env + (size_t)ca * nz;
+    float *__restrict__ ob = oa + nz;
+#pragma unroll
+    for (int j = 0; j < JN; ++j) {
+        const int n = f.u + j * T;
+        const float2 r = lds2(slot + 8u * THREADS * j);
+        const float2 q = c_sqsum(r, v[j]);
+        if (CONV && n >= nz)
+            continue;
+        if (has_a) {
+            const float e = magnitude(q.x, r.x, v[j].x);
+            __stcg(oa + n, e);
+            lmax = fmaxf(lmax, e);
+        }
+        if (has_b) {
+            const float e = magnitude(q.y, r.y, v[j].y);
+            __stcg(ob + n, e);
+            lmax = fmaxf(lmax, e);
+        }
+    }
+    return lmax;
+}
+
+constexpr int kEnvThreads = 256;  // transforms of up to 16 * 256 points
+constexpr int kEnvBigThreads = 512;
+
+// One CTA: the column pairs of one image that THREADS threads hold at a time.
+// Images of different depths share a launch; BIG: the 8192-point transforms.
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? kEnvBigThreads : kEnvThreads, BIG ? 1 : 2)
+    envelope_kernel(const EnvJob *__restrict__ jobs, const int *__restrict__ blk_prefix, int njobs)
+{
+    constexpr int THREADS = BIG ? kEnvBigThreads : kEnvThreads;
+    extern __shared__ __align__(16) float2 esm[];
+    __shared__ float red[32];
+    // blocks in reverse: the beamformer writes a batch's last images last, so
+    // those are still in L2 when this kernel starts (and the log stage, in
+    // launch order, then reads the envelopes written last first)
+    const int blk = gridDim.x - 1 - blockIdx.x;
+    // the log stage's blocks may be scheduled as this grid's CTAs finish (they
+    // wait for the whole grid before reading its results)
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int jb = find_pair_job(blk_prefix, njobs, blk);
+    const EnvJob &J = jobs[jb];
+    const int first = blk - __ldg(blk_prefix + jb);
+    const uint32_t bufs = smem_addr(esm);
+    const uint32_t hold = bufs + (uint32_t)(THREADS * 17 * 8);
+    float lmax = 0.f;
+    auto run = [&](auto lg, auto conv) {
+        constexpr int LG = decltype(lg)::value;
+        constexpr bool CONV = decltype(conv)::value != 0;
+        lmax = envelope_pairs<LG, CONV, THREADS>(J, first * envelope_pairs_per_block(LG), bufs, hold);
+    };
+    auto pick = [&](auto lg) {
+        if (J.conv)
+            run(lg, std::integral_constant<int, 1>());
+        else
+            run(lg, std::integral_constant<int, 0>());
+    };
+    if constexpr (BIG) {
+        run(std::integral_constant<int, 13>(), std::integral_constant<int, 1>());
+    } else {
+        switch (J.lg) {
+        case 5: pick(std::integral_constant<int, 5>()); break;
+        case 6: pick(std::integral_constant<int, 6>()); break;
+        case 7: pick(std::integral_constant<int, 7>()); break;
+        case 8: pick(std::integral_constant<int, 8>()); break;
+        case 9: run(std::integral_constant<int, 9>(), std::integral_constant<int, 1>()); break;
+        case 10: pick(std::integral_constant<int, 10>()); break;
+        case 11: pick(std::integral_constant<int, 11>()); break;
+        default: pick(std::integral_constant<int, 12>()); break;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off; off >>= 1)
+        lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = lmax;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const float m = threadIdx.x < THREADS / 32 ? red[threadIdx.x] : 0.f;
+        const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));  // env >= 0
+        if (threadIdx.x == 0)
+            red_max_global(J.maxbits, w);
+    }
+}
+
 }  // namespace
 
-bool envelope_warp_ok(int nz, int fft_m, int bluestein)
-{
-    return !bluestein && fft_m == nz && nz == kN;
-}
+bool envelope_warp_ok(int nz) { return nz == kN; }
 
 static size_t envelope_warp_smem_bytes()
 {
@@ -446,6 +464,30 @@ cudaError_t launch_envelope_warp(const EnvJob *jobs_dev, const int *pair_prefix_
     envelope_warp_kernel<<<want < cap ? want : cap, 32 * kEnvWarps, smem, stream>>>(
         jobs_dev, pair_prefix_dev, njobs, total_pairs);
     return cudaGetLastError();
+}
+
+template <bool BIG>
+static cudaError_t launch_envelope_t(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,
+                                     int total_blocks, cudaStream_t stream)
+{
+    constexpr int threads = BIG ? kEnvBigThreads : kEnvThreads;
+    const size_t smem = (size_t)threads * (17 + 16) * sizeof(float2);
+    const void *k = (const void *)envelope_kernel<BIG>;
+    int sms = 0;
+    cudaError_t e = kernel_setup(k, smem, threads, true, &sms, nullptr);
+    if (e != cudaSuccess)
+        return e;
+    envelope_kernel<BIG><<<total_blocks, threads, smem, stream>>>(jobs_dev, blk_prefix_dev, njobs);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,
+                            int total_blocks, bool big, cudaStream_t stream)
+{
+    if (njobs <= 0 || total_blocks <= 0)
+        return cudaSuccess;
+    return big ? launch_envelope_t<true>(jobs_dev, blk_prefix_dev, njobs, total_blocks, stream)
+               : launch_envelope_t<false>(jobs_dev, blk_prefix_dev, njobs, total_blocks, stream);
 }
 
 }  // namespace bfi

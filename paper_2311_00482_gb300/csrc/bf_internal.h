@@ -50,6 +50,25 @@ constexpr int kMaxFramesPerJob = 4;
 // BF16, or complex analytic-signal pairs for IQ beamforming (kPrecIQ, FP32).
 enum Prec : int { kPrecF32 = 0, kPrecF16 = 1, kPrecBF16 = 2, kPrecIQ = 3 };
 
+// Layout of the Fft16 transforms (bf_fft16.cuh), shared with the host tables.
+// Twiddles of a level of length 2^L, S = 2^(L-4): exponents 1, 2, 3, 4, 8, 12 of
+// W_(2^L)^t, each a run of S entries, levels L = 5, 6, ... back to back (one
+// table serves every transform length; the other powers are single products).
+constexpr int kFft16MaxLg = 13;
+__host__ __device__ constexpr int fft16_tw_at(int L) { return 6 * ((1 << (L - 4)) - 2); }
+// Bin held by register q of thread u after the forward transform.
+__host__ __device__ inline int fft16_bin(int lg, int u, int q)
+{
+    int p = 16 * u + q, k = 0, mult = 1;
+    for (; lg > 4; lg -= 4, mult <<= 4) {
+        k += (p >> (lg - 4)) * mult;
+        p &= (1 << (lg - 4)) - 1;
+    }
+    return k + p * mult;
+}
+// Bytes of the exchange buffer of one transform.
+__host__ __device__ constexpr int fft16_buf_bytes(int lg) { return (1 << lg) / 16 * 17 * 8; }
+
 // Device-side error bits (written with atomicOr into a per-launch word).
 enum DevErr : int { kErrTimeout = 1, kErrWindow = 2, kErrConfig = 4 };
 
@@ -171,15 +190,17 @@ struct EnvJob {
     float *env;           // [nx][nz] envelope output
     unsigned *maxbits;    // frame maximum of env (float bits), reset to 0 before
     int nx, nz;
-    int fft_m;            // transform size (nz itself when nz is a power of two)
-    int bluestein;        // 1 when nz is not a power of two
+    int lg;               // transforms of 2^lg points (lg = 0: the warp kernel's 512-row images)
+    int conv;             // 1: nz is not a power of two (or below 32): convolved in 2^lg >= 2 nz - 1
     int band;             // 1: keep only bins [kb_lo, kb_hi] (DMAS second-harmonic band-pass)
     int kb_lo, kb_hi;
-    int cols_per_block;   // image columns transformed together by one CTA
-    int vec4;             // 1: y and env are 16-byte aligned and nz a multiple of 4 (vector access)
-    const float2 *tw;     // [fft_m] exp(-2 pi i k / fft_m)
-    const float2 *chirp;  // [nz] exp(i pi n^2 / nz)              (Bluestein only)
-    const float2 *bhat;   // [fft_m] DFT of the chirp convolution kernel (Bluestein only)
+    const float2 *tw;     // warp kernel: [512] exp(-2 pi i k / 512)
+    const float2 *ptw;    // level twiddles of the Fft16 transforms (bf_fft16.cuh)
+    // spectral factors in the transform's register order [q][u] (bin
+    // fft16_bin(lg, u, q)), 1 / 2^lg included: i gh takes the spectrum to the
+    // (band-passed) column's Hilbert transform, gr (band only) to the
+    // band-passed column itself
+    const float *gr, *gh;
 };
 
 // One (frame, mode) envelope image to decibels against its frame maximum.
@@ -220,14 +241,17 @@ cudaError_t launch_fkmig(const FkJob &job, cudaStream_t stream);
 cudaError_t launch_beamform(const BfJob *jobs_dev, const int *tile_prefix_dev, int njobs,
                             int total_tiles, size_t smem_bytes, int prec, int variant, int rows,
                             int nf, int *err_dev, cudaStream_t stream);
+// Envelopes of the other depths (bf_envelope.cu); big: the jobs of lg = 13.
 cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,
-                            int total_blocks, size_t smem_bytes, cudaStream_t stream);
+                            int total_blocks, bool big, cudaStream_t stream);
+// Column pairs one CTA of launch_envelope takes.
+__host__ __device__ constexpr int envelope_pairs_per_block(int lg) { return lg >= 12 ? 1 : 4096 >> lg; }
 cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int njobs,
                        int total_blocks, float dynamic_range_db, cudaStream_t stream);
 // Envelope of 512-row images by the warp-per-column-pair kernel (bf_envelope.cu):
-// the jobs it takes (power-of-two depth of 512, no Bluestein), and its launch
+// the depths it takes, and its launch
 // over total_pairs column pairs (pair_prefix_dev: each job's first pair).
-bool envelope_warp_ok(int nz, int fft_m, int bluestein);
+bool envelope_warp_ok(int nz);
 cudaError_t launch_envelope_warp(const EnvJob *jobs_dev, const int *pair_prefix_dev, int njobs,
                                  int total_pairs, cudaStream_t stream);
 // One frame through the plain baseline kernel (FP32, global loads, one thread
@@ -238,8 +262,6 @@ cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const int2 *valid,
 // staging area (nf > 1) and the pipeline stages.
 size_t beamform_smem_bytes(int wmax, int group, int prec, int nf = 1, int rows = 4);
 int log_blocks(long long pixels);
-int envelope_cols_per_block(int fft_m);
-size_t envelope_smem_bytes(int fft_m, int bluestein);
 
 // Bytes of one stored sample pair for a precision.
 inline int pair_bytes(int prec) { return prec == kPrecIQ ? 16 : prec == kPrecF32 ? 8 : 4; }

@@ -21,10 +21,6 @@
 //                    every delay (and for IQ-DAS / BB-DMAS, Eq. (4), the
 //                    carrier phase) serves all of them, and a storer warp
 //                    writes the staged tile images with bulk copies
-//   envelope_kernel  per image column the analytic signal along depth via a
-//                    shared-memory radix-8 Stockham FFT (Bluestein for other
-//                    lengths), one-sided mask and optional [f0, 3 f0]
-//                    band-pass, magnitude, and the frame maximum
 //   log_kernel       20 log10(env / max) clipped to the -70 dB range of Fig. 3
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -1692,254 +1688,6 @@ __global__ void __launch_bounds__(256) plain_kernel(const BfJob J, const int16_t
         J.y[(size_t)(slot++) * plane + o] = Yp;
 }
 
-// ------------------------------------------------------------- envelope --
-
-__device__ __forceinline__ float spectral_weight(int k, int L, int band, int kb_lo, int kb_hi)
-{
-    float h = (k == 0) ? 1.f : (2 * k < L) ? 2.f : (2 * k == L) ? 1.f : 0.f;
-    if (band && (k < kb_lo || k > kb_hi))
-        h = 0.f;
-    return h;
-}
-
-// Envelope transform buffers: plain, or in the swz layout.  Measured on the
-// 512 x 512 workload: the swizzle removes the strided passes' bank conflicts
-// (shared wavefronts 7.9 M -> 3.2 M per 8 frames) but its index arithmetic
-// adds half again the instructions, and the kernel ends no faster; the
-// per-pass twiddle table alone takes the envelope + log stages from 0.285 to
-// 0.260 ms per 64 frames.
-constexpr bool kEnvSwizzle = false;
-
-// Analytic-signal envelope of an image's columns.  The one-sided spectrum
-// X * H (H = 1 at 0 and L/2, 2 between, 0 for negative frequencies), times
-// the band-pass B for the DMAS image, has as inverse transform r + i h: r is
-// the column filtered by B mirrored onto negative frequencies (the column
-// itself without band-pass) and h its Hilbert transform, the multiplier
-// -i sgn(k) B(|k|) with sgn(0) = sgn(L/2) = 0.  Both are real and linear in
-// the column, so two columns a, b go through one complex transform of
-// a + i b: the inverse transforms of M(k) (A + iB) give r_a + i r_b and
-// h_a + i h_b.
-__global__ void __launch_bounds__(256) envelope_kernel(const EnvJob *__restrict__ jobs,
-                                                       const int *__restrict__ blk_prefix,
-                                                       int njobs)
-{
-    extern __shared__ __align__(16) float2 sbuf[];
-    __shared__ float red[32];
-    // blocks in reverse: the beamformer writes a batch's last images last, so
-    // those are still in L2 when this kernel starts (and the log stage, in
-    // launch order, then reads the envelopes written last first)
-    const int blk = gridDim.x - 1 - blockIdx.x;
-    // the log stage's blocks may be scheduled as this grid's CTAs finish (they
-    // wait for the whole grid before reading its results)
-    asm volatile("griddepcontrol.launch_dependents;");
-    const int jb = find_job(blk_prefix, njobs, blk);
-    const EnvJob J = jobs[jb];
-    const int nz = J.nz, m = J.fft_m;
-    const int lgm = 31 - __clz(m);
-    float lmax = 0.f;
-
-    if (!J.bluestein) {
-        const int C = J.cols_per_block >> 1;  // complex columns (pairs of image columns)
-        const int c0 = (blk - __ldg(blk_prefix + jb)) * J.cols_per_block;
-        float2 *Zb = sbuf, *Pb = sbuf + (size_t)C * m, *Qb = sbuf + (size_t)2 * C * m;
-        float2 *tw = sbuf + (size_t)3 * C * m;
-        float2 *ptw = tw + m;  // per-pass twiddles of the radix-8 passes
-        for (int k = threadIdx.x; k < m; k += blockDim.x)
-            tw[k] = __ldg(J.tw + k);
-        __syncthreads();
-        fill_pass_twiddles(ptw, tw, lgm);
-        // Buffers in the swizzled layout (element t at swz(t)): columns in, four
-        // depths per thread with 16-byte global loads (m >= 4: nz = m)
-        auto at = [](int t) { return swz<kEnvSwizzle>(t); };
-        const int vec = J.vec4 ? 4 : 1;
-        for (int t = threadIdx.x * vec; t < C * m; t += blockDim.x * vec) {
-            const int c = t >> lgm, n = t & (m - 1);
-            const int ca = c0 + 2 * c, cb = ca + 1;
-            if (vec == 4) {
-                const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 a = ca < J.nx ? __ldg(reinterpret_cast<const float4 *>(J.y + (size_t)ca * nz + n)) : z4;
-                const float4 b = cb < J.nx ? __ldg(reinterpret_cast<const float4 *>(J.y + (size_t)cb * nz + n)) : z4;
-                Zb[at(t)] = make_float2(a.x, b.x);
-                Zb[at(t + 1)] = make_float2(a.y, b.y);
-                Zb[at(t + 2)] = make_float2(a.z, b.z);
-                Zb[at(t + 3)] = make_float2(a.w, b.w);
-            } else {
-                const float ya = ca < J.nx ? __ldg(J.y + (size_t)ca * nz + n) : 0.f;
-                const float yb = cb < J.nx ? __ldg(J.y + (size_t)cb * nz + n) : 0.f;
-                Zb[at(t)] = make_float2(ya, yb);
-            }
-        }
-        __syncthreads();
-        float2 *S = fft_r8<kEnvSwizzle>(Zb, Pb, m, lgm, C, tw, false, ptw);  // spectrum of a + i b
-        float2 *F1 = S == Zb ? Pb : Zb;                                 // free buffer
-        const float inv = 1.f / (float)m;
-        if (!J.band) {
-            for (int t = threadIdx.x; t < C * m; t += blockDim.x) {
-                const int k = t & (m - 1);
-                const float sg = (k == 0 || 2 * k == m) ? 0.f : (2 * k < m ? 1.f : -1.f);
-                const float2 sv = S[at(t)];
-                F1[at(t)] = make_float2(sv.y * sg, -sv.x * sg);  // -i sgn(k) S
-            }
-            __syncthreads();
-            const float2 *Hh = fft_r8<kEnvSwizzle>(F1, S, m, lgm, C, tw, true, ptw);
-            for (int t = threadIdx.x * vec; t < C * m; t += blockDim.x * vec) {
-                const int c = t >> lgm, n = t & (m - 1);
-                const int ca = c0 + 2 * c, cb = ca + 1;
-                if (vec == 4) {
-                    const float2 h0 = Hh[at(t)], h1 = Hh[at(t + 1)], h2 = Hh[at(t + 2)],
-                                 h3 = Hh[at(t + 3)];
-                    if (ca < J.nx) {
-                        const float4 a = __ldg(reinterpret_cast<const float4 *>(J.y + (size_t)ca * nz + n));
-                        const float4 e = make_float4(hypotf(a.x, h0.x * inv), hypotf(a.y, h1.x * inv),
-                                                     hypotf(a.z, h2.x * inv), hypotf(a.w, h3.x * inv));
-                        *reinterpret_cast<float4 *>(J.env + (size_t)ca * nz + n) = e;
-                        lmax = fmaxf(lmax, fmaxf(fmaxf(e.x, e.y), fmaxf(e.z, e.w)));
-                    }
-                    if (cb < J.nx) {
-                        const float4 b = __ldg(reinterpret_cast<const float4 *>(J.y + (size_t)cb * nz + n));
-                        const float4 e = make_float4(hypotf(b.x, h0.y * inv), hypotf(b.y, h1.y * inv),
-                                                     hypotf(b.z, h2.y * inv), hypotf(b.w, h3.y * inv));
-                        *reinterpret_cast<float4 *>(J.env + (size_t)cb * nz + n) = e;
-                        lmax = fmaxf(lmax, fmaxf(fmaxf(e.x, e.y), fmaxf(e.z, e.w)));
-                    }
-                    continue;
-                }
-                const float2 h = Hh[at(t)];
-                if (ca < J.nx) {
-                    const float e = hypotf(__ldg(J.y + (size_t)ca * nz + n), h.x * inv);
-                    J.env[(size_t)ca * nz + n] = e;
-                    lmax = fmaxf(lmax, e);
-                }
-                if (cb < J.nx) {
-                    const float e = hypotf(__ldg(J.y + (size_t)cb * nz + n), h.y * inv);
-                    J.env[(size_t)cb * nz + n] = e;
-                    lmax = fmaxf(lmax, e);
-                }
-            }
-        } else {
-            for (int t = threadIdx.x; t < C * m; t += blockDim.x) {
-                const int k = t & (m - 1);
-                const int kk = 2 * k <= m ? k : m - k;  // |k|
-                const float bp = (kk >= J.kb_lo && kk <= J.kb_hi) ? 1.f : 0.f;
-                const float sg = (k == 0 || 2 * k == m) ? 0.f : (2 * k < m ? 1.f : -1.f);
-                const float2 sv = S[at(t)];
-                const float2 r = make_float2(sv.x * bp, sv.y * bp);
-                S[at(t)] = r;
-                Qb[at(t)] = make_float2(r.y * sg, -r.x * sg);
-            }
-            __syncthreads();
-            float2 *R = fft_r8<kEnvSwizzle>(S, F1, m, lgm, C, tw, true, ptw);
-            float2 *F2 = R == S ? F1 : S;
-            const float2 *Hh = fft_r8<kEnvSwizzle>(Qb, F2, m, lgm, C, tw, true, ptw);
-            for (int t = threadIdx.x * vec; t < C * m; t += blockDim.x * vec) {
-                const int c = t >> lgm, n = t & (m - 1);
-                const int ca = c0 + 2 * c, cb = ca + 1;
-                if (vec == 4) {
-                    float2 rr[4], hh[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        rr[u] = R[at(t + u)];
-                        hh[u] = Hh[at(t + u)];
-                    }
-                    if (ca < J.nx) {
-                        const float4 e = make_float4(hypotf(rr[0].x, hh[0].x) * inv, hypotf(rr[1].x, hh[1].x) * inv,
-                                                     hypotf(rr[2].x, hh[2].x) * inv, hypotf(rr[3].x, hh[3].x) * inv);
-                        *reinterpret_cast<float4 *>(J.env + (size_t)ca * nz + n) = e;
-                        lmax = fmaxf(lmax, fmaxf(fmaxf(e.x, e.y), fmaxf(e.z, e.w)));
-                    }
-                    if (cb < J.nx) {
-                        const float4 e = make_float4(hypotf(rr[0].y, hh[0].y) * inv, hypotf(rr[1].y, hh[1].y) * inv,
-                                                     hypotf(rr[2].y, hh[2].y) * inv, hypotf(rr[3].y, hh[3].y) * inv);
-                        *reinterpret_cast<float4 *>(J.env + (size_t)cb * nz + n) = e;
-                        lmax = fmaxf(lmax, fmaxf(fmaxf(e.x, e.y), fmaxf(e.z, e.w)));
-                    }
-                    continue;
-                }
-                const float2 rv = R[at(t)], hv = Hh[at(t)];
-                if (ca < J.nx) {
-                    const float e = hypotf(rv.x, hv.x) * inv;
-                    J.env[(size_t)ca * nz + n] = e;
-                    lmax = fmaxf(lmax, e);
-                }
-                if (cb < J.nx) {
-                    const float e = hypotf(rv.y, hv.y) * inv;
-                    J.env[(size_t)cb * nz + n] = e;
-                    lmax = fmaxf(lmax, e);
-                }
-            }
-        }
-    } else {
-        // one column per block through Bluestein's chirp transforms
-        const int c0 = blk - __ldg(blk_prefix + jb);
-        float2 *A = sbuf, *B = sbuf + m, *tw = sbuf + (size_t)3 * m;
-        for (int k = threadIdx.x; k < m; k += blockDim.x)
-            tw[k] = __ldg(J.tw + k);
-        const float *__restrict__ y = J.y + (size_t)c0 * nz;
-        const float2 *__restrict__ w = J.chirp;
-        const float2 *__restrict__ bh = J.bhat;
-        const float inv_m = 1.f / (float)m;
-        // forward DFT: X_k = conj(w_k) * (a (*) w)_k with a_n = y_n conj(w_n)
-        for (int n = threadIdx.x; n < m; n += blockDim.x) {
-            float2 v = make_float2(0.f, 0.f);
-            if (n < nz) {
-                const float2 c = __ldg(w + n);
-                const float yn = __ldg(y + n);
-                v = make_float2(yn * c.x, -yn * c.y);
-            }
-            A[n] = v;
-        }
-        __syncthreads();
-        float2 *X = fft_r8(A, B, m, lgm, 1, tw, false);
-        for (int k = threadIdx.x; k < m; k += blockDim.x)
-            X[k] = cmul(X[k], __ldg(bh + k));
-        __syncthreads();
-        float2 *O = X == A ? B : A;
-        float2 *Cb = fft_r8(X, O, m, lgm, 1, tw, true);
-        float2 *D = Cb == A ? B : A;
-        // masked spectrum, conjugated and pre-multiplied by conj(w) for the second
-        // pass: the inverse DFT of S is conj(DFT(conj S)) / nz
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            float2 v = make_float2(0.f, 0.f);
-            if (k < nz) {
-                const float2 c = __ldg(w + k);
-                const float2 cc = make_float2(c.x, -c.y);
-                float2 xk = cmul(make_float2(Cb[k].x * inv_m, Cb[k].y * inv_m), cc);
-                const float h = spectral_weight(k, nz, J.band, J.kb_lo, J.kb_hi);
-                xk = make_float2(xk.x * h, -xk.y * h);
-                v = cmul(xk, cc);
-            }
-            D[k] = v;
-        }
-        __syncthreads();
-        float2 *E = fft_r8(D, Cb, m, lgm, 1, tw, false);
-        for (int k = threadIdx.x; k < m; k += blockDim.x)
-            E[k] = cmul(E[k], __ldg(bh + k));
-        __syncthreads();
-        float2 *F = fft_r8(E, E == A ? B : A, m, lgm, 1, tw, true);
-        const float inv = inv_m / (float)nz;
-        float *__restrict__ env = J.env + (size_t)c0 * nz;
-        for (int n = threadIdx.x; n < nz; n += blockDim.x) {
-            const float e = hypotf(F[n].x, F[n].y) * inv;
-            env[n] = e;
-            lmax = fmaxf(lmax, e);
-        }
-    }
-#pragma unroll
-    for (int off = 16; off; off >>= 1)
-        lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
-    if ((threadIdx.x & 31) == 0)
-        red[threadIdx.x >> 5] = lmax;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-#pragma unroll
-        for (int off = 16; off; off >>= 1)
-            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-        if (threadIdx.x == 0)
-            atomicMax(J.maxbits, __float_as_uint(v));  // env >= 0: bit order = value order
-    }
-}
-
 // ------------------------------------------------------------ f-k migration --
 
 // Per channel record: transform along time (zero-padded to nt), then the
@@ -2185,21 +1933,6 @@ size_t beamform_smem_bytes(int wmax, int group, int prec, int nf, int rows)
            (size_t)stages_for_rows(rows) * stage_bytes(group, wmax, pair_bytes(prec), nf);
 }
 
-// Image columns per envelope CTA for a power-of-two transform: two per
-// complex column, up to 2048 complex points per buffer.
-int envelope_cols_per_block(int fft_m) { return 2 * (fft_m >= 2048 ? 1 : 2048 / fft_m); }
-
-// Shared memory of an envelope CTA: three transform buffers and the twiddles.
-size_t envelope_smem_bytes(int fft_m, int bluestein)
-{
-    const int c = bluestein ? 1 : envelope_cols_per_block(fft_m) / 2;
-    int lgm = 0;
-    while ((1 << lgm) < fft_m)
-        ++lgm;
-    const size_t passes = bluestein ? 0 : (size_t)pass_twiddle_count(lgm);
-    return (3u * (size_t)c * fft_m + (size_t)fft_m + passes) * sizeof(float2);
-}
-
 cudaError_t launch_plan(const PlanJob &job, int *err_dev, cudaStream_t stream)
 {
     dim3 grid(job.tiles_x * job.tiles_z, job.na);
@@ -2308,19 +2041,6 @@ cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const int2 *valid,
         plain_kernel<false, true><<<blocks, 256, 0, stream>>>(job, rf, valid, dx2, nxp, ns);
     else
         plain_kernel<false, false><<<blocks, 256, 0, stream>>>(job, rf, valid, dx2, nxp, ns);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,
-                            int total_blocks, size_t smem, cudaStream_t stream)
-{
-    if (njobs <= 0 || total_blocks <= 0)
-        return cudaSuccess;
-    int sms = 0;
-    cudaError_t e = kernel_setup((const void *)envelope_kernel, smem, 256, false, &sms, nullptr);
-    if (e != cudaSuccess)
-        return e;
-    envelope_kernel<<<total_blocks, 256, smem, stream>>>(jobs_dev, blk_prefix_dev, njobs);
     return cudaGetLastError();
 }
 

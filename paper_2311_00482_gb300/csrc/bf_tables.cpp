@@ -16,6 +16,8 @@
 
 namespace bfi {
 
+static constexpr double kPi = 3.14159265358979323846;
+
 double grid_coord(double lo, double hi, int n, int j)
 {
     if (n == 1)
@@ -271,6 +273,33 @@ void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
     }
 }
 
+void fft_twiddles(int n, std::vector<float> &tw)
+{
+    tw.resize((size_t)n * 2);
+    for (int k = 0; k < n; ++k) {
+        const double ang = -2.0 * kPi * (double)k / (double)n;
+        tw[2 * k] = (float)std::cos(ang);
+        tw[2 * k + 1] = (float)std::sin(ang);
+    }
+}
+
+void fft16_twiddles(std::vector<float> &tw)
+{
+    const int e[6] = {1, 2, 3, 4, 8, 12};
+    tw.resize((size_t)fft16_tw_at(kFft16MaxLg + 1) * 2);
+    for (int L = 5; L <= kFft16MaxLg; ++L) {
+        const int S = 1 << (L - 4);
+        for (int i = 0; i < 6; ++i)
+            for (int t = 0; t < S; ++t) {
+                const double ang = -2.0 * kPi * (double)(t * e[i]) / (double)(1 << L);
+                float *w = &tw[2 * ((size_t)fft16_tw_at(L) + i * S + t)];
+                w[0] = (float)std::cos(ang);
+                w[1] = (float)std::sin(ang);
+            }
+    }
+}
+
+// In-place radix-2 transform in double precision.
 static void fft_inplace(std::vector<std::complex<double>> &a)
 {
     const size_t n = a.size();
@@ -282,64 +311,86 @@ static void fft_inplace(std::vector<std::complex<double>> &a)
         if (i < j)
             std::swap(a[i], a[j]);
     }
-    const double pi = 3.14159265358979323846;
-    for (size_t len = 2; len <= n; len <<= 1) {
+    std::vector<std::complex<double>> w(n / 2);
+    for (size_t k = 0; k < n / 2; ++k) {
+        const double ang = -2.0 * kPi * (double)k / (double)n;
+        w[k] = std::complex<double>(std::cos(ang), std::sin(ang));
+    }
+    for (size_t len = 2; len <= n; len <<= 1)
         for (size_t i = 0; i < n; i += len)
             for (size_t j = 0; j < len / 2; ++j) {
-                double ang = -2.0 * pi * (double)j / (double)len;
-                std::complex<double> w(std::cos(ang), std::sin(ang));
-                std::complex<double> u = a[i + j], v = a[i + j + len / 2] * w;
+                const std::complex<double> x = a[i + j + len / 2], t = w[j * (n / len)];
+                const std::complex<double> u = a[i + j],
+                                           v(x.real() * t.real() - x.imag() * t.imag(),
+                                             x.real() * t.imag() + x.imag() * t.real());
                 a[i + j] = u + v;
                 a[i + j + len / 2] = u - v;
             }
-    }
 }
 
-void envelope_tables(int nz, EnvHost &out)
+// The one-sided mask of a depth nz as real operators on the column: r keeps the
+// bins |k| in the band (all of them without one), h their Hilbert transform
+// (multiplier -i sgn(k), sgn(0) = sgn(nz / 2) = 0); the envelope is |r + i h|.
+void envelope_tables(int nz, bool band, int lo, int hi, EnvHost &out)
 {
-    const double pi = 3.14159265358979323846;
-    out.nz = nz;
-    const bool pow2 = (nz & (nz - 1)) == 0;
-    int m = 1;
-    if (pow2)
-        m = nz;
-    else
-        while (m < 2 * nz - 1)
-            m <<= 1;
-    out.fft_m = m;
-    out.bluestein = pow2 ? 0 : 1;
-    out.tw.resize((size_t)m * 2);
-    for (int k = 0; k < m; ++k) {
-        double ang = -2.0 * pi * (double)k / (double)m;
-        out.tw[2 * k] = (float)std::cos(ang);
-        out.tw[2 * k + 1] = (float)std::sin(ang);
-    }
-    out.chirp.clear();
-    out.bhat.clear();
-    if (!pow2) {
-        std::vector<std::complex<double>> w(nz), b(m, 0.0);
-        for (int n = 0; n < nz; ++n) {
-            long long r = ((long long)n * n) % (2LL * nz);
-            double ang = pi * (double)r / (double)nz;
-            w[n] = std::complex<double>(std::cos(ang), std::sin(ang));
-        }
-        for (int n = 0; n < nz; ++n) {
-            b[n] = w[n];
-            if (n > 0)
-                b[m - n] = w[n];
-        }
-        fft_inplace(b);
-        out.chirp.resize(2 * nz);
-        out.bhat.resize(2 * m);
-        for (int n = 0; n < nz; ++n) {
-            out.chirp[2 * n] = (float)w[n].real();
-            out.chirp[2 * n + 1] = (float)w[n].imag();
-        }
+    const bool direct = nz >= 32 && (nz & (nz - 1)) == 0;
+    out.conv = direct ? 0 : 1;
+    out.lg = 5;
+    while ((1 << out.lg) < (direct ? nz : 2 * nz - 1))
+        ++out.lg;
+    const int m = 1 << out.lg, T = m / 16;
+    std::vector<double> R(m), H(m);  // factors of the real and the i gh operator per bin
+    if (direct) {
         for (int k = 0; k < m; ++k) {
-            out.bhat[2 * k] = (float)b[k].real();
-            out.bhat[2 * k + 1] = (float)b[k].imag();
+            const int ka = 2 * k <= m ? k : m - k;
+            const bool in = !band || (ka >= lo && ka <= hi);
+            R[k] = in ? 1.0 : 0.0;
+            H[k] = (!in || k == 0 || 2 * k == m) ? 0.0 : (2 * k < m ? -1.0 : 1.0);
+        }
+    } else {
+        // impulse responses of period nz: sums of cos / sin(2 pi k n / nz) over the
+        // band's bins a .. b strictly between 0 and nz / 2 in closed form (angles
+        // reduced in integers), the bins 0 and nz / 2 by themselves
+        const int a = std::max(1, band ? lo : 1), b = std::min((nz - 1) / 2, band ? hi : nz);
+        const bool dc = !band, ny = nz % 2 == 0 && (!band || (lo <= nz / 2 && nz / 2 <= hi));
+        std::vector<std::complex<double>> c(m, 0.0);
+        for (int n = 0; n < nz; ++n) {
+            double sc = 0.0, ss = 0.0;
+            if (a <= b) {
+                if (n == 0) {
+                    sc = (double)(b - a + 1);
+                } else {
+                    auto ang = [&](long long q) {  // pi q n / nz
+                        return kPi * (double)(q * n % (2LL * nz)) / (double)nz;
+                    };
+                    const double hi2 = ang(2LL * b + 1), lo2 = ang(2LL * a - 1);
+                    const double s = 2.0 * std::sin(kPi * (double)n / (double)nz);
+                    sc = (std::sin(hi2) - std::sin(lo2)) / s;
+                    ss = (std::cos(lo2) - std::cos(hi2)) / s;
+                }
+            }
+            const double r = (2.0 * sc + (dc ? 1.0 : 0.0) + (ny ? (n % 2 ? -1.0 : 1.0) : 0.0)) / nz;
+            const double h = 2.0 * ss / nz;
+            c[n] = std::complex<double>(r, h);
+            if (n > 0)  // lag n - nz
+                c[m - nz + n] = std::complex<double>(r, h);
+        }
+        fft_inplace(c);  // r even, h odd: FFT(r) is real, FFT(h) imaginary
+        for (int k = 0; k < m; ++k) {
+            const double x = c[k].real(), y = c[(m - k) % m].real();
+            R[k] = 0.5 * (x + y);
+            H[k] = 0.5 * (y - x);
         }
     }
+    out.gh.resize(m);
+    out.gr.resize(band ? m : 0);
+    for (int u = 0; u < T; ++u)
+        for (int q = 0; q < 16; ++q) {
+            const int k = fft16_bin(out.lg, u, q);
+            out.gh[(size_t)q * T + u] = (float)(H[k] / m);
+            if (band)
+                out.gr[(size_t)q * T + u] = (float)(R[k] / m);
+        }
 }
 
 }  // namespace bfi

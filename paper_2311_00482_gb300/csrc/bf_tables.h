@@ -34,9 +34,11 @@ struct PlanHost {
     int wmax = 0, box = 0, group = 1, nsp = 0, rows = 8, align = 2;
 };
 
+// Envelope transform of a depth: length 2^lg and the spectral factors of
+// EnvJob (gr only with a band).
 struct EnvHost {
-    int nz = 0, fft_m = 0, bluestein = 0;
-    std::vector<float> tw, chirp, bhat;  // interleaved re / im
+    int lg = 0, conv = 0;
+    std::vector<float> gr, gh;
 };
 
 double grid_coord(double lo, double hi, int n, int j);
@@ -57,6 +59,11 @@ void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, i
 void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
                        const std::vector<double> &sc, bool stolt, std::vector<int> &i0,
                        std::vector<float> &aw);
-void envelope_tables(int nz, EnvHost &out);
+// exp(-2 pi i k / n) for k < n, interleaved.
+void fft_twiddles(int n, std::vector<float> &tw);
+// The level twiddles of every Fft16 transform (layout: bf_fft16.cuh), interleaved.
+void fft16_twiddles(std::vector<float> &tw);
+// band: keep the bins lo .. hi only.
+void envelope_tables(int nz, bool band, int lo, int hi, EnvHost &out);
 
 }  // namespace bfi
