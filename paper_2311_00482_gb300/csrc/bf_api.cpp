@@ -127,33 +127,34 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// 2-D tensor map over a row-major table of `rows` rows of `cols` elements of
-// `elem` bytes (4 or 8), read in boxes of box_cols x box_rows; out-of-range
-// elements read as zero.
+// Tensor map over a row-major table of `rows` rows of `cols` elements of `elem`
+// bytes (4 or 8), read in boxes of box_cols x box_rows; planes > 0: `planes` such
+// tables back to back, boxes box_planes deep.  Out-of-range elements read as zero.
 static int encode_map(CUtensorMap *map, void *base, int rows, int cols, int elem, int box_cols,
-                      int box_rows)
+                      int box_rows, int planes = 0, int box_planes = 1)
 {
     auto enc = tensor_map_encoder();
     if (!enc)
         return fail(BF_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * (cuuint64_t)elem};
-    cuuint32_t boxd[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    const cuuint64_t pitch = (cuuint64_t)cols * (cuuint64_t)elem;
+    cuuint64_t strides[2] = {pitch, pitch * (cuuint64_t)rows};
+    cuuint32_t boxd[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+    cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(map, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32,
-                     2, base, dims, strides, boxd, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                     planes > 0 ? 3 : 2, base, dims, strides, boxd, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(BF_ECUDA, "cuTensorMapEncodeTiled failed (%d): %d x %d of %d bytes, box %d x %d",
                     (int)r, rows, cols, elem, box_cols, box_rows);
     return BF_OK;
 }
 
-static int encode_pairs_map(CUtensorMap *map, void *base, int rows, int nsp, int box, int prec)
+static int encode_pairs_map(CUtensorMap *map, void *base, int rows, int nsp, int box, int run, int prec)
 {
     const int k = pair_elems(prec);  // IQ pairs: two 8-byte elements each
-    return encode_map(map, base, rows, nsp * k, pair_bytes(prec) / k, box * k, 1);
+    return encode_map(map, base, rows, nsp * k, pair_bytes(prec) / k, box * k, run);
 }
 
 // Pairs per frame of one tensor copy of an nf-frame job's interleaved window
@@ -244,34 +245,84 @@ static int env_tables(int nz, bool band, int lo, int hi, std::shared_ptr<EnvTabl
 
 // ------------------------------------------------------------------ plans --
 
-// Tile configuration of a workload: what bf_autotune measured fastest for it,
-// else entry 0 (4 rows per thread, 32-row tiles, three CTAs per SM, measured
-// faster than 8 rows on every grid tried); BF_TILE_ROWS=8 forces entry 3,
-// BF_TILE_ROWS=2 entry 6 (16-row tiles of up to 22 channels per stage; DAS /
-// DMAS of RF records, IQ-DAS / BB-DMAS; others keep entry 0).
-static int choose_cfg(const bf_handle *h, const PlanKey &key)
+// BF_TILE_ROWS=8 forces entry 3 of kTileConfigs, 4 entry 0, 2 entry 6 (16-row tiles
+// of up to 22 channels per stage); -1: not set.
+static int forced_cfg()
 {
-    if (const char *e = std::getenv("BF_TILE_ROWS")) {
-        if (std::atoi(e) == 8)
-            return 3;
-        if (std::atoi(e) == 4)
-            return 0;
-        if (std::atoi(e) == 2)
-            return 6;
-    }
+    const char *e = std::getenv("BF_TILE_ROWS");
+    const int rows = e ? std::atoi(e) : 0;
+    return rows == 8 ? 3 : rows == 4 ? 0 : rows == 2 ? 6 : -1;
+}
+
+static PlanKey tuned_key(PlanKey k)
+{
+    k.cfg = 0;
+    return k;
+}
+
+// Configuration of a workload (of kTileConfigs, or a solo one): BF_TILE_ROWS, else
+// what bf_autotune measured fastest for it, else by the frames that share it.
+// Beamforming time per 512 x 512 frame, 32 frames in a batch, DAS + DMAS of one
+// angle / DMAS of three: alone (solo) 13.7 / 22.3 us, in pairs on 32-row tiles 7.4 /
+// 21.0 us, in fours on 16-row tiles 5.9 / 16.2 us.
+static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w, bool narrow_ok)
+{
+    const int forced = forced_cfg();
+    if (forced >= 0)
+        return forced;
     auto it = h->tuned.find(key);
-    return it == h->tuned.end() ? 0 : it->second;
+    if (it != h->tuned.end())
+        return it->second;
+    // Alone: split the channels of a row pair over four warps below 3/4 of a 16-row
+    // tile per SM, over two below 3/2 (152 SMs; splits 1 / 2 / 4, DMAS of three angles:
+    // 32 tiles 26.2 / 16.0 / 11.9 us, 112 tiles 20.4 / 16.0 / 13.9, 128 tiles 20.1 /
+    // 16.0 / 20.1, 220 tiles 28.3 / 24.2 / 32.4, 325 tiles 26.2 / 26.6 / 36.5, 512
+    // tiles 32.4 / 34.4 / 54.9).  The frame's own tiles decide, also in a batch: a
+    // frame's sums do not depend on what it is launched with.
+    if (w.alone && key.prec != kPrecIQ) {
+        const int tiles = (h->g.nx + kTileCols - 1) / kTileCols * ((h->g.nz + 15) / 16);
+        return kSoloConfig + (4 * tiles <= 3 * h->sms ? 2 : 2 * tiles <= 3 * h->sms ? 1 : 0);
+    }
+    if (w.peers >= kMaxFramesPerJob && narrow_ok)
+        return key.prec == kPrecIQ ? 4 : 6;
+    return 0;
+}
+
+// The angle tables of a plan key, shared by its tilings (the handle's lock is held).
+static int angle_tables_dev(bf_handle *h, PlanKey key, std::shared_ptr<AngleTablesDev> &out)
+{
+    key.prec = key.cfg = 0;
+    auto it = h->angle_tabs.find(key);
+    if (it != h->angle_tabs.end()) {
+        out = it->second;
+        return BF_OK;
+    }
+    PlanHost ph;
+    angle_tables(h->g, h->geo, key.ns, key.angles, ph);
+    const std::vector<int16_t> valid(ph.valid.begin(), ph.valid.end());  // rows are below 2^15
+    auto t = std::make_shared<AngleTablesDev>();
+    int rc = t->colK.upload(ph.colK.data(), ph.colK.size() * sizeof(int));
+    if (!rc) rc = t->colF.upload(ph.colF.data(), ph.colF.size() * sizeof(float));
+    if (!rc) rc = t->rowK.upload(ph.rowK.data(), ph.rowK.size() * sizeof(int));
+    if (!rc) rc = t->rowF.upload(ph.rowF.data(), ph.rowF.size() * sizeof(float));
+    if (!rc) rc = t->valid.upload(valid.data(), valid.size() * sizeof(int16_t));
+    if (rc)
+        return rc;
+    h->angle_tabs.emplace(std::move(key), t);
+    out = t;
+    return BF_OK;
 }
 
 int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t flags, Plan **out,
-                int cfg)
+                const PlanWish &wish)
 {
-    const int prec = frame_prec(flags);
-    const bool narrow_ok = (flags & BF_MODE_MASK & ~(BF_DAS | BF_DMAS)) == 0;
+    const int prec = frame_prec(flags), cfg = wish.cfg;
+    const bool narrow_ok = sharing_modes(flags);
     PlanKey key{ns, prec, std::vector<double>(angles, angles + na), 0};
     std::lock_guard<std::mutex> lk(h->mu);
-    key.cfg = (cfg >= 0 && cfg < kNumTileConfigs) ? cfg : choose_cfg(h, key);
-    if (kTileConfigs[key.cfg].rows == 2 && !narrow_ok) {
+    key.cfg = (cfg >= 0 && cfg < kNumTileConfigs) ? cfg : choose_cfg(h, key, wish, narrow_ok);
+    const bool solo = key.cfg >= kSoloConfig;
+    if (!solo && kTileConfigs[key.cfg].rows == 2 && !narrow_ok) {
         if (cfg >= 0)
             return fail(BF_EINVAL, "two-row tiles serve DAS / DMAS and IQ-DAS / BB-DMAS only");
         key.cfg = 0;
@@ -281,36 +332,83 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
         *out = it->second.get();
         return BF_OK;
     }
-    PlanHost ph;
-    const TileConfig tc = kTileConfigs[key.cfg];
-    angle_tables(h->g, h->geo, ns, key.angles, prec, tc.rows, tc.stage_bytes, ph);
-    if (beamform_smem_bytes(ph.wmax, ph.group, prec, 1, ph.rows) > (size_t)kMaxSmemPerCta)
+    // the default tiles' window bounds the pixel spacing, whichever tiles a rule chose
+    const TileConfig tc = kTileConfigs[solo ? 0 : key.cfg];
+    int wmax = 0, box = 0, group = 0;
+    auto fits = [&](const TileConfig &t) {
+        tile_window(h->g, key.angles, prec, tile_rows(t.rows), 1, wmax, box);
+        group = stage_channels(wmax, prec, t.rows, t.stage_bytes, h->g.ne);
+        return beamform_smem_bytes(wmax, group, prec, 1, t.rows) <= (size_t)kMaxSmemPerCta;
+    };
+    const bool by_rule = cfg < 0 && forced_cfg() < 0 && h->tuned.find(tuned_key(key)) == h->tuned.end();
+    if ((by_rule && !fits(kTileConfigs[0])) || !fits(tc))
         return fail(BF_EINVAL,
                     "pixel spacing too coarse for the sample rate: one tile needs %d samples per channel",
-                    ph.wmax);
+                    wmax);
+    int rows = tc.rows, bands = kWarps, tr = tile_rows(tc.rows), split = 0, ang = 1, ngr = 1, run = 1;
+    if (solo) {
+        split = 1 << (key.cfg - kSoloConfig);
+        rows = 2;
+        bands = kWarps / split;
+        tr = rows * bands;
+        // Channels per window copy (four, two or one) and angles per stage (up to
+        // four): the most whose windows for one copy's channels leave three CTAs per
+        // SM their shared memory; failing that what fits one CTA.
+        const int all = BF_DMAS | BF_CF | BF_PDAS, pb = pair_bytes(prec);
+        auto per_channel = [&](int an) { return kTileCols * 4 * (1 + an) + an * wmax * pb; };
+        run = h->g.ne >= 4 ? 4 : h->g.ne >= 2 ? 2 : 1;
+        for (ang = std::min(kSoloAngles, na);;) {
+            tile_window(h->g, key.angles, prec, tr, run, wmax, box);
+            if (wmax == box && run * per_channel(ang) <= kSoloStageBytes)
+                break;
+            if (run > 1)
+                run /= 2;
+            else if (ang > 1 && (ang > 2 || solo_smem_bytes(wmax, 1, prec, ang, split, all) >
+                                                (size_t)kMaxSmemPerCta))
+                --ang;
+            else
+                break;
+        }
+        // angle groups and channel steps as even as possible
+        ngr = (na + ang - 1) / ang;
+        ang = (na + ngr - 1) / ngr;
+        const int cap = std::min({kMaxGroup, 32 / ang * run, h->g.ne}) / run * run;
+        group = std::min(cap, std::max(run, kSoloStageBytes / per_channel(ang) / run * run));
+        const int steps = (h->g.ne + group - 1) / group;
+        group = std::min(cap, ((h->g.ne + steps - 1) / steps + run - 1) / run * run);
+    }
     auto p = std::make_unique<Plan>();
+    int rc = angle_tables_dev(h, key, p->at);
+    if (rc)
+        return rc;
     p->ns = ns;
     p->na = na;
     p->prec = prec;
-    p->wmax = ph.wmax;
-    p->box = ph.box;
-    p->group = ph.group;
-    p->nsp = ph.nsp;
-    p->rows = ph.rows;
+    p->wmax = wmax;
+    p->box = box;
+    p->run = run;
+    p->group = group;
+    p->nsp = (ns + kPadL + 7) / 8 * 8;
+    p->rows = rows;
+    p->split = split;
+    p->ang = ang;
+    p->ang_groups = ngr;
     p->tiles_x = (h->g.nx + kTileCols - 1) / kTileCols;
-    p->tiles_z = (h->g.nz + tile_rows(ph.rows) - 1) / tile_rows(ph.rows);
+    p->tiles_z = (h->g.nz + tr - 1) / tr;
     const int nxp = pad_cols(h->g.nx), ne = h->g.ne;
-    int rc = p->colK.upload(ph.colK.data(), ph.colK.size() * sizeof(int));
-    if (!rc) rc = p->colF.upload(ph.colF.data(), ph.colF.size() * sizeof(float));
-    if (!rc) rc = p->rowK.upload(ph.rowK.data(), ph.rowK.size() * sizeof(int));
-    if (!rc) rc = p->rowF.upload(ph.rowF.data(), ph.rowF.size() * sizeof(float));
-    if (!rc) rc = p->valid.upload(ph.valid.data(), ph.valid.size() * sizeof(int));
-    if (!rc) rc = p->wtab.ensure((size_t)na * p->tiles_x * p->tiles_z * ne * sizeof(int));
-    if (!rc) rc = p->btab.ensure((size_t)na * p->tiles_x * p->tiles_z * ne * sizeof(int));
+    const size_t ntiles = (size_t)p->tiles_x * p->tiles_z;
+    if (solo) {
+        const size_t steps = (size_t)ngr * ((ne + group - 1) / group);
+        if (!rc) rc = p->wtab.ensure(steps * ntiles * solo_record_words(ang, group / run) * sizeof(int));
+    } else {
+        if (!rc) rc = p->wtab.ensure(na * ntiles * ne * sizeof(int));
+        if (!rc) rc = p->btab.ensure(na * ntiles * ne * sizeof(int));
+    }
     if (rc)
         return rc;
     CUtensorMap maps[2];
-    rc = encode_map(&maps[0], p->valid.p, na * ne, nxp, 8, kTileCols, p->group);
+    rc = encode_map(&maps[0], p->at->valid.p, solo ? ne : na * ne, nxp, 4, kTileCols, p->group,
+                    solo ? na : 0, ang);
     if (!rc)
         rc = encode_map(&maps[1], h->dx2.p, ne, nxp, 4, kTileCols, p->group);
     if (!rc)
@@ -319,12 +417,12 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
         return rc;
     // window starts of every (angle, tile, channel), once per plan
     PlanJob pj{};
-    pj.colK = (const int *)p->colK.p;
-    pj.colF = (const float *)p->colF.p;
-    pj.rowK = (const int *)p->rowK.p;
-    pj.rowF = (const float *)p->rowF.p;
+    pj.colK = (const int *)p->at->colK.p;
+    pj.colF = (const float *)p->at->colF.p;
+    pj.rowK = (const int *)p->at->rowK.p;
+    pj.rowF = (const float *)p->at->rowF.p;
     pj.rowZ = (const float *)h->rowZ.p;
-    pj.valid = (const int2 *)p->valid.p;
+    pj.valid = (const short2 *)p->at->valid.p;
     pj.dx2 = (const float *)h->dx2.p;
     pj.wtab = (int *)p->wtab.p;
     pj.btab = (int *)p->btab.p;
@@ -334,10 +432,14 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
     pj.na = na;
     pj.ne = ne;
     pj.rows = p->rows;
+    pj.bands = bands;
     pj.tiles_x = p->tiles_x;
     pj.tiles_z = p->tiles_z;
     pj.wmax = p->wmax;
-    pj.align = ph.align;
+    pj.align = 16 / pair_bytes(prec);
+    pj.ang_groups = ngr;
+    pj.run = run;
+    pj.group = group;
     DevMem errw;
     rc = errw.ensure(sizeof(int));
     if (rc)
@@ -349,7 +451,7 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
     int herr = 0;
     e = cudaMemsetAsync(errw.p, 0, sizeof(int), st);
     if (e == cudaSuccess)
-        e = launch_plan(pj, (int *)errw.p, st);
+        e = solo ? launch_solo_plan(pj, (int *)errw.p, st) : launch_plan(pj, (int *)errw.p, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&herr, errw.p, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess)
@@ -430,9 +532,30 @@ size_t frame_out_bytes(const bf_handle *h, uint32_t flags)
 
 static int plan_frames_per_job(const Plan *p, int modes, int prec, int cap);
 
+// The frame's tensor map of its own pairs, encoded when the layout changed
+// (uploaded by upload_maps).
+static int frame_map(const FramePrep &f, FrameScratch &s, int rows)
+{
+    const Plan *p = f.plan;
+    if (s.map_base == s.pairs.p && s.map_rows == rows && s.map_nsp == p->nsp &&
+        s.map_box == p->box && s.map_run == p->run && s.map_prec == f.prec)
+        return BF_OK;
+    int rc = encode_pairs_map(&s.map_host, s.pairs.p, rows, p->nsp, p->box, p->run, f.prec);
+    if (rc)
+        return rc;
+    s.map_base = s.pairs.p;
+    s.map_rows = rows;
+    s.map_nsp = p->nsp;
+    s.map_box = p->box;
+    s.map_run = p->run;
+    s.map_prec = f.prec;
+    s.map_dirty = true;
+    return BF_OK;
+}
+
 int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *angles, int na,
-                  uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int cfg,
-                  int nf_cap)
+                  uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int nf_cap,
+                  PlanWish wish, bool late_solo)
 {
     int rc = check_frame_args(h, ns, angles, na, flags);
     if (rc)
@@ -440,7 +563,13 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     const int prec = frame_prec(flags);
     const bool iq = prec == kPrecIQ;
     Plan *plan = nullptr;
-    rc = handle_plan(h, ns, angles, na, flags, &plan, cfg);
+    wish.alone = nf_cap == 1 || !sharing_modes(flags);
+    Plan *solo = nullptr;
+    rc = handle_plan(h, ns, angles, na, flags, &plan, wish);
+    if (!rc && late_solo && !wish.alone) {
+        wish.alone = true;
+        rc = handle_plan(h, ns, angles, na, flags, &solo, wish);
+    }
     if (rc)
         return rc;
     const int modes = flags & (BF_MODE_MASK | BF_IQ_MASK), nm = frame_images(flags);
@@ -465,6 +594,7 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     fp = FramePrep{};
     fp.h = h;
     fp.plan = plan;
+    fp.solo = solo;
     fp.rf = rf_dev;
     fp.ns = ns;
     fp.na = na;
@@ -484,18 +614,9 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     fp.maxbits = (unsigned *)s.maxbits.p;
     fp.map_dev = (CUtensorMap *)s.map.p;
     fp.nf_cap = cap;
-    if (s.map_base != s.pairs.p || s.map_rows != rows || s.map_nsp != plan->nsp ||
-        s.map_box != plan->box || s.map_prec != prec) {
-        rc = encode_pairs_map(&s.map_host, s.pairs.p, rows, plan->nsp, plan->box, prec);
-        if (rc)
-            return rc;
-        s.map_base = s.pairs.p;
-        s.map_rows = rows;
-        s.map_nsp = plan->nsp;
-        s.map_box = plan->box;
-        s.map_prec = prec;
-        s.map_dirty = true;
-    }
+    rc = frame_map(fp, s, rows);
+    if (rc)
+        return rc;
     fp.map_host = s.map_host;
     fp.map_dirty = s.map_dirty;
     fp.scratch = &s;
@@ -525,7 +646,7 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
 static int plan_frames_per_job(const Plan *p, int modes, int prec, int cap)
 {
     const int m = modes & (BF_MODE_MASK | BF_IQ_MASK);
-    if ((m & ~(BF_DAS | BF_DMAS | BF_IQ_MASK)) != 0)
+    if (p->split || !sharing_modes((uint32_t)m))
         return 1;
     if (prec == kPrecIQ && demod_smem_bytes(p->ns, true) > (size_t)kMaxSmemPerCta)
         return 1;  // a frame pair's demodulation does not fit one CTA
@@ -580,6 +701,27 @@ static bool shareable(const FramePrep &a, const FramePrep &b)
            a.prec == b.prec && a.na == b.na && a.ns == b.ns;
 }
 
+int use_solo_plans(std::vector<FramePrep> &frames)
+{
+    for (size_t i = 0; i < frames.size(); ++i) {
+        FramePrep &f = frames[i];
+        if (!f.solo || !f.solo->split)
+            continue;
+        bool alone = true;
+        for (size_t j = 0; j < frames.size() && alone; ++j)
+            alone = j == i || !(frames[j].solo == f.solo && shareable(f, frames[j]));
+        if (!alone)
+            continue;
+        f.plan = f.solo;
+        int rc = frame_map(f, *f.scratch, f.na * f.h->g.ne);
+        if (rc)
+            return rc;
+        f.map_host = f.scratch->map_host;
+        f.map_dirty = f.scratch->map_dirty;
+    }
+    return BF_OK;
+}
+
 void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
 {
     hl = HostLaunch{};
@@ -616,10 +758,10 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         const bf_handle *h = f.h;
         const Plan *p = f.plan;
         BfJob j{};
-        j.colK = (const int *)p->colK.p;
-        j.colF = (const float *)p->colF.p;
-        j.rowK = (const int *)p->rowK.p;
-        j.rowF = (const float *)p->rowF.p;
+        j.colK = (const int *)p->at->colK.p;
+        j.colF = (const float *)p->at->colF.p;
+        j.rowK = (const int *)p->at->rowK.p;
+        j.rowF = (const float *)p->at->rowF.p;
         j.rowZ = (const float *)h->rowZ.p;
         j.wtab = (const int *)p->wtab.p;
         j.btab = (const int *)p->btab.p;
@@ -635,6 +777,8 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         j.wmax = p->wmax;
         j.box = p->box;
         j.group = p->group;
+        j.ang_groups = p->ang_groups;
+        j.run = p->run;
         j.rows = p->rows;
         // the IQ kernel reads its two combiners from the DAS / DMAS slots of the mode word
         j.modes = f.prec == kPrecIQ ? (((f.modes & BF_IQDAS) ? BF_DAS : 0) |
@@ -659,16 +803,20 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
             j.rf_map = (const CUtensorMap *)f.scratch->map_nf.p;
             j.box = box_nf;
         }
+        const int combiners = j.modes & (BF_DMAS | BF_CF | BF_PDAS);
         const int variant =
-            ((nf * 16 + p->rows) * 4 + f.prec) * 16 + (j.modes & (BF_DMAS | BF_CF | BF_PDAS));
+            (((p->split * 8 + nf) * 16 + p->rows) * 4 + f.prec) * 16 + combiners;
         groups[variant].push_back(j);
-        const size_t sm = beamform_smem_bytes(p->wmax, p->group, f.prec, nf, p->rows);
+        const size_t sm = p->split
+                              ? solo_smem_bytes(p->wmax, p->group, f.prec, p->ang, p->split, combiners)
+                              : beamform_smem_bytes(p->wmax, p->group, f.prec, nf, p->rows);
         group_smem[variant] = std::max(group_smem[variant], sm);
         hl.smem = std::max(hl.smem, sm);
     }
     for (auto &kv : groups) {
         HostLaunch::Group g;
-        g.nf = kv.first / (16 * 4 * 16);
+        g.split = kv.first / (8 * 16 * 4 * 16);
+        g.nf = (kv.first / (16 * 4 * 16)) % 8;
         g.rows = (kv.first / 64) % 16;
         g.prec = (kv.first / 16) % 4;
         g.variant = kv.first % 16;
@@ -964,9 +1112,12 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
     for (const HostLaunch::Group &g : hl.groups) {
-        e = launch_beamform((const BfJob *)dl.jobs.p + g.first,
-                            (const int *)dl.tile_prefix.p + g.prefix_first, g.count, g.tiles, g.smem,
-                            g.prec, g.variant, g.rows, g.nf, (int *)dl.err.p, st);
+        const BfJob *jobs = (const BfJob *)dl.jobs.p + g.first;
+        const int *prefix = (const int *)dl.tile_prefix.p + g.prefix_first;
+        e = g.split ? launch_solo(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant, g.split,
+                                  (int *)dl.err.p, st)
+                    : launch_beamform(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant,
+                                      g.rows, g.nf, (int *)dl.err.p, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "beamform launch");
     }
@@ -1085,6 +1236,9 @@ BF_API int bf_create(const bf_geometry *geom, const bf_grid *grid, double fs_hz,
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaStreamCreate");
     h->stream = h->own_stream;
+    e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "cudaDeviceGetAttribute");
     geometry_tables(g, h->geo);
     int rc = h->rowZ.upload(h->geo.rowZ.data(), h->geo.rowZ.size() * sizeof(float));
     if (!rc) rc = h->dx2.upload(h->geo.dx2.data(), h->geo.dx2.size() * sizeof(float));
@@ -1152,7 +1306,8 @@ BF_API int bf_beamform(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         if (rc)
             return rc;
         Plan *plan = nullptr;
-        rc = handle_plan(h, n_samples, angles_rad, n_angles, flags, &plan);
+        rc = handle_plan(h, n_samples, angles_rad, n_angles, flags, &plan,
+                         PlanWish{-1, 1, true});
         if (rc)
             return rc;
         if (plan == cc.plan && flags == cc.flags && rf_dev == cc.rf && out_dev == cc.out &&
@@ -1390,7 +1545,7 @@ BF_API int bf_beamform_plain(bf_handle *h, const int16_t *rf_dev, int32_t n_samp
     HostLaunch hl;
     build_launch(frames, hl);
     const BfJob &job = hl.jobs[0];
-    cudaError_t e = launch_plain(job, rf_dev, (const int2 *)frames[0].plan->valid.p,
+    cudaError_t e = launch_plain(job, rf_dev, (const short2 *)frames[0].plan->at->valid.p,
                                  (const float *)h->dx2.p, pad_cols(h->g.nx), n_samples, h->stream);
     if (e != cudaSuccess)
         return cuda_fail(e, "plain kernel launch");
@@ -1466,7 +1621,7 @@ BF_API int bf_host_tables(const bf_geometry *geom, const bf_grid *grid, double f
     geometry_tables(g, geo);
     PlanHost ph;
     angle_tables(g, geo, n_samples, std::vector<double>(angles_rad, angles_rad + n_angles),
-                 kPrecF32, 8, kTileConfigs[0].stage_bytes, ph);
+                 ph);
     const int nxp = pad_cols(g.nx);
     if (valid_rows)  // [na][ne][nxp][2] -> [na][nx][ne][2]
         for (int a = 0; a < n_angles; ++a)
@@ -1552,7 +1707,7 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
         for (int i = 0; i < frames && !prc; ++i)
             prc = prepare_frame(h, (const int16_t *)rf.p, n_samples, angles_rad, n_angles, fl,
                                 (float *)out.p + (size_t)i * (out_bytes / sizeof(float)),
-                                scratch[i], fr[i], c, kMaxFramesPerJob);
+                                scratch[i], fr[i], kMaxFramesPerJob, PlanWish{c});
         if (prc)
             continue;  // this configuration does not fit the workload
         HostLaunch hl;
@@ -1610,6 +1765,15 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
 
 // ------------------------------------------------------------------ batch --
 
+// Whether two frames of a batch can share a beamforming job (see shareable).
+static bool same_job(const bf_frame &a, const bf_frame &b)
+{
+    const uint32_t m = BF_MODE_MASK | BF_IQ_MASK | BF_PREC_MASK;
+    return a.h == b.h && a.n_samples == b.n_samples && a.n_angles == b.n_angles &&
+           (a.mode_and_flags & m) == (b.mode_and_flags & m) && a.n_angles > 0 && a.angles_rad &&
+           b.angles_rad && std::equal(a.angles_rad, a.angles_rad + a.n_angles, b.angles_rad);
+}
+
 BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
 {
     if (!frames || !out || n < 1)
@@ -1630,9 +1794,12 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
         cudaSetDevice(dev);
         if (!is_device_pointer(f.rf_dev) || !is_device_pointer(f.out_dev))
             return fail(BF_EINVAL, "frame %d: batches need device pointers", i);
+        int peers = 0;  // frames of the batch with the same plan and combiners
+        for (int j = 0; j < n; ++j)
+            peers += same_job(f, frames[j]) ? 1 : 0;
         int rc = prepare_frame(f.h, f.rf_dev, f.n_samples, f.angles_rad, f.n_angles,
-                               f.mode_and_flags, f.out_dev, b->scratch[i], b->frames[i], -1,
-                               kMaxFramesPerJob);
+                               f.mode_and_flags, f.out_dev, b->scratch[i], b->frames[i],
+                               peers > 1 ? kMaxFramesPerJob : 1, PlanWish{-1, peers});
         if (rc)
             return fail(rc, "frame %d: %s", i, g_err.c_str());
     }

@@ -339,7 +339,7 @@ public:
     int submit(bf_handle *h, const int16_t *rf, int ns, const double *angles, int na,
                uint32_t flags, uint64_t *ticket, bool wait_copy = true,
                std::vector<Deferred> *defer = nullptr, float *dest = nullptr,
-               uint64_t dest_group = 0, const CopyRoute *dest_route = nullptr);
+               uint64_t dest_group = 0, const CopyRoute *dest_route = nullptr, int peers = 1);
     // a fresh id for the destinations of one bf_submit_many_into call
     uint64_t next_dest_group() { return next_group_.fetch_add(1) + 1; }
     int flush(std::vector<Deferred> &defer);
@@ -441,7 +441,7 @@ void Engine::put_free(std::unique_ptr<Slot> s)
 
 int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles, int na,
                    uint32_t flags, uint64_t *ticket, bool wait_copy, std::vector<Deferred> *defer,
-                   float *dest, uint64_t dest_group, const CopyRoute *dest_route)
+                   float *dest, uint64_t dest_group, const CopyRoute *dest_route, int peers)
 {
     int rc = check_frame_args(h, ns, angles, na, flags);
     if (rc)
@@ -470,7 +470,8 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
     // admission by device memory: the slot may have to grow
     const int prec = frame_prec(flags);
     Plan *plan = nullptr;
-    rc = handle_plan(h, ns, angles, na, flags, &plan);
+    rc = handle_plan(h, ns, angles, na, flags, &plan,
+                     PlanWish{-1, peers, !sharing_modes(flags)});
     // staged pairs: room for the frames of a multi-frame job this frame may lead
     const int cap = plan ? job_frames_cap(plan, flags, kMaxFramesPerJob) : 1;
     size_t need = rf_bytes + out_bytes +
@@ -518,7 +519,7 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
         rc = fail(BF_ECUDA, "cudaEventCreate");
     if (!rc)
         rc = prepare_frame(h, (const int16_t *)s.rf.p, ns, angles, na, flags, (float *)s.out.p,
-                           s.scratch, req->fp, -1, kMaxFramesPerJob);
+                           s.scratch, req->fp, kMaxFramesPerJob, PlanWish{-1, peers}, peers == 1);
     if (rc) {
         std::lock_guard<std::mutex> lk(mu_);
         const size_t grow = need > before ? need - before : 0;
@@ -681,6 +682,8 @@ void Engine::launch(std::vector<std::shared_ptr<Request>> &reqs)
         f.out = to;
     }
     HostLaunch hl;
+    if (!rc)
+        rc = use_solo_plans(frames);
     build_launch(frames, hl);
     if (!rc)
         rc = upload_maps(frames, st, true);
@@ -1132,7 +1135,7 @@ static int submit_many(bf_handle *h, int32_t n, const int16_t *const *rf, int32_
             }
             rc = eng->submit(h, rf[k], n_samples, angles_rad, n_angles, flags, tickets_out + k,
                              false, &defer, outs ? outs[k] : nullptr, group,
-                             group ? &one_route : nullptr);
+                             group ? &one_route : nullptr, n);
             if (rc)
                 break;
         }

@@ -62,7 +62,7 @@ struct DevMem {
 struct PlanKey {
     int ns, prec;
     std::vector<double> angles;
-    int cfg = 0;  // index into kTileConfigs
+    int cfg = 0;  // index into kTileConfigs, or kSoloConfig + log2 of the split
     bool operator<(const PlanKey &o) const
     {
         if (ns != o.ns)
@@ -75,13 +75,24 @@ struct PlanKey {
     }
 };
 
-// Device tables of one (handle, sample count, precision, angle set): the
-// transmit tables, the counted-row intervals, the per-tile window starts and
-// the tensor maps through which the beamformer stages its per-tile tables.
+// Device tables of one (handle, sample count, angle set), shared by its plans: the
+// transmit tables and the counted-row intervals.
+struct AngleTablesDev {
+    DevMem colK, colF, rowK, rowF, valid;
+};
+
+// Tiling of one (handle, sample count, precision, angle set): the tables above, the
+// per-tile window starts and the tensor maps through which the beamformer stages
+// its per-tile tables.
 struct Plan {
+    std::shared_ptr<AngleTablesDev> at;
     int ns = 0, na = 0, prec = 0;
     int wmax = 0, box = 0, group = 1, nsp = 0, rows = 8, tiles_x = 0, tiles_z = 0;
-    DevMem colK, colF, rowK, rowF, valid, wtab, btab;
+    // solo plans (split > 0): warps per row pair, angles per stage, groups of them,
+    // channels per window copy
+    int split = 0, ang = 1, ang_groups = 1;
+    int run = 1;
+    DevMem wtab, btab;
     DevMem maps;  // CUtensorMap[2]: valid rows, dx^2
 };
 
@@ -101,7 +112,7 @@ struct FrameScratch {
     DevMem pairs, y, env, maxbits, map;
     CUtensorMap map_host{};
     void *map_base = nullptr;
-    int map_rows = 0, map_nsp = 0, map_box = 0, map_prec = -1;
+    int map_rows = 0, map_nsp = 0, map_box = 0, map_run = 0, map_prec = -1;
     bool map_dirty = false;
     // as the lead of a multi-frame job: pairs holds the job's frames interleaved
     // ([row][pair][frame]) and map_nf describes that layout
@@ -115,6 +126,7 @@ struct FrameScratch {
 struct FramePrep {
     bf_handle *h = nullptr;
     Plan *plan = nullptr;
+    Plan *solo = nullptr;  // the plan to use if the launch has no partner for the frame, or null
     std::shared_ptr<EnvTablesDev> et[2];  // envelope tables: without band, the DMAS band
     std::shared_ptr<FftTablesDev> ft;     // level twiddles, or the warp kernel's 512-point table
     std::shared_ptr<FftTablesDev> dt;     // demodulation transform tables (n_samples; IQ only)
@@ -133,8 +145,8 @@ struct FramePrep {
 };
 
 struct HostLaunch {
-    struct Group {  // one beamforming launch
-        int prec, variant, rows, nf, first, count, prefix_first, tiles;
+    struct Group {  // one beamforming launch (split > 0: solo jobs)
+        int prec, variant, rows, nf, split, first, count, prefix_first, tiles;
         size_t smem;
     };
     struct IGroup {  // one ingest launch
@@ -204,7 +216,7 @@ struct CallCache {
 }  // namespace bfi
 
 struct bf_handle {
-    int device = 0;
+    int device = 0, sms = 1;
     bfi::GeomHost g;
     bfi::GeometryHost geo;
     cudaStream_t stream = nullptr, own_stream = nullptr;
@@ -213,6 +225,8 @@ struct bf_handle {
     double pdas_p = 2.0;  // order of the pDAS combiner
     std::mutex mu;  // plans, tickets, slot pool
     std::map<bfi::PlanKey, std::unique_ptr<bfi::Plan>> plans;
+    // their angle tables (key prec = cfg = 0)
+    std::map<bfi::PlanKey, std::shared_ptr<bfi::AngleTablesDev>> angle_tabs;
     std::map<bfi::PlanKey, int> tuned;  // tile configuration bf_autotune chose (key cfg = 0)
     bfi::FrameScratch scratch;     // bf_beamform
     bfi::DeviceLaunch launch;      // bf_beamform
@@ -237,13 +251,23 @@ struct bf_batch {
 
 namespace bfi {
 
+// What is known about a frame's launch when its plan is chosen.
+struct PlanWish {
+    int cfg = -1;   // a configuration of kTileConfigs, or < 0: by the rules of choose_cfg
+    int peers = 1;  // frames of this plan and combiners submitted together (jobs of four)
+    bool alone = false;  // the frame shares its plan with no other: RF frames take solo tiles
+};
 // Plan of a frame with these arguments (`flags`: its mode and precision bits).
-// cfg < 0: the configuration bf_autotune chose for this workload, else the
-// default; a two-row configuration serves DAS / DMAS of RF records and
-// IQ-DAS / BB-DMAS only (an explicit one is refused for other frames, a tuned
-// one replaced by the default).
+// BF_TILE_ROWS and bf_autotune's choice for the workload come before the rules; a
+// two-row configuration serves DAS / DMAS of RF records and IQ-DAS / BB-DMAS only
+// (an explicit one is refused for other frames, a tuned one replaced by the default).
 int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t flags, Plan **out,
-                int cfg = -1);
+                const PlanWish &wish = {});
+// Whether frames with these combiners ever share a job.
+inline bool sharing_modes(uint32_t flags)
+{
+    return (flags & BF_MODE_MASK & ~(uint32_t)(BF_DAS | BF_DMAS)) == 0;
+}
 int check_frame_args(bf_handle *h, int ns, const double *angles, int na, uint32_t flags);
 size_t frame_out_bytes(const bf_handle *h, uint32_t flags);
 // Storage code of a frame's staged records (kPrecIQ for the IQ combiners).
@@ -251,9 +275,14 @@ int frame_prec(uint32_t flags);
 // nf_cap: frames of one plan a later build_launch may put in one job with
 // this frame (1: alone, as a single bf_beamform call); the frame's scratch
 // is sized for the multi-frame jobs its plan and combiners allow up to that.
+// With nf_cap 1, or combiners no job shares, the plan is a solo plan where one
+// applies; late_solo: also find that plan for a frame that may turn out alone
+// (use_solo_plans).
 int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *angles, int na,
-                  uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int cfg = -1,
-                  int nf_cap = 1);
+                  uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int nf_cap = 1,
+                  PlanWish wish = {}, bool late_solo = false);
+// Frames of a launch that share no job with another one go over to their solo plans.
+int use_solo_plans(std::vector<FramePrep> &frames);
 // Frames (at most cap) of one plan that can share a beamforming job with a
 // frame of these flags (1 unless the combiners are DAS / DMAS of RF records
 // or IQ-DAS / BB-DMAS; IQ frames with records above 4096 samples alone).

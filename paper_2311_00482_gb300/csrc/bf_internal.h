@@ -43,6 +43,17 @@ constexpr TileConfig kTileConfigs[] = {{4, 24 << 10}, {4, 16 << 10}, {4, 32 << 1
 // otherwise (measured fastest for each).
 __host__ __device__ constexpr int stages_for_rows(int rows) { return rows == 2 ? 2 : 3; }
 constexpr int kNumTileConfigs = 7;
+// Solo tiles (bf_solo.cu): frames that share their plan with no other frame.
+// Configuration kSoloConfig + k runs SPLIT = 2^k: tiles of 16 / SPLIT rows.  Not
+// among the autotuner's candidates; angles share a stage, at most kSoloAngles.
+constexpr int kSoloConfig = kNumTileConfigs, kSoloAngles = 4;
+constexpr int kSoloStages = 2, kSoloStageBytes = 33 << 10;
+// Record of one (step, tile): 8 masks of fully and 8 of partly counted channels,
+// then the window starts [angle][run of channels]; [step][tile] in the plan's table.
+__host__ __device__ constexpr int solo_record_words(int ang, int runs)
+{
+    return 2 * kWarps + ang * runs;
+}
 // Frames of one plan that one beamforming job may carry (sharing every delay).
 constexpr int kMaxFramesPerJob = 4;
 
@@ -85,7 +96,7 @@ struct BfJob {
                           // channel, bit 8 + b every pixel of the band does
     const uint16_t *apcnt;// [nx][nz]  channels inside the aperture (CF denominator)
     const CUtensorMap *rf_map;     // sample pairs [na * ne][nsp]
-    const CUtensorMap *valid_map;  // int2 [na * ne][nxp]: first / last counted row, (-1, -1) if none
+    const CUtensorMap *valid_map;  // short2 [na * ne][nxp]: first / last counted row, (-1, -1) if none
     const CUtensorMap *dx2_map;    // float [ne][nxp]: max((kappa * (x_p - x_i))^2, 1e-30)
     float *y;             // [nmodes][nx][nz] beamformed output
     // further frames of the same plan sharing every delay (multi-frame jobs;
@@ -100,6 +111,10 @@ struct BfJob {
     int wmax;             // window length (pairs) staged per channel and tile
     int box;              // TMA box width (pairs); wmax is a multiple of it
     int group;            // channels per stage
+    // solo jobs: groups the angles are walked in; adjacent channels whose windows one
+    // copy brings (1, 2 or 4).  wtab then holds the records of solo_record_words,
+    // rf_map boxes are run rows high and valid_map is [na][ne][nxp].
+    int ang_groups, run;
     int rows;             // rows per thread (tile height = kWarps * rows)
     int modes;            // BF_DAS | BF_DMAS | BF_CF | BF_PDAS
     int tiles_x, tiles_z;
@@ -121,11 +136,12 @@ struct PlanJob {
     const int *rowK;
     const float *rowF;
     const float *rowZ;
-    const int2 *valid;    // [na][ne][nxp]
+    const short2 *valid;  // [na][ne][nxp]
     const float *dx2;     // [ne][nxp]
     int *wtab;            // [na][tiles][ne]
     int *btab;            // [na][tiles][ne]
-    int nx, nxp, nz, na, ne, rows, tiles_x, tiles_z, wmax, align;
+    int nx, nxp, nz, na, ne, rows, bands, tiles_x, tiles_z, wmax, align;
+    int ang_groups, run, group;  // solo plans
 };
 
 // One frame's int16 records to staged sample pairs.
@@ -248,6 +264,13 @@ cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, i
 __host__ __device__ constexpr int envelope_pairs_per_block(int lg) { return lg >= 12 ? 1 : 4096 >> lg; }
 cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int njobs,
                        int total_blocks, float dynamic_range_db, cudaStream_t stream);
+// Jobs of solo plans (bf_solo.cu; RF precisions, any RF combiners), all of one split.
+cudaError_t launch_solo(const BfJob *jobs_dev, const int *tile_prefix_dev, int njobs, int total_tiles,
+                        size_t smem_bytes, int prec, int variant, int split, int *err_dev,
+                        cudaStream_t stream);
+cudaError_t launch_solo_plan(const PlanJob &job, int *err_dev, cudaStream_t stream);
+// ang: angles of a stage; split: warps per row pair.
+size_t solo_smem_bytes(int wmax, int group, int prec, int ang, int split, int variant);
 // Envelope of 512-row images by the warp-per-column-pair kernel (bf_envelope.cu):
 // the depths it takes, and its launch
 // over total_pairs column pairs (pair_prefix_dev: each job's first pair).
@@ -256,7 +279,7 @@ cudaError_t launch_envelope_warp(const EnvJob *jobs_dev, const int *pair_prefix_
                                  int total_pairs, cudaStream_t stream);
 // One frame through the plain baseline kernel (FP32, global loads, one thread
 // per pixel); job.y receives the beamformed modes.
-cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const int2 *valid, const float *dx2,
+cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const short2 *valid, const float *dx2,
                          int nxp, int ns, cudaStream_t stream);
 // Dynamic shared memory of a beamforming CTA: header, the multi-frame
 // staging area (nf > 1) and the pipeline stages.

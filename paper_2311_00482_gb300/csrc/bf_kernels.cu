@@ -22,8 +22,6 @@
 //                    carrier phase) serves all of them, and a storer warp
 //                    writes the staged tile images with bulk copies
 //   log_kernel       20 log10(env / max) clipped to the -70 dB range of Fig. 3
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <limits.h>
 
 #include <algorithm>
@@ -32,151 +30,12 @@
 #include <utility>
 
 #include "../../include/bf.h"
+#include "bf_device.cuh"
 #include "bf_fft.cuh"
 #include "bf_internal.h"
 
 namespace bfi {
 namespace {
-
-constexpr float kRoundMagic = 12582912.0f;  // 1.5 * 2^23: x + magic rounds x to an integer
-constexpr int kRoundBits = 0x4B400000;      // bit pattern of kRoundMagic
-constexpr unsigned long long kWaitNs = 4000000000ull;  // bounded wait per CTA (4 s)
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_fence_init()
-{
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Wait for a barrier phase until the CTA's deadline; false (and an error bit)
-// if it passed.  Every wait of the CTA shares one deadline, so a stuck copy
-// costs at most kWaitNs before the CTA gives up on all remaining steps.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity,
-                                          unsigned long long deadline, int *err)
-{
-    if (mbar_try_wait(bar, parity))
-        return true;
-    while (global_ns() < deadline)
-        if (mbar_try_wait(bar, parity))
-            return true;
-    atomicOr(err, kErrTimeout);
-    return false;
-}
-
-// One 2-D tensor-map box into shared memory, completing on `bar`.
-__device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *map, int x, int y,
-                                       uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ float rsqrt_approx(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ float sqrt_approx(float x)
-{
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// x^e for x >= 0, e > 0 as 2^(e log2 x) on the special-function unit
-// (x = 0: log2 gives -inf, 2^-inf = 0).
-__device__ __forceinline__ float pow_approx(float x, float e)
-{
-    float l, y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(l * e));
-    return y;
-}
-
-// sign(v) |v|^(1/p) of one delayed sample; p = 2 takes the square root.
-__device__ __forceinline__ float pdas_root(float v, float inv_p, bool square)
-{
-    const float av = fabsf(v);
-    return copysignf(square ? sqrt_approx(av) : pow_approx(av, inv_p), v);
-}
-
-// Receive path length beyond the depth term, in samples:
-//   q = sqrt(d2 + z^2) - z = d2 / (sqrt(d2 + z^2) + z),
-// d2 = (kappa (x_p - x_i))^2, z = kappa z_p.  The large, pixel-only part of
-// the delay (transmit leg + depth) comes from the host as an exact integer +
-// remainder, so FP32 only has to carry this small term, formed without
-// cancellation; its relative error (a few ulp) keeps the delay within ~1e-6
-// samples (float32 emulation: 1e-6 rms, 1e-5 max over |x_p - x_i| <= z_p / 3).
-// dx2 >= 1e-30 (host floor), so the square root never sees 0; dx2 + z^2 is
-// formed with one rounding.
-__device__ __forceinline__ float rx_excess(float dx2, float z)
-{
-    const float s = fmaf(z, z, dx2);
-    const float r = s * rsqrt_approx(s);
-    return dx2 * rcp_approx(r + z);
-}
-
-__device__ __forceinline__ int find_job(const int *__restrict__ prefix, int njobs, int bid)
-{
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(prefix + mid) <= bid)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
 
 // ------------------------------------------------------------------ plan --
 
@@ -184,7 +43,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanJob J, int *__restr
 {
     const int t = blockIdx.x, a = blockIdx.y;
     const int tx = t % J.tiles_x, tz = t / J.tiles_x;
-    const int th = kWarps * J.rows;
+    const int th = J.bands * J.rows;
     const int tz0 = tz * th, tz_last = min(tz0 + th - 1, J.nz - 1);
     for (int i = threadIdx.x; i < J.ne; i += blockDim.x) {
         int kmin = INT_MAX, kmax = INT_MIN;
@@ -193,9 +52,9 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanJob J, int *__restr
             const int ix = tx * kTileCols + w;
             if (ix >= J.nx)
                 break;
-            const int2 vr = J.valid[((size_t)a * J.ne + i) * J.nxp + ix];
+            const short2 vr = J.valid[((size_t)a * J.ne + i) * J.nxp + ix];
             // row bands of the consumer warps: does some / every pixel of this column count?
-            for (int b = 0; b < kWarps; ++b) {
+            for (int b = 0; b < J.bands; ++b) {
                 const int b0 = tz0 + b * J.rows, b1 = min(b0 + J.rows - 1, J.nz - 1);
                 if (b0 > b1)
                     continue;  // band below the grid: nothing to store there
@@ -204,7 +63,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanJob J, int *__restr
                 if (!(vr.x <= b0 && vr.y >= b1))
                     full &= ~(1u << b);
             }
-            const int r0 = max(vr.x, tz0), r1 = min(vr.y, tz_last);
+            const int r0 = max((int)vr.x, tz0), r1 = min((int)vr.y, tz_last);
             if (r0 > r1)
                 continue;
             const float d2 = J.dx2[(size_t)i * J.nxp + ix];
@@ -481,110 +340,11 @@ struct SmemHeader {
 constexpr int kHeaderBytes = 4608;
 static_assert(sizeof(SmemHeader) <= kHeaderBytes, "header");
 
-// Sample pairs read from shared memory through 32-bit shared-window addresses.
-template <int PREC>
-struct PairIO;
-
-template <>
-struct PairIO<kPrecF32> {
-    static constexpr int kBytes = 8;
-    __device__ static __forceinline__ float interp(uint32_t addr, float al)
-    {
-        float mid, diff;
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(mid), "=f"(diff) : "r"(addr));
-        return fmaf(al, diff, mid);
-    }
-};
-
-template <>
-struct PairIO<kPrecF16> {
-    static constexpr int kBytes = 4;
-    __device__ static __forceinline__ float interp(uint32_t addr, float al)
-    {
-        unsigned w;
-        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(addr));
-        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w));
-        return fmaf(al + 0.5f, f.y - f.x, f.x);
-    }
-};
-
-template <>
-struct PairIO<kPrecBF16> {
-    static constexpr int kBytes = 4;
-    __device__ static __forceinline__ float interp(uint32_t addr, float al)
-    {
-        unsigned w;
-        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(addr));
-        const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xffff0000u);
-        return fmaf(al + 0.5f, hi - lo, lo);
-    }
-};
-
-// Loads through 32-bit shared-window addresses (the consumer loop's tables).
-__device__ __forceinline__ float4 lds_f32x4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(addr));
-    return v;
-}
-
-__device__ __forceinline__ int2 lds_int2(uint32_t addr)
-{
-    int2 v;
-    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-    return v;
-}
-
-__device__ __forceinline__ float lds_f32(uint32_t addr)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-    return v;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void sts_f32x2(uint32_t addr, float a, float b)
-{
-    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
-}
-
-// This thread's shared-memory writes, visible to the async proxy (bulk copies).
-__device__ __forceinline__ void fence_proxy_async_smem()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Bulk copy shared -> global (16-byte aligned addresses, size a multiple of 16),
-// tracked in this thread's bulk groups.
-__device__ __forceinline__ void bulk_store(void *gdst, uint32_t ssrc, unsigned bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
-                 "r"(ssrc), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-
-// Every committed bulk copy of this thread has read its shared-memory source.
-__device__ __forceinline__ void bulk_wait_read()
-{
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
-// Every committed bulk copy of this thread is complete.
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
-// Bytes of one pipeline stage: tables (int2 rows + float dx^2) and windows.
+// Bytes of one pipeline stage: tables (short2 rows + float dx^2) and windows.
 // (nf frames' windows per channel in multi-frame jobs)
 __host__ __device__ __forceinline__ int stage_bytes(int group, int wmax, int pb, int nf = 1)
 {
-    return group * (kTileCols * 12 + nf * wmax * pb);
+    return group * (kTileCols * 8 + nf * wmax * pb);
 }
 
 // Multi-frame jobs stage their images in shared memory for the storer warp:
@@ -604,70 +364,6 @@ template <int NF>
 constexpr int beamform_threads()
 {
     return kThreads + 32 + (NF > 1 ? 32 : 0);
-}
-
-// ---- packed FP32 pairs (Blackwell f32x2 arithmetic): two rows' delays at once
-typedef unsigned long long f32x2_t;
-
-__device__ __forceinline__ f32x2_t pk2(float lo, float hi)
-{
-    f32x2_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-
-__device__ __forceinline__ void upk2(f32x2_t v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
-__device__ __forceinline__ f32x2_t fma2(f32x2_t a, f32x2_t b, f32x2_t c)
-{
-    f32x2_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ f32x2_t add2(f32x2_t a, f32x2_t b)
-{
-    f32x2_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2_t sub2(f32x2_t a, f32x2_t b)
-{
-    f32x2_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2_t mul2(f32x2_t a, f32x2_t b)
-{
-    f32x2_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-// Rounded delays of rows j and j + 1 for one channel (d2 packed twice): the
-// rx_excess arithmetic of both rows in paired instructions, each half with
-// exactly the scalar version's operations and roundings, plus the pixels'
-// remainders.  m holds the delay plus the rounding constant (integer in its
-// low bits), al the offset in [-1/2, 1/2].
-__device__ __forceinline__ void delay2(f32x2_t D2, f32x2_t Zp, f32x2_t Fp, float &ma, float &mb,
-                                       float &ala, float &alb)
-{
-    const f32x2_t s = fma2(Zp, Zp, D2);
-    float sa, sb;
-    upk2(s, sa, sb);
-    const f32x2_t r = mul2(s, pk2(rsqrt_approx(sa), rsqrt_approx(sb)));
-    float da, db;
-    upk2(add2(r, Zp), da, db);
-    const f32x2_t x = fma2(D2, pk2(rcp_approx(da), rcp_approx(db)), Fp);
-    const f32x2_t MG = pk2(kRoundMagic, kRoundMagic);
-    const f32x2_t m = add2(x, MG);
-    upk2(m, ma, mb);
-    upk2(sub2(x, sub2(m, MG)), ala, alb);
 }
 
 // Per-angle constants of a thread's rows, packed in row pairs for delay2: the
@@ -992,7 +688,7 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
     // launch's flat (frame, tile) list.  The stage ring runs on across tiles
     // (ring position r), so the copies of a CTA's next tile are in flight while
     // it finishes the current one.  Every stage has the launch's largest
-    // stage size; inside a stage the layout is the job's: int2 rows [G][32],
+    // stage size; inside a stage the layout is the job's: short2 rows [G][32],
     // float dx^2 [G][32], windows [G][wmax].
     constexpr int EPI = epi_bytes(NF, ROWS);
     constexpr int kStages = stages_for_rows(ROWS);
@@ -1087,7 +783,7 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
             const CUtensorMap *valid_map = J->valid_map;
             const CUtensorMap *dx2_map = J->dx2_map;
             const int box = J->box;
-            const unsigned meta_bytes = (unsigned)G * kTileCols * 12;
+            const unsigned meta_bytes = (unsigned)G * kTileCols * 8;
             // window start and band flags of this lane's channel at step s
             auto window_of = [&](int s) -> int2 {
                 const int a = s / ngroups, g = s - a * ngroups;
@@ -1182,13 +878,13 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&sh.full[st], total + meta_bytes);
                     tma_2d(base, valid_map, tx * kTileCols, a * ne + i0, &sh.full[st]);
-                    tma_2d(base + (size_t)G * kTileCols * 8, dx2_map, tx * kTileCols, i0,
+                    tma_2d(base + (size_t)G * kTileCols * 4, dx2_map, tx * kTileCols, i0,
                            &sh.full[st]);
                 }
                 __syncwarp();
                 if (bytes) {
                     unsigned char *dst =
-                        base + (size_t)G * kTileCols * 12 + (size_t)lane * NF * wmax * PB;
+                        base + (size_t)G * kTileCols * 8 + (size_t)lane * NF * wmax * PB;
                     const int row = a * ne + i0 + lane;
                     // multi-frame jobs: the frames' pairs interleaved ([pair][frame]),
                     // box pairs of every frame per copy
@@ -1293,16 +989,16 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
                 P.set(Z, fp);
             }
             const uint32_t base = smem_u32(stage_base(st));
-            const uint32_t vrb = base + (uint32_t)lane * 8;                          // int2 [G][32]
-            const uint32_t d2b = base + (uint32_t)G * kTileCols * 8 + (uint32_t)lane * 4;  // float [G][32]
-            const uint32_t wins = base + (uint32_t)G * kTileCols * 12;
+            const uint32_t vrb = base + (uint32_t)lane * 4;                          // short2 [G][32]
+            const uint32_t d2b = base + (uint32_t)G * kTileCols * 4 + (uint32_t)lane * 4;  // float [G][32]
+            const uint32_t wins = base + (uint32_t)G * kTileCols * 8;
             const uint32_t wfb = smem_u32(&sh.wf[st][0]);
             const int nf = sh.nfull[st][warp], nt = sh.ntot[st][warp];
             const uint8_t *L = sh.list[st][warp];
             auto win_of = [&](int c) { return wins + (uint32_t)(c * NF * wmax * PB); };
             auto w0_of = [&](int c) { return lds_int2(wfb + (uint32_t)c * 8).x; };
             auto d2_of = [&](int c) { return lds_f32(d2b + (uint32_t)c * (kTileCols * 4)); };
-            auto vr_of = [&](int c) { return lds_int2(vrb + (uint32_t)c * (kTileCols * 8)); };
+            auto vr_of = [&](int c) { return lds_rows(vrb + (uint32_t)c * (kTileCols * 4)); };
             int k = 0;
             if constexpr (IQ && NF > 1) {
                 // every channel once, its delay and carrier phase serving every frame
@@ -1630,7 +1326,7 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
 // and served paths.  Same tables and the same split delay as beamform_kernel.
 template <bool DMAS, bool CF>
 __global__ void __launch_bounds__(256) plain_kernel(const BfJob J, const int16_t *__restrict__ rf,
-                                                    const int2 *__restrict__ valid,
+                                                    const short2 *__restrict__ valid,
                                                     const float *__restrict__ dx2, int nxp, int ns)
 {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1645,7 +1341,7 @@ __global__ void __launch_bounds__(256) plain_kernel(const BfJob J, const int16_t
         const float f = __ldg(J.colF + a * J.nx + ix) + __ldg(J.rowF + a * J.nz + iz) - 0.5f;
         float T1 = 0.f, T2 = 0.f, P1 = 0.f;
         for (int i = 0; i < J.ne; ++i) {
-            const int2 vr = __ldg(valid + ((size_t)a * J.ne + i) * nxp + ix);
+            const short2 vr = __ldg(valid + ((size_t)a * J.ne + i) * nxp + ix);
             if (iz < vr.x || iz > vr.y)
                 continue;
             const float x = rx_excess(__ldg(dx2 + (size_t)i * nxp + ix), Z) + f;
@@ -2027,7 +1723,7 @@ cudaError_t launch_beamform(const BfJob *jobs_dev, const int *tile_prefix_dev, i
                                   cf, pdas, rows, err_dev, stream);
 }
 
-cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const int2 *valid, const float *dx2,
+cudaError_t launch_plain(const BfJob &job, const int16_t *rf, const short2 *valid, const float *dx2,
                          int nxp, int ns, cudaStream_t stream)
 {
     const long long px = (long long)job.nx * job.nz;

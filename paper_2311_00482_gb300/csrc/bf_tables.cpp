@@ -108,8 +108,7 @@ void geometry_tables(const GeomHost &g, GeometryHost &out)
 }
 
 void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
-                  const std::vector<double> &angles, int prec, int rows_per_thread,
-                  int stage_bytes, PlanHost &out)
+                  const std::vector<double> &angles, PlanHost &out)
 {
     const double kappa = g.fs / g.c;
     const int na = (int)angles.size();
@@ -121,10 +120,8 @@ void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
     // An empty row range is (-1, -1): row -1 never exists, and the kernel's
     // test (row - first) <= (last - first) in unsigned arithmetic stays exact.
     out.valid.assign((size_t)na * g.ne * nxp * 2, -1);
-    double smax = 0.0;
     for (int a = 0; a < na; ++a) {
         const double st = std::sin(angles[a]), ct = std::cos(angles[a]);
-        smax = std::max(smax, std::fabs(st));
         for (int ix = 0; ix < g.nx; ++ix) {
             double v = kappa * (grid_coord(g.x0, g.x1, g.nx, ix) * st);
             double k = std::nearbyint(v);
@@ -166,6 +163,16 @@ void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
             out.valid[o + 1] = hi;
         }
     });
+    out.nsp = (ns + kPadL + 7) / 8 * 8;
+}
+
+void tile_window(const GeomHost &g, const std::vector<double> &angles, int prec, int tile_rows,
+                 int run, int &wmax, int &box_out)
+{
+    const double kappa = g.fs / g.c;
+    double smax = 0.0;
+    for (double a : angles)
+        smax = std::max(smax, std::fabs(std::sin(a)));
     // Window of sample pairs one tile needs per channel, over the pixels that
     // count it: the delay grows by at most (1 + cos) kappa dz <= 2 kappa dz per
     // row and by at most (|sin| + 1 / sqrt(1 + 4 F^2)) kappa dx per column (the
@@ -173,15 +180,23 @@ void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
     // sqrt((x_p - x_i)^2 + z_p^2) inside the aperture |x_p - x_i| <= z_p / (2 F)).
     // Two counted pixels of a tile are joined by a row-then-column or
     // column-then-row path inside the aperture (the aperture widens with
-    // depth), so the spread adds up along it.  The planner checks every window
-    // against wmax (an error, never a silent clamp).
+    // depth), so the spread adds up along it.  Between the channels of a run the
+    // receive leg changes by at most 1 / sqrt(1 + 4 F^2) of their distance: the
+    // counted (x_p, z_p, x_i) form a convex cone, on which every one of these slopes
+    // holds, so a segment from one counted (pixel, channel) to another adds them up
+    // too.  The planner checks every window against wmax (an error, never a silent
+    // clamp).
     const int align = 16 / pair_bytes(prec);
     const double dz = g.nz > 1 ? (g.z1 - g.z0) / (double)(g.nz - 1) : 0.0;
     const double dx = g.nx > 1 ? (g.x1 - g.x0) / (double)(g.nx - 1) : 0.0;
-    const int rows = std::min(tile_rows(rows_per_thread), g.nz) - 1;
+    const int rows = std::min(tile_rows, g.nz) - 1;
     const int cols = std::min(kTileCols, g.nx) - 1;
     const double rx_slope = 1.0 / std::sqrt(1.0 + 4.0 * g.fnum * g.fnum);
     double spread = 2.0 * kappa * dz * rows + (smax + rx_slope) * kappa * dx * cols;
+    double reach = 0.0;  // widest run of channels
+    for (int i = 0; i + 1 < g.ne; ++i)
+        reach = std::max(reach, g.xe[std::min(i + run, g.ne) - 1] - g.xe[i]);
+    spread += rx_slope * kappa * reach;
     int span = (int)std::ceil(spread) + 1 + 4 + align;
     // Box widths are whole multiples of 128 bytes, so every shared-memory
     // destination of a tensor copy (channel stride wmax, box offsets) stays
@@ -191,16 +206,17 @@ void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
     int nb = (span + maxbox - 1) / maxbox;
     int box = (span + nb - 1) / nb;
     box = (box + box_align - 1) / box_align * box_align;
-    out.box = box;
-    out.wmax = nb * box;
-    out.nsp = (ns + kPadL + 7) / 8 * 8;
-    out.rows = rows_per_thread;
-    out.align = align;
-    int grp = stage_bytes / (out.wmax * pair_bytes(prec) + kTileCols * 12);
+    box_out = box;
+    wmax = nb * box;
+}
+
+int stage_channels(int wmax, int prec, int rows_per_thread, int stage_bytes, int ne)
+{
+    const int grp = stage_bytes / (wmax * pair_bytes(prec) + kTileCols * 12);
     // at most 16 channels per stage on 32- and 64-row tiles (three stages: more
     // leaves one CTA per SM), up to kMaxGroup on 16-row tiles (two stages)
     const int cap = rows_per_thread == 2 ? kMaxGroup : 16;
-    out.group = std::max(1, std::min(cap, std::min(grp, g.ne)));
+    return std::max(1, std::min(cap, std::min(grp, ne)));
 }
 
 void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, int &hi)

@@ -31,7 +31,7 @@ struct PlanHost {
     std::vector<int> colK, rowK;
     std::vector<float> colF, rowF;
     std::vector<int> valid;        // [na][ne][nxp][2] first / last counted row (padding: none)
-    int wmax = 0, box = 0, group = 1, nsp = 0, rows = 8, align = 2;
+    int nsp = 0;
 };
 
 // Envelope transform of a depth: length 2^lg and the spectral factors of
@@ -43,12 +43,14 @@ struct EnvHost {
 
 double grid_coord(double lo, double hi, int n, int j);
 void geometry_tables(const GeomHost &g, GeometryHost &out);
-// rows: rows per thread of the beamforming tile (tile height kWarps * rows);
-// stage_bytes: target bytes of sample windows per pipeline stage (sets the
-// channels per stage)
+// Window of sample pairs a tile of tile_rows rows needs per run of `run` adjacent
+// channels, and the width of the tensor copies it is fetched in.
+void tile_window(const GeomHost &g, const std::vector<double> &angles, int prec, int tile_rows,
+                 int run, int &wmax, int &box);
 void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
-                  const std::vector<double> &angles, int prec, int rows, int stage_bytes,
-                  PlanHost &out);
+                  const std::vector<double> &angles, PlanHost &out);
+// Channels per pipeline stage whose sample windows take stage_bytes.
+int stage_channels(int wmax, int prec, int rows_per_thread, int stage_bytes, int ne);
 void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, int &hi);
 // Plane-wave f-k mapping of every (angle, Kz bin q = 1 .. nt/2, Kx bin m):
 // i0 [na][nt/2][nk] the temporal bin below the mapped position (-1: nothing
