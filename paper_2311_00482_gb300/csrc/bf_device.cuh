@@ -305,10 +305,12 @@ __device__ __forceinline__ f32x2_t mul2(f32x2_t a, f32x2_t b)
 // Rounded delays of rows j and j + 1 for one channel (d2 packed twice): the
 // rx_excess arithmetic of both rows in paired instructions, each half with
 // exactly the scalar version's operations and roundings, plus the pixels'
-// remainders.  m holds the delay plus the rounding constant (integer in its
-// low bits), al the offset in [-1/2, 1/2].
-__device__ __forceinline__ void delay2(f32x2_t D2, f32x2_t Zp, f32x2_t Fp, float &ma, float &mb,
-                                       float &ala, float &alb)
+// remainders.  M: the rounding constant plus the integer parts of the pixels'
+// terms, so m holds the whole delay in its low bits (one addition rounds and adds
+// the integer part; the bits times the pair size plus a channel's entry are a
+// sample pair's address), al the offset in [-1/2, 1/2].
+__device__ __forceinline__ void delay2(f32x2_t D2, f32x2_t Zp, f32x2_t Fp, f32x2_t M, float &ma,
+                                       float &mb, float &ala, float &alb)
 {
     const f32x2_t s = fma2(Zp, Zp, D2);
     float sa, sb;
@@ -317,10 +319,26 @@ __device__ __forceinline__ void delay2(f32x2_t D2, f32x2_t Zp, f32x2_t Fp, float
     float da, db;
     upk2(add2(r, Zp), da, db);
     const f32x2_t x = fma2(D2, pk2(rcp_approx(da), rcp_approx(db)), Fp);
-    const f32x2_t MG = pk2(kRoundMagic, kRoundMagic);
-    const f32x2_t m = add2(x, MG);
+    const f32x2_t m = add2(x, M);
     upk2(m, ma, mb);
-    upk2(sub2(x, sub2(m, MG)), ala, alb);
+    upk2(sub2(x, sub2(m, M)), ala, alb);
+}
+
+// Address of the sample pair at rounded delay m: `step` bytes per pair, ent the
+// channel's entry (the address of index zero).  CHECK: held inside the window
+// [win, win + last], for pixels that do not count the channel.
+template <uint32_t STEP, bool CHECK>
+__device__ __forceinline__ uint32_t pair_at(float m, uint32_t ent, uint32_t win, uint32_t last)
+{
+    const uint32_t p = (uint32_t)__float_as_int(m) * STEP + ent;
+    return CHECK ? win + min(p - win, last) : p;
+}
+
+// Entry of a window that starts at address win with staged pair w0 (ref: the tile's
+// reference integer part, which the pixels' terms are relative to).
+__device__ __forceinline__ uint32_t window_entry(uint32_t win, int w0, int ref, uint32_t step)
+{
+    return win - (uint32_t)(w0 + kRoundBits - ref - kPadL) * step;
 }
 
 }  // namespace

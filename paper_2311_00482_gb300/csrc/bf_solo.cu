@@ -160,13 +160,9 @@ __device__ __forceinline__ void solo_channels(SoloAcc &A, const int4 (&E)[NCH], 
             float m0, m1, l0, l1;
             upk2(m, m0, m1);
             upk2(sub2(x, sub2(m, A.M[k])), l0, l1);
-            uint32_t p0 = (uint32_t)__float_as_int(m0) * PB + (uint32_t)ent[k];
-            uint32_t p1 = (uint32_t)__float_as_int(m1) * PB + (uint32_t)ent[k];
-            if (CHECK) {
-                const uint32_t win = K.win + (uint32_t)k * K.wstep;
-                p0 = win + min(p0 - win, K.last);
-                p1 = win + min(p1 - win, K.last);
-            }
+            const uint32_t win = K.win + (uint32_t)k * K.wstep;
+            const uint32_t p0 = pair_at<PB, CHECK>(m0, (uint32_t)ent[k], win, K.last);
+            const uint32_t p1 = pair_at<PB, CHECK>(m1, (uint32_t)ent[k], win, K.last);
             float v0 = PairIO<PREC>::interp(p0, l0);
             float v1 = PairIO<PREC>::interp(p1, l1);
             if (CHECK) {
@@ -300,8 +296,8 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                 if (lane < amax * runs)
                     for (int q = 0; q < run; ++q)
                         reinterpret_cast<int *>(&sh.ent[st][cq * run + q])[kq] =
-                            (int)(wins + (uint32_t)((kq * G + cq * run + q) * wmax * PB) -
-                                  (uint32_t)(w + kRoundBits - kref - kPadL) * (uint32_t)PB);
+                            (int)window_entry(
+                                wins + (uint32_t)((kq * G + cq * run + q) * wmax * PB), w, kref, PB);
                 if (lane < 2 * kWarps)
                     sh.mask[st][lane] = (uint32_t)m;
                 const bool mine = lane < an * runs && w != kNoWindow;
