@@ -162,9 +162,14 @@ def _nbytes(x):
     return x.nbytes
 
 
+_dp = ctypes.POINTER(ctypes.c_double)
+
+
 def _angles(angles):
-    a = np.ascontiguousarray(np.atleast_1d(np.asarray(angles, dtype=np.float64)))
-    return a, a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+    if not (type(angles) is np.ndarray and angles.dtype == np.float64 and angles.ndim == 1
+            and angles.flags.c_contiguous):
+        angles = np.ascontiguousarray(np.atleast_1d(np.asarray(angles, dtype=np.float64)))
+    return angles, ctypes.cast(angles.ctypes.data, _dp)
 
 
 def bf_create(n_elements, pitch_m, f_number, grid, fs_hz, f0_hz, c_mps, x_elem_m=None):

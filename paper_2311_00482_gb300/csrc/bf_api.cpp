@@ -130,7 +130,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 // Tensor map over a row-major table of `rows` rows of `cols` elements of `elem`
 // bytes (4 or 8), read in boxes of box_cols x box_rows; planes > 0: `planes` such
 // tables back to back, boxes box_planes deep.  Out-of-range elements read as zero.
-static int encode_map(CUtensorMap *map, void *base, int rows, int cols, int elem, int box_cols,
+static int encode_map(CUtensorMap *map, const void *base, int rows, int cols, int elem, int box_cols,
                       int box_rows, int planes = 0, int box_planes = 1)
 {
     auto enc = tensor_map_encoder();
@@ -142,19 +142,13 @@ static int encode_map(CUtensorMap *map, void *base, int rows, int cols, int elem
     cuuint32_t boxd[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(map, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32,
-                     planes > 0 ? 3 : 2, base, dims, strides, boxd, estr,
+                     planes > 0 ? 3 : 2, const_cast<void *>(base), dims, strides, boxd, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(BF_ECUDA, "cuTensorMapEncodeTiled failed (%d): %d x %d of %d bytes, box %d x %d",
                     (int)r, rows, cols, elem, box_cols, box_rows);
     return BF_OK;
-}
-
-static int encode_pairs_map(CUtensorMap *map, void *base, int rows, int nsp, int box, int run, int prec)
-{
-    const int k = pair_elems(prec);  // IQ pairs: two 8-byte elements each
-    return encode_map(map, base, rows, nsp * k, pair_bytes(prec) / k, box * k, run);
 }
 
 // Pairs per frame of one tensor copy of an nf-frame job's interleaved window
@@ -532,27 +526,6 @@ size_t frame_out_bytes(const bf_handle *h, uint32_t flags)
 
 static int plan_frames_per_job(const Plan *p, int modes, int prec, int cap);
 
-// The frame's tensor map of its own pairs, encoded when the layout changed
-// (uploaded by upload_maps).
-static int frame_map(const FramePrep &f, FrameScratch &s, int rows)
-{
-    const Plan *p = f.plan;
-    if (s.map_base == s.pairs.p && s.map_rows == rows && s.map_nsp == p->nsp &&
-        s.map_box == p->box && s.map_run == p->run && s.map_prec == f.prec)
-        return BF_OK;
-    int rc = encode_pairs_map(&s.map_host, s.pairs.p, rows, p->nsp, p->box, p->run, f.prec);
-    if (rc)
-        return rc;
-    s.map_base = s.pairs.p;
-    s.map_rows = rows;
-    s.map_nsp = p->nsp;
-    s.map_box = p->box;
-    s.map_run = p->run;
-    s.map_prec = f.prec;
-    s.map_dirty = true;
-    return BF_OK;
-}
-
 int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *angles, int na,
                   uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int nf_cap,
                   PlanWish wish, bool late_solo)
@@ -579,16 +552,12 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     // room for the frames of a job this frame may lead (interleaved pairs)
     const int cap = plan_frames_per_job(plan, modes, prec, nf_cap);
     rc = s.pairs.ensure((size_t)cap * rows * plan->nsp * pair_bytes(prec));
-    if (!rc && cap > 1)
-        rc = s.map_nf.ensure(sizeof(CUtensorMap));
     if (!rc && stage != BF_OUT_RF && !iq)  // IQ images are magnitudes already
         rc = s.y.ensure(nm * img * sizeof(float));
     if (!rc && stage == BF_OUT_LOGDB)
         rc = s.env.ensure(nm * img * sizeof(float));
     if (!rc)
         rc = s.maxbits.ensure(4 * sizeof(unsigned));
-    if (!rc)
-        rc = s.map.ensure(sizeof(CUtensorMap));
     if (rc)
         return rc;
     fp = FramePrep{};
@@ -612,13 +581,7 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
         fp.env = stage == BF_OUT_ENV ? out_dev : (stage == BF_OUT_LOGDB ? (float *)s.env.p : nullptr);
     }
     fp.maxbits = (unsigned *)s.maxbits.p;
-    fp.map_dev = (CUtensorMap *)s.map.p;
     fp.nf_cap = cap;
-    rc = frame_map(fp, s, rows);
-    if (rc)
-        return rc;
-    fp.map_host = s.map_host;
-    fp.map_dirty = s.map_dirty;
     fp.scratch = &s;
     if (stage != BF_OUT_RF && !iq) {
         const bool warp = envelope_warp_ok(h->g.nz);
@@ -668,29 +631,25 @@ static int max_frames_per_job(const FramePrep &a)
     return plan_frames_per_job(a.plan, a.modes, a.prec, a.nf_cap);
 }
 
-// The lead frame's tensor map of its job's interleaved pairs, encoded when the
-// layout changed (uploaded by upload_maps).
-static int lead_map(const FramePrep &f, int nf, int box)
+// Tensor map over the pairs of a job that frame f leads (nf frames interleaved, box
+// pairs per copy), encoded when the layout changed.
+static int job_map(const FramePrep &f, int nf, int box, CUtensorMap &out)
 {
     FrameScratch &S = *f.scratch;
-    const int rows = f.na * f.h->g.ne, nsp = f.plan->nsp;
-    if (!S.map_nf.p)
-        return fail(BF_EINVAL, "frame scratch has no multi-frame map");
-    if (S.mapnf_base == f.pairs && S.mapnf_rows == rows && S.mapnf_nsp == nsp &&
-        S.mapnf_box == box && S.mapnf_prec == f.prec && S.mapnf_nf == nf)
-        return BF_OK;
-    const int k = pair_elems(f.prec);  // IQ pairs: two 8-byte elements each
-    int rc = encode_map(&S.map_nf_host, f.pairs, rows, nsp * nf * k, pair_bytes(f.prec) / k,
-                        box * nf * k, 1);
-    if (rc)
-        return rc;
-    S.mapnf_base = f.pairs;
-    S.mapnf_rows = rows;
-    S.mapnf_nsp = nsp;
-    S.mapnf_box = box;
-    S.mapnf_prec = f.prec;
-    S.mapnf_nf = nf;
-    S.mapnf_dirty = true;
+    const Plan *p = f.plan;
+    const int rows = f.na * f.h->g.ne, run = nf == 1 ? p->run : 1;
+    const int key[7] = {rows, p->nsp, box, run, f.prec, nf, 1};
+    if (S.map_base != f.pairs || !std::equal(key, key + 7, S.map_key)) {
+        const int k = pair_elems(f.prec);  // IQ pairs: two 8-byte elements each
+        S.map_key[6] = 0;
+        int rc = encode_map(&S.map, f.pairs, rows, p->nsp * nf * k, pair_bytes(f.prec) / k,
+                            box * nf * k, run);
+        if (rc)
+            return rc;
+        S.map_base = f.pairs;
+        std::copy(key, key + 7, S.map_key);
+    }
+    out = S.map;
     return BF_OK;
 }
 
@@ -701,7 +660,7 @@ static bool shareable(const FramePrep &a, const FramePrep &b)
            a.prec == b.prec && a.na == b.na && a.ns == b.ns;
 }
 
-int use_solo_plans(std::vector<FramePrep> &frames)
+void use_solo_plans(std::vector<FramePrep> &frames)
 {
     for (size_t i = 0; i < frames.size(); ++i) {
         FramePrep &f = frames[i];
@@ -710,19 +669,12 @@ int use_solo_plans(std::vector<FramePrep> &frames)
         bool alone = true;
         for (size_t j = 0; j < frames.size() && alone; ++j)
             alone = j == i || !(frames[j].solo == f.solo && shareable(f, frames[j]));
-        if (!alone)
-            continue;
-        f.plan = f.solo;
-        int rc = frame_map(f, *f.scratch, f.na * f.h->g.ne);
-        if (rc)
-            return rc;
-        f.map_host = f.scratch->map_host;
-        f.map_dirty = f.scratch->map_dirty;
+        if (alone)
+            f.plan = f.solo;
     }
-    return BF_OK;
 }
 
-void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
+int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
 {
     hl = HostLaunch{};
     std::map<int, std::vector<BfJob>> groups;
@@ -747,8 +699,14 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         const int avail = (int)cand.size() + 1;
         int nf = avail >= 4 ? 4 : avail >= 2 ? 2 : 1;
         const int box_nf = nf > 1 ? interleaved_box(f.plan->wmax, nf, f.prec) : 0;
-        if (nf > 1 && lead_map(f, nf, box_nf) != BF_OK)
+        CUtensorMap map;
+        if (nf > 1 && job_map(f, nf, box_nf, map) != BF_OK)
             nf = 1;  // no interleaved map: every frame alone
+        if (nf == 1) {
+            int rc = job_map(f, 1, f.plan->box, map);
+            if (rc)
+                return rc;
+        }
         for (int q = 0; q < nf - 1; ++q) {
             more[q] = &frames[cand[q]];
             taken[cand[q]] = 1;
@@ -766,7 +724,8 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         j.wtab = (const int *)p->wtab.p;
         j.btab = (const int *)p->btab.p;
         j.apcnt = (const uint16_t *)h->apcnt.p;
-        j.rf_map = f.map_dev;
+        j.rf_map = (const CUtensorMap *)hl.maps.size();
+        hl.maps.push_back(map);
         j.valid_map = (const CUtensorMap *)p->maps.p;
         j.dx2_map = (const CUtensorMap *)p->maps.p + 1;
         j.y = f.y;
@@ -799,10 +758,8 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
                                     ? more[q]->maxbits
                                     : nullptr;
         }
-        if (nf > 1) {  // the frames' pairs interleaved in the lead's scratch
-            j.rf_map = (const CUtensorMap *)f.scratch->map_nf.p;
+        if (nf > 1)  // the frames' pairs interleaved in the lead's scratch
             j.box = box_nf;
-        }
         const int combiners = j.modes & (BF_DMAS | BF_CF | BF_PDAS);
         const int variant =
             (((p->split * 8 + nf) * 16 + p->rows) * 4 + f.prec) * 16 + combiners;
@@ -984,74 +941,73 @@ void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         }
     }
     hl.log_blocks = (int)blks;
+    return BF_OK;
 }
 
 int DeviceLaunch::upload(const HostLaunch &hl, cudaStream_t st, bool async)
 {
-    auto put = [&](DevMem &d, const void *src, size_t n) -> int {
-        if (n == 0)
-            return BF_OK;
-        int rc = d.reserve(n);
-        if (rc)
-            return rc;
-        cudaError_t e = async ? cudaMemcpyAsync(d.p, src, n, cudaMemcpyHostToDevice, st)
-                              : cudaMemcpy(d.p, src, n, cudaMemcpyHostToDevice);
-        return e == cudaSuccess ? BF_OK : cuda_fail(e, "cudaMemcpy (job list)");
+    size_t total = 0;
+    auto room = [&](size_t n) {  // tensor maps want 64-byte alignment
+        const size_t at = total;
+        total += (n + 127) & ~(size_t)127;
+        return at;
     };
-    int rc = put(jobs, hl.jobs.data(), hl.jobs.size() * sizeof(BfJob));
-    if (!rc) rc = put(tile_prefix, hl.tile_prefix.data(), hl.tile_prefix.size() * sizeof(int));
-    if (!rc) rc = put(ingest, hl.ingest.data(), hl.ingest.size() * sizeof(IngestJob));
-    if (!rc) rc = put(ingest_prefix, hl.ingest_prefix.data(), hl.ingest_prefix.size() * sizeof(int));
-    for (int b = 0; b < 2; ++b) {
-        if (!rc) rc = put(env[b], hl.env[b].data(), hl.env[b].size() * sizeof(EnvJob));
-        if (!rc) rc = put(env_prefix[b], hl.env_prefix[b].data(), hl.env_prefix[b].size() * sizeof(int));
-    }
-    if (!rc) rc = put(envw, hl.envw.data(), hl.envw.size() * sizeof(EnvJob));
-    if (!rc) rc = put(envw_prefix, hl.envw_prefix.data(), hl.envw_prefix.size() * sizeof(int));
-    if (!rc) rc = put(log, hl.log.data(), hl.log.size() * sizeof(LogJob));
-    if (!rc) rc = put(blk_prefix, hl.blk_prefix.data(), hl.blk_prefix.size() * sizeof(int));
-    if (!rc) rc = put(demod, hl.demod.data(), hl.demod.size() * sizeof(DemodJob));
-    if (!rc) rc = put(demod_prefix, hl.demod_prefix.data(), hl.demod_prefix.size() * sizeof(int));
-    if (!rc) rc = err.ensure(sizeof(int));
-    return rc;
-}
-
-// Tensor maps of frames whose scratch changed go to device memory (before any
-// kernel reads them).
-int upload_maps(std::vector<FramePrep> &frames, cudaStream_t st, bool async)
-{
-    auto copy = [&](void *dst, const CUtensorMap *src) -> int {
-        cudaError_t e = async ? cudaMemcpyAsync(dst, src, sizeof(CUtensorMap),
-                                                cudaMemcpyHostToDevice, st)
-                              : cudaMemcpy(dst, src, sizeof(CUtensorMap), cudaMemcpyHostToDevice);
-        return e == cudaSuccess ? BF_OK : cuda_fail(e, "cudaMemcpy (tensor map)");
+    std::vector<std::pair<const void *, std::pair<size_t, size_t>>> parts;  // source, (offset, bytes)
+    auto add = [&](const auto &v) {
+        const size_t n = v.size() * sizeof(v[0]), at = room(n);
+        parts.push_back({v.data(), {at, n}});
+        return at;
     };
-    for (FramePrep &f : frames) {
-        FrameScratch &S = *f.scratch;
-        if (f.map_dirty) {
-            int rc = copy(f.map_dev, &S.map_host);
-            if (rc)
-                return rc;
-            S.map_dirty = false;
-            f.map_dirty = false;
-        }
-        if (S.mapnf_dirty) {  // the frame leads a multi-frame job
-            int rc = copy(S.map_nf.p, &S.map_nf_host);
-            if (rc)
-                return rc;
-            S.mapnf_dirty = false;
-        }
+    const size_t a_maps = add(hl.maps), a_jobs = add(hl.jobs), a_tp = add(hl.tile_prefix),
+                 a_in = add(hl.ingest), a_ip = add(hl.ingest_prefix), a_e0 = add(hl.env[0]),
+                 a_ep0 = add(hl.env_prefix[0]), a_e1 = add(hl.env[1]), a_ep1 = add(hl.env_prefix[1]),
+                 a_ew = add(hl.envw), a_ewp = add(hl.envw_prefix), a_log = add(hl.log),
+                 a_bp = add(hl.blk_prefix), a_dm = add(hl.demod), a_dp = add(hl.demod_prefix);
+    int rc = pack.reserve(std::max<size_t>(total, 128));
+    if (!rc)
+        rc = err.ensure(sizeof(int));
+    if (rc)
+        return rc;
+    char *d = (char *)pack.p;
+    std::vector<char> host(total);
+    for (const auto &q : parts)
+        if (q.second.second)
+            std::memcpy(host.data() + q.second.first, q.first, q.second.second);
+    for (size_t k = 0; k < hl.jobs.size(); ++k) {  // map indices to addresses
+        BfJob j = hl.jobs[k];
+        j.rf_map = (const CUtensorMap *)(d + a_maps) + (size_t)j.rf_map;
+        std::memcpy(host.data() + a_jobs + k * sizeof(BfJob), &j, sizeof j);
     }
+    if (total) {
+        cudaError_t e = async ? cudaMemcpyAsync(d, host.data(), total, cudaMemcpyHostToDevice, st)
+                              : cudaMemcpy(d, host.data(), total, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess)
+            return cuda_fail(e, "cudaMemcpy (job lists)");
+    }
+    jobs = (const BfJob *)(d + a_jobs);
+    tile_prefix = (const int *)(d + a_tp);
+    ingest = (const IngestJob *)(d + a_in);
+    ingest_prefix = (const int *)(d + a_ip);
+    env[0] = (const EnvJob *)(d + a_e0);
+    env[1] = (const EnvJob *)(d + a_e1);
+    env_prefix[0] = (const int *)(d + a_ep0);
+    env_prefix[1] = (const int *)(d + a_ep1);
+    envw = (const EnvJob *)(d + a_ew);
+    envw_prefix = (const int *)(d + a_ewp);
+    log = (const LogJob *)(d + a_log);
+    blk_prefix = (const int *)(d + a_bp);
+    demod = (const DemodJob *)(d + a_dm);
+    demod_prefix = (const int *)(d + a_dp);
     return BF_OK;
 }
 
 // The envelope launches of a set of frames: 512-row images, then the others.
 static cudaError_t launch_envelopes(const HostLaunch &hl, DeviceLaunch &dl, cudaStream_t st)
 {
-    cudaError_t e = launch_envelope_warp((const EnvJob *)dl.envw.p, (const int *)dl.envw_prefix.p,
+    cudaError_t e = launch_envelope_warp(dl.envw, dl.envw_prefix,
                                          (int)hl.envw.size(), hl.envw_pairs, st);
     for (int b = 1; b >= 0 && e == cudaSuccess; --b)
-        e = launch_envelope((const EnvJob *)dl.env[b].p, (const int *)dl.env_prefix[b].p,
+        e = launch_envelope(dl.env[b], dl.env_prefix[b],
                             (int)hl.env[b].size(), hl.env_blocks[b], b == 1, st);
     return e;
 }
@@ -1095,14 +1051,14 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
     for (const HostLaunch::IGroup &g : hl.igroups) {
-        e = launch_ingest((const IngestJob *)dl.ingest.p + g.first,
-                          (const int *)dl.ingest_prefix.p + g.prefix_first, g.count, g.rows, g.prec,
+        e = launch_ingest(dl.ingest + g.first,
+                          dl.ingest_prefix + g.prefix_first, g.count, g.rows, g.prec,
                           st);
         if (e != cudaSuccess)
             return cuda_fail(e, "ingest launch");
     }
     if (!hl.demod.empty()) {
-        e = launch_demod((const DemodJob *)dl.demod.p, (const int *)dl.demod_prefix.p,
+        e = launch_demod(dl.demod, dl.demod_prefix,
                          (int)hl.demod.size(), hl.demod_rows, hl.demod_max_ns, hl.demod_pairs, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "demodulation launch");
@@ -1112,8 +1068,8 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
     for (const HostLaunch::Group &g : hl.groups) {
-        const BfJob *jobs = (const BfJob *)dl.jobs.p + g.first;
-        const int *prefix = (const int *)dl.tile_prefix.p + g.prefix_first;
+        const BfJob *jobs = dl.jobs + g.first;
+        const int *prefix = dl.tile_prefix + g.prefix_first;
         e = g.split ? launch_solo(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant, g.split,
                                   (int *)dl.err.p, st)
                     : launch_beamform(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant,
@@ -1128,7 +1084,7 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     if (e != cudaSuccess)
         return cuda_fail(e, "envelope launch");
     if (!hl.log.empty()) {
-        e = launch_log((const LogJob *)dl.log.p, (const int *)dl.blk_prefix.p, (int)hl.log.size(),
+        e = launch_log(dl.log, dl.blk_prefix, (int)hl.log.size(),
                        hl.log_blocks, 70.0f, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "log launch");
@@ -1301,18 +1257,12 @@ BF_API int bf_beamform(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         return fail(BF_EINVAL, "null data pointer");
     cudaSetDevice(h->device);
     CallCache &cc = h->call;
-    if (cc.valid) {  // the same call as last time: no preparation, no uploads
-        int rc = check_frame_args(h, n_samples, angles_rad, n_angles, flags);
-        if (rc)
-            return rc;
-        Plan *plan = nullptr;
-        rc = handle_plan(h, n_samples, angles_rad, n_angles, flags, &plan,
-                         PlanWish{-1, 1, true});
-        if (rc)
-            return rc;
-        if (plan == cc.plan && flags == cc.flags && rf_dev == cc.rf && out_dev == cc.out &&
-            n_samples == cc.ns && n_angles == cc.na && h->pdas_p == cc.pdas_p &&
-            h->stream == cc.stream) {
+    if (cc.valid) {  // the same call as last time: no checks, no preparation, no uploads
+        if (flags == cc.flags && rf_dev == cc.rf && out_dev == cc.out && n_samples == cc.ns &&
+            n_angles == (int)cc.angles.size() && angles_rad && h->pdas_p == cc.pdas_p &&
+            h->stream == cc.stream && forced_cfg() == cc.forced &&
+            std::equal(cc.angles.begin(), cc.angles.end(), angles_rad)) {
+            int rc = BF_OK;
             if (!cc.exec && ++cc.hits >= 1) {  // a repeat: capture the launches once
                 cudaStream_t cap;
                 cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
@@ -1352,8 +1302,7 @@ BF_API int bf_beamform(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     if (rc)
         return rc;
     HostLaunch hl;
-    build_launch(frames, hl);
-    rc = upload_maps(frames, h->stream, true);
+    rc = build_launch(frames, hl);
     if (!rc)
         rc = h->launch.upload(hl, h->stream, true);
     if (!rc && !h->err_cleared) {
@@ -1364,12 +1313,12 @@ BF_API int bf_beamform(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         rc = enqueue(frames, hl, h->launch, h->stream);
     if (!rc) {
         cc.valid = true;
-        cc.plan = frames[0].plan;
+        cc.forced = forced_cfg();
         cc.flags = flags;
         cc.rf = rf_dev;
         cc.out = out_dev;
         cc.ns = n_samples;
-        cc.na = n_angles;
+        cc.angles.assign(angles_rad, angles_rad + n_angles);
         cc.pdas_p = h->pdas_p;
         cc.stream = h->stream;
         cc.frames = frames;
@@ -1543,7 +1492,9 @@ BF_API int bf_beamform_plain(bf_handle *h, const int16_t *rf_dev, int32_t n_samp
     if (rc)
         return rc;
     HostLaunch hl;
-    build_launch(frames, hl);
+    rc = build_launch(frames, hl);
+    if (rc)
+        return rc;
     const BfJob &job = hl.jobs[0];
     cudaError_t e = launch_plain(job, rf_dev, (const short2 *)frames[0].plan->at->valid.p,
                                  (const float *)h->dx2.p, pad_cols(h->g.nx), n_samples, h->stream);
@@ -1570,7 +1521,7 @@ BF_API int bf_beamform_plain(bf_handle *h, const int16_t *rf_dev, int32_t n_samp
             rc = cuda_fail(e, "envelope launch");
     }
     if (!rc && !hl.log.empty()) {
-        e = launch_log((const LogJob *)h->launch.log.p, (const int *)h->launch.blk_prefix.p,
+        e = launch_log(h->launch.log, h->launch.blk_prefix,
                        (int)hl.log.size(), hl.log_blocks, 70.0f, h->stream);
         if (e != cudaSuccess)
             rc = cuda_fail(e, "log launch");
@@ -1711,9 +1662,8 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
         if (prc)
             continue;  // this configuration does not fit the workload
         HostLaunch hl;
-        build_launch(fr, hl);
         DeviceLaunch dl;
-        rc = upload_maps(fr, st, false);
+        rc = build_launch(fr, hl);
         if (!rc)
             rc = dl.upload(hl, st, false);
         if (!rc && cudaMemsetAsync(dl.err.p, 0, sizeof(int), st) != cudaSuccess)
@@ -1753,6 +1703,7 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
                     std::vector<double>(angles_rad, angles_rad + n_angles), 0};
         h->tuned[key] = best;
     }
+    h->call.clear();  // bf_beamform's last call may have used another configuration
     if (rows_out)
         *rows_out = kTileConfigs[best].rows;
     if (stage_bytes_out)
@@ -1804,8 +1755,7 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
             return fail(rc, "frame %d: %s", i, g_err.c_str());
     }
     b->device = dev;
-    build_launch(b->frames, b->hl);
-    int rc = upload_maps(b->frames, nullptr, false);
+    int rc = build_launch(b->frames, b->hl);
     if (!rc)
         rc = b->dl.upload(b->hl, nullptr, false);
     if (rc)

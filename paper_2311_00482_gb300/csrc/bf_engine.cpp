@@ -196,7 +196,7 @@ struct Slot {
     size_t device_bytes() const
     {
         return rf.bytes + out.bytes + scratch.pairs.bytes + scratch.y.bytes + scratch.env.bytes +
-               scratch.maxbits.bytes + scratch.map.bytes;
+               scratch.maxbits.bytes;
     }
 };
 
@@ -682,13 +682,9 @@ void Engine::launch(std::vector<std::shared_ptr<Request>> &reqs)
         f.out = to;
     }
     HostLaunch hl;
+    use_solo_plans(frames);
     if (!rc)
-        rc = use_solo_plans(frames);
-    build_launch(frames, hl);
-    if (!rc)
-        rc = upload_maps(frames, st, true);
-    for (size_t i = 0; i < reqs.size(); ++i)
-        reqs[i]->fp.map_dirty = false;
+        rc = build_launch(frames, hl);
     if (!rc)
         rc = R.dl.upload(hl, st, true);
     if (!rc && cudaMemsetAsync(R.dl.err.p, 0, sizeof(int), st) != cudaSuccess)

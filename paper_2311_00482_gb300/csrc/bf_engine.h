@@ -107,20 +107,15 @@ struct EnvTablesDev {
 };
 
 // Device scratch of one in-flight frame: staged sample pairs, beamformed
-// image, envelope, frame maxima and the tensor map over the pairs.
+// image, envelope and frame maxima.
 struct FrameScratch {
-    DevMem pairs, y, env, maxbits, map;
-    CUtensorMap map_host{};
-    void *map_base = nullptr;
-    int map_rows = 0, map_nsp = 0, map_box = 0, map_run = 0, map_prec = -1;
-    bool map_dirty = false;
     // as the lead of a multi-frame job: pairs holds the job's frames interleaved
-    // ([row][pair][frame]) and map_nf describes that layout
-    DevMem map_nf;
-    CUtensorMap map_nf_host{};
-    void *mapnf_base = nullptr;
-    int mapnf_rows = 0, mapnf_nsp = 0, mapnf_box = 0, mapnf_prec = -1, mapnf_nf = 0;
-    bool mapnf_dirty = false;
+    // ([row][pair][frame])
+    DevMem pairs, y, env, maxbits;
+    // the tensor map over the pairs encoded last, and what it was encoded for
+    CUtensorMap map{};
+    const void *map_base = nullptr;
+    int map_key[7] = {};  // rows, nsp, box, run, prec, frames, set
 };
 
 struct FramePrep {
@@ -137,9 +132,6 @@ struct FramePrep {
     void *pairs = nullptr;
     float *y = nullptr, *env = nullptr;
     unsigned *maxbits = nullptr;
-    CUtensorMap *map_dev = nullptr;
-    CUtensorMap map_host{};
-    bool map_dirty = false;
     FrameScratch *scratch = nullptr;
     int nf_cap = 1;  // frames of a job this frame may lead (its pairs buffer holds that many)
 };
@@ -152,7 +144,8 @@ struct HostLaunch {
     struct IGroup {  // one ingest launch
         int prec, first, count, prefix_first, rows;  // rows: the launch's CTAs
     };
-    std::vector<BfJob> jobs;
+    std::vector<BfJob> jobs;        // rf_map: index into maps until the upload
+    std::vector<CUtensorMap> maps;  // over the jobs' sample pairs
     std::vector<int> tile_prefix;
     std::vector<Group> groups;
     size_t smem = 0;
@@ -176,25 +169,33 @@ struct HostLaunch {
     bool demod_pairs = false;  // some demodulation job covers a frame pair
 };
 
+// Device copy of a launch description: every list in one allocation, sent in one
+// transfer (each transfer costs the stream a few microseconds before its kernels).
 struct DeviceLaunch {
-    DevMem jobs, tile_prefix, ingest, ingest_prefix, env[2], env_prefix[2], log, blk_prefix, err;
-    DevMem envw, envw_prefix;
-    DevMem demod, demod_prefix;
+    DevMem pack, err;
+    const BfJob *jobs = nullptr;
+    const IngestJob *ingest = nullptr;
+    const EnvJob *env[2] = {nullptr, nullptr}, *envw = nullptr;
+    const LogJob *log = nullptr;
+    const DemodJob *demod = nullptr;
+    const int *tile_prefix = nullptr, *ingest_prefix = nullptr, *env_prefix[2] = {nullptr, nullptr},
+              *envw_prefix = nullptr, *blk_prefix = nullptr, *demod_prefix = nullptr;
     int upload(const HostLaunch &hl, cudaStream_t st, bool async);
 };
 
 struct Request;
 
 // The last bf_beamform call of a handle, kept so that the same call again
-// (same plan, flags, buffers, order p and stream) skips the host-side
+// (same arguments, order p, stream and BF_TILE_ROWS) skips the host-side
 // preparation and, from its second repetition on, replays one CUDA graph.
 struct CallCache {
     bool valid = false;
-    const Plan *plan = nullptr;
+    int forced = -1;  // BF_TILE_ROWS's configuration
     uint32_t flags = 0;
     const int16_t *rf = nullptr;
     float *out = nullptr;
-    int ns = 0, na = 0;
+    int ns = 0;
+    std::vector<double> angles;
     double pdas_p = 0;
     cudaStream_t stream = nullptr;
     int hits = 0;
@@ -282,13 +283,12 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
                   uint32_t flags, float *out_dev, FrameScratch &s, FramePrep &fp, int nf_cap = 1,
                   PlanWish wish = {}, bool late_solo = false);
 // Frames of a launch that share no job with another one go over to their solo plans.
-int use_solo_plans(std::vector<FramePrep> &frames);
+void use_solo_plans(std::vector<FramePrep> &frames);
 // Frames (at most cap) of one plan that can share a beamforming job with a
 // frame of these flags (1 unless the combiners are DAS / DMAS of RF records
 // or IQ-DAS / BB-DMAS; IQ frames with records above 4096 samples alone).
 int job_frames_cap(const Plan *p, uint32_t flags, int cap);
-void build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl);
-int upload_maps(std::vector<FramePrep> &frames, cudaStream_t st, bool async);
+int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl);
 // Stage marks of a captured graph on a side branch: mark k is recorded on the
 // side stream after it joins the capture behind stage k (fork[k] recorded on
 // the capture stream), so each mark node depends on the work it closes and no
