@@ -230,9 +230,36 @@ static __device__ __forceinline__ void sts2(uint32_t a, float2 v)
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
-// buf: the transform's exchange buffer; tab: the twiddle table; bar: a named
-// barrier (1 .. 15) of the transform's T threads, used where T > 32.
+// Shared-memory twiddles of one length: level L's entries start here, after those of
+// the levels above it; fft16_tab_shared(lg, below the last level) is their number.
+__host__ __device__ constexpr int fft16_tab_shared(int lg, int L)
+{
+    int n = 0;
+    for (int l = lg; l > L && l > 4; l -= 4)
+        n += 6 << (l - 4);
+    return n;
+}
+
+// Fill them (all threads of the CTA; a barrier must follow).
 template <int LG>
+static __device__ __forceinline__ void fft16_fill_shared(float2 *tab)
+{
+#pragma unroll
+    for (int l = LG; l > 4; l -= 4) {
+        const int S = 1 << (l - 4);
+        for (int t = threadIdx.x; t < 6 * S; t += blockDim.x) {
+            const int i = t / S, e = i < 4 ? i + 1 : 4 * (i - 2);  // exponents 1, 2, 3, 4, 8, 12
+            float sn, cs;
+            sincospif(-2.0f * (float)((t - i * S) * e) / (float)(1 << l), &sn, &cs);
+            tab[fft16_tab_shared(LG, l) + t] = make_float2(cs, sn);
+        }
+    }
+}
+
+// buf: the transform's exchange buffer; tab: the twiddle table (fft16_tw_at's layout;
+// TAB_SHARED: in shared memory, the levels of this length only, fft16_tab_shared);
+// bar: a named barrier (1 .. 15) of the transform's T threads, used where T > 32.
+template <int LG, bool TAB_SHARED = false>
 struct Fft16 {
     static constexpr int M = 1 << LG, T = M / 16;
     static constexpr int kLast = (LG - 1) % 4 + 1;  // log2 length of the last level
@@ -286,14 +313,24 @@ struct Fft16 {
     __device__ __forceinline__ void twiddle(float2 (&v)[16]) const
     {
         constexpr int S = 1 << (L - 4);
-        const float2 *__restrict__ t = tab + fft16_tw_at(L) + (u & (S - 1));
         float2 w[16];
-        w[1] = __ldg(t);
-        w[2] = __ldg(t + S);
-        w[3] = __ldg(t + 2 * S);
-        w[4] = __ldg(t + 3 * S);
-        w[8] = __ldg(t + 4 * S);
-        w[12] = __ldg(t + 5 * S);
+        if constexpr (TAB_SHARED) {
+            const uint32_t t = smem_addr(tab) + 8u * (uint32_t)(fft16_tab_shared(LG, L) + (u & (S - 1)));
+            w[1] = lds2(t);
+            w[2] = lds2(t + 8u * S);
+            w[3] = lds2(t + 16u * S);
+            w[4] = lds2(t + 24u * S);
+            w[8] = lds2(t + 32u * S);
+            w[12] = lds2(t + 40u * S);
+        } else {
+            const float2 *__restrict__ t = tab + fft16_tw_at(L) + (u & (S - 1));
+            w[1] = __ldg(t);
+            w[2] = __ldg(t + S);
+            w[3] = __ldg(t + 2 * S);
+            w[4] = __ldg(t + 3 * S);
+            w[8] = __ldg(t + 4 * S);
+            w[12] = __ldg(t + 5 * S);
+        }
         if (INV) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) {

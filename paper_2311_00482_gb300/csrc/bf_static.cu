@@ -7,7 +7,7 @@
 // the allocator must not be entered at all.  bf_logdb_static serves them: it
 // takes a beamformed image the caller already holds on the device and writes
 // its -70 dB log-compressed envelope into the caller's output, and its only
-// scratch (the envelope image and the frame maximum) is a fixed array compiled
+// scratch (the envelope image and its maxima) is a fixed array compiled
 // into this library.  Every GPU that loads the library holds that array
 // (kStaticPixels floats, 4 MiB) until the process exits.
 //
@@ -20,6 +20,7 @@
 
 #include "../../include/bf.h"
 #include "bf_engine.h"
+#include "bf_envelope_pairs.cuh"
 #include "bf_fft.cuh"
 #include "bf_internal.h"
 
@@ -29,16 +30,58 @@ namespace {
 constexpr size_t kStaticPixels = (size_t)1 << 20;  // largest nx * nz accepted
 constexpr int kMaxDevices = 64;
 
-// [0, kStaticPixels): envelope image; [kStaticPixels]: frame maximum (float bits).
-__device__ __align__(256) float g_static_scratch[kStaticPixels + 64];
+// [0, kStaticPixels): envelope image; from kStaticPixels: the envelope CTAs' maxima.
+constexpr int kStaticMaxima = 512;
+__device__ __align__(256) float g_static_scratch[kStaticPixels + kStaticMaxima];
+
+// The CTA's largest value into its slot of the maxima.
+__device__ __forceinline__ void block_max(float v, float *__restrict__ slot)
+{
+    __shared__ float red[32];
+#pragma unroll
+    for (int off = 16; off; off >>= 1)
+        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
+#pragma unroll
+        for (int off = 16; off; off >>= 1)
+            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+        if (threadIdx.x == 0)
+            *slot = v;
+    }
+}
+
+// Depths of 32 rows and more: the envelope kernel's transforms, with twiddles and
+// masks computed here.  512 x 512 with the band-pass: 17.5 us as radix-4 passes over
+// shared memory by 64 CTAs of eight columns; a CTA now holds T-thread transforms of
+// 4096 points in all.
+template <int LG>
+__global__ void __launch_bounds__(256, 2)
+    static_envelope16_kernel(const float *__restrict__ y, int nx, int band, int kb_lo, int kb_hi,
+                             float *__restrict__ env, float *__restrict__ maxima)
+{
+    extern __shared__ __align__(16) float2 sbuf[];
+    asm volatile("griddepcontrol.launch_dependents;");
+    float2 *tab = sbuf + 256 * (17 + 16);
+    fft16_fill_shared<LG>(tab);
+    __syncthreads();
+    const uint32_t bufs = smem_addr(sbuf);
+    const float v = envelope_pairs<LG, false, 256, true>(
+        y, env, nx, 1 << LG, blockIdx.x * envelope_pairs_per_block(LG), band != 0, tab,
+        MaskFactors<LG>{kb_lo, kb_hi, band != 0}, bufs, bufs + 256 * 17 * 8);
+    block_max(v, maxima + blockIdx.x);
+}
 
 __global__ void __launch_bounds__(256) static_envelope_kernel(const float *__restrict__ y, int nx,
                                                               int nz, int band, int kb_lo,
                                                               int kb_hi, float *__restrict__ env,
-                                                              unsigned *__restrict__ maxbits)
+                                                              float *__restrict__ maxima)
 {
+    asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(16) float2 sbuf[];
-    __shared__ float red[32];
     const int m = nz, lgm = 31 - __clz(m);
     const int C = m >= 2048 ? 1 : 2048 / m;  // complex columns: pairs of image columns
     const int c0 = blockIdx.x * 2 * C;
@@ -88,35 +131,63 @@ __global__ void __launch_bounds__(256) static_envelope_kernel(const float *__res
             lmax = fmaxf(lmax, e);
         }
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1)
-        lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
-    if ((threadIdx.x & 31) == 0)
-        red[threadIdx.x >> 5] = lmax;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-#pragma unroll
-        for (int off = 16; off; off >>= 1)
-            v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-        if (threadIdx.x == 0)
-            atomicMax(maxbits, __float_as_uint(v));
-    }
+    block_max(lmax, maxima + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict__ env, size_t n,
-                                                         const unsigned *__restrict__ maxbits,
+// Sixteen pixels per thread; the image's maximum from the envelope CTAs' maxima.
+constexpr int kStaticLogPixels = 4096;
+__global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict__ env, int n, int vec4,
+                                                         const float *__restrict__ maxima, int nmax,
                                                          float *__restrict__ out, float dr)
 {
-    const float peak = __uint_as_float(*maxbits);
-    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-         p += (size_t)gridDim.x * blockDim.x) {
-        const float e = env[p];
-        float d = -dr;
-        if (e > 0.f && peak > 0.f)
-            d = fminf(fmaxf(20.f * log10f(e / peak), -dr), 0.f);
-        out[p] = d;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the envelope kernel has completed
+    __shared__ float red[8];
+    float peak = 0.f;
+    for (int k = threadIdx.x; k < nmax; k += blockDim.x)
+        peak = fmaxf(peak, __ldcg(maxima + k));
+    peak = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(peak)));  // >= 0
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = peak;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w)
+        peak = fmaxf(peak, red[w]);
+    // 20 log10(e / peak) = (20 log10 2) (log2 e - log2 peak), as log_kernel
+    const float lp = peak > 0.f ? __log2f(peak) : 0.f;
+    auto db = [&](float e) {
+        return (e > 0.f && peak > 0.f) ? fminf(fmaxf(6.0205999132796239f * (__log2f(e) - lp), -dr), 0.f)
+                                       : -dr;
+    };
+    const int base = blockIdx.x * kStaticLogPixels;
+    if (vec4) {
+#pragma unroll
+        for (int u = 0; u < kStaticLogPixels / 1024; ++u) {
+            const int p = base + 4 * (threadIdx.x + 256 * u);
+            if (p < n) {
+                const float4 e = __ldcg(reinterpret_cast<const float4 *>(env + p));
+                *reinterpret_cast<float4 *>(out + p) = make_float4(db(e.x), db(e.y), db(e.z), db(e.w));
+            }
+        }
+        return;
     }
+    for (int p = base + threadIdx.x; p < min(base + kStaticLogPixels, n); p += 256)
+        out[p] = db(__ldcg(env + p));
+}
+
+template <int LG>
+cudaError_t launch_static16(const float *y, int nx, int band, int lo, int hi, float *env,
+                            float *maxima, int *blocks, cudaStream_t st)
+{
+    const size_t smem = (256 * (17 + 16) + fft16_tab_shared(LG, 4)) * sizeof(float2);
+    int sms = 0;
+    cudaError_t e = kernel_setup((const void *)static_envelope16_kernel<LG>, smem, 256, true, &sms,
+                                 nullptr);
+    if (e != cudaSuccess)
+        return e;
+    const int per = 2 * envelope_pairs_per_block(LG);
+    *blocks = (nx + per - 1) / per;
+    static_envelope16_kernel<LG><<<*blocks, 256, smem, st>>>(y, nx, band, lo, hi, env, maxima);
+    return cudaGetLastError();
 }
 
 std::mutex g_static_mu;
@@ -238,26 +309,48 @@ extern "C" BF_API int bf_logdb_static(const float *y_dev, int32_t nx, int32_t nz
     int kb_lo = 1, kb_hi = 0;
     bandpass_bins(nz, z0_m, z1_m, c_mps, f0_hz, kb_lo, kb_hi);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    float *env = scratch;
-    unsigned *maxbits = reinterpret_cast<unsigned *>(scratch + kStaticPixels);
-    cudaError_t e = cudaMemsetAsync(maxbits, 0, sizeof(unsigned), st);  // the maximum starts at 0
-    if (e != cudaSuccess)
-        return cuda_fail(e, "cudaMemsetAsync (static scratch)");
-    const int C = nz >= 2048 ? 1 : 2048 / nz;
-    const size_t smem = (3u * (size_t)C * nz + (size_t)nz) * sizeof(float2);
-    int sms = 0;
-    e = kernel_setup((const void *)static_envelope_kernel, smem, 256, false, &sms, nullptr);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "cudaFuncSetAttribute");
-    const int blocks = (nx + 2 * C - 1) / (2 * C);
-    static_envelope_kernel<<<blocks, 256, smem, st>>>(y_dev, nx, nz, bandpass ? 1 : 0, kb_lo, kb_hi,
-                                                      env, maxbits);
-    e = cudaGetLastError();
+    float *env = scratch, *maxima = scratch + kStaticPixels;
+    const int band = bandpass ? 1 : 0;
+    int lg = 0, blocks = 0;
+    while ((1 << lg) < nz)
+        ++lg;
+    cudaError_t e = cudaSuccess;
+    switch (lg) {
+    case 5: e = launch_static16<5>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 6: e = launch_static16<6>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 7: e = launch_static16<7>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 8: e = launch_static16<8>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 9: e = launch_static16<9>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 10: e = launch_static16<10>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 11: e = launch_static16<11>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    case 12: e = launch_static16<12>(y_dev, nx, band, kb_lo, kb_hi, env, maxima, &blocks, st); break;
+    default: {  // fewer than 32 rows
+        const int C = 2048 / nz;
+        const size_t smem = (3u * (size_t)C * nz + (size_t)nz) * sizeof(float2);
+        int sms = 0;
+        e = kernel_setup((const void *)static_envelope_kernel, smem, 256, false, &sms, nullptr);
+        if (e != cudaSuccess)
+            return cuda_fail(e, "cudaFuncSetAttribute");
+        blocks = (nx + 2 * C - 1) / (2 * C);
+        static_envelope_kernel<<<blocks, 256, smem, st>>>(y_dev, nx, nz, band, kb_lo, kb_hi, env,
+                                                          maxima);
+        e = cudaGetLastError();
+    }
+    }
     if (e != cudaSuccess)
         return cuda_fail(e, "envelope launch");
-    const size_t n = (size_t)nx * nz;
-    const int lb = (int)std::min<size_t>((n + 255) / 256, 4096);
-    static_log_kernel<<<lb, 256, 0, st>>>(env, n, maxbits, db_dev, 70.0f);
-    e = cudaGetLastError();
+    const int n = nx * nz;
+    const int vec4 = n % 4 == 0 && (reinterpret_cast<uintptr_t>(db_dev) & 15) == 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + kStaticLogPixels - 1) / kStaticLogPixels));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];  // scheduled while the envelope kernel's last CTAs run
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, static_log_kernel, (const float *)env, n, vec4, (const float *)maxima,
+                           blocks, db_dev, 70.0f);
     return e == cudaSuccess ? BF_OK : cuda_fail(e, "log launch");
 }
