@@ -594,7 +594,7 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
             return rc;
     }
     if (iq) {
-        rc = fft_tables(ns, fp.dt);  // twiddles of the length-ns transforms
+        rc = fft_tables(ns < 32 ? ns : 0, fp.dt);
         if (rc)
             return rc;
     }
@@ -611,8 +611,8 @@ static int plan_frames_per_job(const Plan *p, int modes, int prec, int cap)
     const int m = modes & (BF_MODE_MASK | BF_IQ_MASK);
     if (p->split || !sharing_modes((uint32_t)m))
         return 1;
-    if (prec == kPrecIQ && demod_smem_bytes(p->ns, true) > (size_t)kMaxSmemPerCta)
-        return 1;  // a frame pair's demodulation does not fit one CTA
+    if (prec == kPrecIQ && p->ns > 4096)
+        return 1;  // long records: every frame alone
     for (int nf = p->rows == 2 ? 4 : p->rows == 4 ? 2 : 1; nf > 1; nf /= 2)
         if (nf <= cap &&
             beamform_smem_bytes(p->wmax, p->group, prec, nf, p->rows) <= (size_t)kMaxSmemPerCta &&
@@ -815,18 +815,19 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
             while ((1 << d.lgn) < f.ns)
                 ++d.lgn;
             d.rot = make_float2((float)std::cos(2.0 * kPi * r), (float)-std::sin(2.0 * kPi * r));
-            d.tw = (const float2 *)f.dt->tw.p;
+            (f.ns < 32 ? d.tw : d.ptw) = (const float2 *)f.dt->tw.p;
             d.maxbits = a.stage != BF_OUT_RF ? a.maxbits : nullptr;
             if (nf > 1) {
                 const FramePrep &b = frames[job[2 * q + 1]];
                 d.rf2 = b.rf;
                 d.maxbits2 = b.stage != BF_OUT_RF ? b.maxbits : nullptr;
-                hl.demod_pairs = true;
             }
-            hl.demod_prefix.push_back(hl.demod_rows);
-            hl.demod_rows += d.rows;
-            hl.demod_max_ns = std::max(hl.demod_max_ns, f.ns);
-            hl.demod.push_back(d);
+            const int kind = f.ns < 32 ? 2 : f.ns > 4096 ? 1 : 0;
+            const int per = kind == 2 ? 1 : demod_units_per_block(d.lgn);
+            const int units = kind == 2 || nf > 1 ? d.rows : (d.rows + 1) / 2;
+            hl.demod_prefix[kind].push_back(hl.demod_blocks[kind]);
+            hl.demod_blocks[kind] += (units + per - 1) / per;
+            hl.demod[kind].push_back(d);
         }
     }
     for (size_t fi = 0; fi < frames.size(); ++fi) {
@@ -962,7 +963,12 @@ int DeviceLaunch::upload(const HostLaunch &hl, cudaStream_t st, bool async)
                  a_in = add(hl.ingest), a_ip = add(hl.ingest_prefix), a_e0 = add(hl.env[0]),
                  a_ep0 = add(hl.env_prefix[0]), a_e1 = add(hl.env[1]), a_ep1 = add(hl.env_prefix[1]),
                  a_ew = add(hl.envw), a_ewp = add(hl.envw_prefix), a_log = add(hl.log),
-                 a_bp = add(hl.blk_prefix), a_dm = add(hl.demod), a_dp = add(hl.demod_prefix);
+                 a_bp = add(hl.blk_prefix);
+    size_t a_dm[3], a_dp[3];
+    for (int k = 0; k < 3; ++k) {
+        a_dm[k] = add(hl.demod[k]);
+        a_dp[k] = add(hl.demod_prefix[k]);
+    }
     int rc = pack.reserve(std::max<size_t>(total, 128));
     if (!rc)
         rc = err.ensure(sizeof(int));
@@ -996,8 +1002,10 @@ int DeviceLaunch::upload(const HostLaunch &hl, cudaStream_t st, bool async)
     envw_prefix = (const int *)(d + a_ewp);
     log = (const LogJob *)(d + a_log);
     blk_prefix = (const int *)(d + a_bp);
-    demod = (const DemodJob *)(d + a_dm);
-    demod_prefix = (const int *)(d + a_dp);
+    for (int k = 0; k < 3; ++k) {
+        demod[k] = (const DemodJob *)(d + a_dm[k]);
+        demod_prefix[k] = (const int *)(d + a_dp[k]);
+    }
     return BF_OK;
 }
 
@@ -1057,9 +1065,10 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
         if (e != cudaSuccess)
             return cuda_fail(e, "ingest launch");
     }
-    if (!hl.demod.empty()) {
-        e = launch_demod(dl.demod, dl.demod_prefix,
-                         (int)hl.demod.size(), hl.demod_rows, hl.demod_max_ns, hl.demod_pairs, st);
+    for (int k = 0; k < 3; ++k) {
+        const int n = (int)hl.demod[k].size();
+        e = k == 2 ? launch_demod(dl.demod[k], dl.demod_prefix[k], n, hl.demod_blocks[k], st)
+                   : launch_demod16(dl.demod[k], dl.demod_prefix[k], n, hl.demod_blocks[k], k == 1, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "demodulation launch");
     }
@@ -1777,7 +1786,8 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
     for (auto &m : b->marks)
         if (e == cudaSuccess)
             e = cudaEventCreate(&m);
-    b->launches = (int)b->hl.igroups.size() + (b->hl.demod.empty() ? 0 : 1) +
+    b->launches = (int)b->hl.igroups.size() + (b->hl.demod[0].empty() ? 0 : 1) +
+                  (b->hl.demod[1].empty() ? 0 : 1) + (b->hl.demod[2].empty() ? 0 : 1) +
                   (int)b->hl.groups.size() + (b->hl.env[0].empty() ? 0 : 1) +
                   (b->hl.env[1].empty() ? 0 : 1) + (b->hl.envw.empty() ? 0 : 1) +
                   (b->hl.log.empty() ? 0 : 1);

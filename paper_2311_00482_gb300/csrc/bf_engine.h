@@ -124,7 +124,7 @@ struct FramePrep {
     Plan *solo = nullptr;  // the plan to use if the launch has no partner for the frame, or null
     std::shared_ptr<EnvTablesDev> et[2];  // envelope tables: without band, the DMAS band
     std::shared_ptr<FftTablesDev> ft;     // level twiddles, or the warp kernel's 512-point table
-    std::shared_ptr<FftTablesDev> dt;     // demodulation transform tables (n_samples; IQ only)
+    std::shared_ptr<FftTablesDev> dt;     // demodulation twiddles (IQ only)
     const int16_t *rf = nullptr;
     int ns = 0, na = 0, modes = 0, stage = 0, prec = 0;
     double pdas_p = 2.0;
@@ -163,10 +163,11 @@ struct HostLaunch {
     std::vector<LogJob> log;
     std::vector<int> blk_prefix;
     int log_blocks = 0;
-    std::vector<DemodJob> demod;   // IQ frames: records to analytic-signal pairs
-    std::vector<int> demod_prefix;
-    int demod_rows = 0, demod_max_ns = 0;
-    bool demod_pairs = false;  // some demodulation job covers a frame pair
+    // IQ frames, records to analytic-signal pairs: [0] 32 to 4096 samples, [1] 8192, [2]
+    // fewer than 32
+    std::vector<DemodJob> demod[3];
+    std::vector<int> demod_prefix[3];
+    int demod_blocks[3] = {0, 0, 0};
 };
 
 // Device copy of a launch description: every list in one allocation, sent in one
@@ -177,9 +178,10 @@ struct DeviceLaunch {
     const IngestJob *ingest = nullptr;
     const EnvJob *env[2] = {nullptr, nullptr}, *envw = nullptr;
     const LogJob *log = nullptr;
-    const DemodJob *demod = nullptr;
+    const DemodJob *demod[3] = {nullptr, nullptr, nullptr};
     const int *tile_prefix = nullptr, *ingest_prefix = nullptr, *env_prefix[2] = {nullptr, nullptr},
-              *envw_prefix = nullptr, *blk_prefix = nullptr, *demod_prefix = nullptr;
+              *envw_prefix = nullptr, *blk_prefix = nullptr,
+              *demod_prefix[3] = {nullptr, nullptr, nullptr};
     int upload(const HostLaunch &hl, cudaStream_t st, bool async);
 };
 

@@ -177,7 +177,8 @@ struct DemodJob {
     int nf, fi;           // frames of the beamforming job, the (first) frame's index in it
     unsigned *maxbits2;   // nf > 1: the second frame's image maxima (or null)
     float2 rot;           // exp(-j 2 pi f0 / fs)
-    const float2 *tw;     // [ns] exp(-2 pi i k / ns)
+    const float2 *tw;     // records below 32 samples: [ns] exp(-2 pi i k / ns)
+    const float2 *ptw;    // the others: level twiddles of the Fft16 transforms
     unsigned *maxbits;    // the frame's image maxima, zeroed by the job's first CTA (or null)
 };
 
@@ -245,10 +246,14 @@ cudaError_t launch_plan(const PlanJob &job, int *err_dev, cudaStream_t stream);
 // total_blocks: the jobs' rows x chunks (blk_prefix_dev: each job's first CTA).
 cudaError_t launch_ingest(const IngestJob *jobs_dev, const int *blk_prefix_dev, int njobs,
                           int total_blocks, int prec, cudaStream_t stream);
-// pairs: some job demodulates a frame pair (four transform buffers per CTA)
+// Demodulation of records below 32 samples, one row (or frame pair's row) per CTA.
 cudaError_t launch_demod(const DemodJob *jobs_dev, const int *row_prefix_dev, int njobs,
-                         int total_rows, int max_ns, bool pairs, cudaStream_t stream);
-size_t demod_smem_bytes(int ns, bool pairs);
+                         int total_rows, cudaStream_t stream);
+// Demodulation of the others (bf_demod.cu); big: records of 8192 samples.
+cudaError_t launch_demod16(const DemodJob *jobs_dev, const int *blk_prefix_dev, int njobs,
+                           int total_blocks, bool big, cudaStream_t stream);
+// Units (a frame's row pairs, a frame pair's rows) one CTA of launch_demod16 takes.
+__host__ __device__ constexpr int demod_units_per_block(int lg) { return lg >= 12 ? 1 : 4096 >> lg; }
 // f-k migration launches (bf_kernels.cu), in order on `stream`.
 cudaError_t launch_fkmig(const FkJob &job, cudaStream_t stream);
 // nf: frames per job (1, 2 or 4, with 4 on two-row tiles only; the frames of

@@ -259,10 +259,10 @@ __device__ __forceinline__ float4 demod_pair(const float2 *A, int j, int m, floa
                        (b.y - a0.y) * inv);
 }
 
-// One channel record per CTA (of one frame, or of the two frames of a frame
-// pair of a multi-frame job): analytic signal, then the complex interpolation
-// pairs of the IQ beamformer.
-__global__ void __launch_bounds__(256) demod_kernel(const DemodJob *__restrict__ jobs,
+// One channel record of fewer than 32 samples per CTA (of one frame, or of the two
+// frames of a frame pair of a multi-frame job): analytic signal, then the complex
+// interpolation pairs of the IQ beamformer.  (Longer records: bf_demod.cu.)
+__global__ void __launch_bounds__(32) demod_kernel(const DemodJob *__restrict__ jobs,
                                                     const int *__restrict__ row_prefix, int njobs)
 {
     extern __shared__ __align__(16) float2 dbuf[];
@@ -1638,19 +1638,13 @@ cudaError_t launch_ingest(const IngestJob *jobs_dev, const int *blk_prefix_dev, 
     return cudaGetLastError();
 }
 
-size_t demod_smem_bytes(int ns, bool pairs) { return (size_t)(pairs ? 4 : 3) * ns * sizeof(float2); }
-
 cudaError_t launch_demod(const DemodJob *jobs_dev, const int *row_prefix_dev, int njobs,
-                         int total_rows, int max_ns, bool pairs, cudaStream_t stream)
+                         int total_rows, cudaStream_t stream)
 {
     if (njobs <= 0 || total_rows <= 0)
         return cudaSuccess;
-    const size_t smem = demod_smem_bytes(max_ns, pairs);
-    int sms = 0;
-    cudaError_t e = kernel_setup((const void *)demod_kernel, smem, 256, false, &sms, nullptr);
-    if (e != cudaSuccess)
-        return e;
-    demod_kernel<<<total_rows, 256, smem, stream>>>(jobs_dev, row_prefix_dev, njobs);
+    // four transform buffers of at most 16 points
+    demod_kernel<<<total_rows, 32, 4 * 16 * sizeof(float2), stream>>>(jobs_dev, row_prefix_dev, njobs);
     return cudaGetLastError();
 }
 
