@@ -1378,16 +1378,6 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         ++lgk;
     }
     const double c = h->g.c, fs = h->g.fs, dz = c / (2.0 * fs);
-    std::vector<float> beta((size_t)n_angles * ne);
-    std::vector<double> sc((size_t)2 * n_angles);
-    for (int a = 0; a < n_angles; ++a) {
-        sc[2 * a] = std::sin(angles_rad[a]);
-        sc[2 * a + 1] = std::cos(angles_rad[a]);
-        for (int i = 0; i < ne; ++i) {
-            const double x = ((double)i - 0.5 * (double)(ne - 1)) * pitch;
-            beta[(size_t)a * ne + i] = (float)(kPi * x * sc[2 * a] / ((double)nt * dz));
-        }
-    }
     // The mapping tables (geometry only): rebuilt when the sample count, the
     // angles or the mapping change.
     const int half = nt / 2;
@@ -1395,21 +1385,28 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     std::vector<double> key{(double)n_samples, stolt ? 1.0 : 0.0};
     key.insert(key.end(), angles_rad, angles_rad + n_angles);
     const bool rebuild = key != h->fk_key;
+    const bool regs = nt >= 32 && nk >= 32;  // both axes by the register transforms
     std::shared_ptr<FftTablesDev> tt, tk;
-    int rc = fft_tables(nt, tt);
-    if (!rc)
+    int rc = fft_tables(regs ? 0 : nt, tt);
+    if (!rc && !regs)
         rc = fft_tables(nk, tk);
     const size_t nf = (size_t)nt / 2 + 1, img = (size_t)ne * n_samples;
     if (!rc)
-        rc = h->fk_D.ensure((size_t)n_angles * nf * nk * sizeof(float2));
+        rc = h->fk_D.ensure((size_t)n_angles * nk * (nf + (regs ? fk_pitch(nt) : 0)) * sizeof(float2));
     if (!rc)
         rc = h->fk_spec.ensure((size_t)(nt / 2) * nk * sizeof(float2));
     if (!rc && stage == BF_OUT_LOGDB)
         rc = h->fk_img.ensure(img * sizeof(float));
     if (!rc)
         rc = h->fk_max.ensure(sizeof(unsigned));
-    if (!rc)
-        rc = h->fk_beta.ensure(beta.size() * sizeof(float));
+    if (!rc && rebuild) {
+        // the previous call's kernels may still read the tables that are replaced
+        h->fk_key.clear();
+        cudaError_t ce = cudaStreamSynchronize(h->stream);
+        rc = ce == cudaSuccess ? BF_OK : cuda_fail(ce, "cudaStreamSynchronize");
+    }
+    if (!rc && rebuild)
+        rc = h->fk_beta.ensure((size_t)n_angles * ne * sizeof(float));
     if (!rc && rebuild)
         rc = h->fk_i0.ensure((size_t)n_angles * npts * sizeof(int));
     if (!rc && rebuild)
@@ -1417,25 +1414,33 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     if (rc)
         return rc;
     if (rebuild) {
+        std::vector<float> beta((size_t)n_angles * ne);
+        std::vector<double> sc((size_t)2 * n_angles);
+        for (int a = 0; a < n_angles; ++a) {
+            sc[2 * a] = std::sin(angles_rad[a]);
+            sc[2 * a + 1] = std::cos(angles_rad[a]);
+            for (int i = 0; i < ne; ++i) {
+                const double x = ((double)i - 0.5 * (double)(ne - 1)) * pitch;
+                const double turns = x * sc[2 * a] / ((double)nt * dz);  // half turns per bin
+                beta[(size_t)a * ne + i] = (float)(regs ? turns : kPi * turns);
+            }
+        }
         std::vector<int> i0;
         std::vector<float> aw;
-        fk_mapping_tables(ne, nt, nk, pitch, dz, sc, stolt, i0, aw);
+        fk_mapping_tables(nt, nk, pitch, dz, sc, stolt, regs ? lgk : 0, i0, aw);
         cudaError_t ce = cudaMemcpy(h->fk_i0.p, i0.data(), i0.size() * sizeof(int),
                                     cudaMemcpyHostToDevice);
         if (ce == cudaSuccess)
             ce = cudaMemcpy(h->fk_aw.p, aw.data(), aw.size() * sizeof(float), cudaMemcpyHostToDevice);
+        if (ce == cudaSuccess)
+            ce = cudaMemcpy(h->fk_beta.p, beta.data(), beta.size() * sizeof(float),
+                            cudaMemcpyHostToDevice);
         if (ce != cudaSuccess)
             return cuda_fail(ce, "bf_fkmig mapping tables");
         h->fk_key = key;
     }
     h->call.clear();  // the device tables above may have moved
     cudaStream_t st = h->stream;
-    cudaError_t e = cudaMemcpyAsync(h->fk_beta.p, beta.data(), beta.size() * sizeof(float),
-                                    cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && stage == BF_OUT_LOGDB)
-        e = cudaMemsetAsync(h->fk_max.p, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "bf_fkmig setup");
     FkJob J{};
     J.rf = rf_dev;
     J.D = (float2 *)h->fk_D.p;
@@ -1445,8 +1450,13 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     J.beta = (const float *)h->fk_beta.p;
     J.map_i0 = (const int *)h->fk_i0.p;
     J.map_aw = (const float2 *)h->fk_aw.p;
-    J.tw_t = (const float2 *)tt->tw.p;
-    J.tw_k = (const float2 *)tk->tw.p;
+    if (regs) {
+        J.ptw = (const float2 *)tt->tw.p;
+        J.E = J.D + (size_t)n_angles * nf * nk;
+    } else {
+        J.tw_t = (const float2 *)tt->tw.p;
+        J.tw_k = (const float2 *)tk->tw.p;
+    }
     J.na = n_angles;
     J.ne = ne;
     J.ns = n_samples;
@@ -1454,7 +1464,7 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     J.lgt = lgt;
     J.nk = nk;
     J.lgk = lgk;
-    e = launch_fkmig(J, st);
+    cudaError_t e = regs ? launch_fkmig16(J, st) : launch_fkmig(J, st);
     if (e != cudaSuccess)
         return cuda_fail(e, "f-k migration launch");
     if (stage == BF_OUT_LOGDB) {
@@ -1465,14 +1475,7 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         l.maxbits = J.maxbits;
         l.n = (int)img;
         l.vec4 = (img % 4 == 0 && ((uintptr_t)l.env & 15) == 0 && ((uintptr_t)l.out & 15) == 0) ? 1 : 0;
-        rc = h->fk_log.upload(&l, sizeof l);
-        int zero = 0;
-        if (!rc)
-            rc = h->fk_logp.upload(&zero, sizeof zero);
-        if (rc)
-            return rc;
-        e = launch_log((const LogJob *)h->fk_log.p, (const int *)h->fk_logp.p, 1,
-                       log_blocks((long long)img), 70.0f, st);
+        e = launch_log_one(l, 70.0f, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "log launch");
     }

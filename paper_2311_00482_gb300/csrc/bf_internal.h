@@ -80,6 +80,16 @@ __host__ __device__ inline int fft16_bin(int lg, int u, int q)
 // Bytes of the exchange buffer of one transform.
 __host__ __device__ constexpr int fft16_buf_bytes(int lg) { return (1 << lg) / 16 * 17 * 8; }
 
+// f-k migration by the register transforms: entries of a lateral bin's row of temporal
+// bins 0 .. nt/2 (whole 32-byte sectors); the Kx bin at position p of the lateral
+// transform's register order.
+__host__ __device__ constexpr int fk_pitch(int nt) { return nt / 2 + 4; }
+__host__ __device__ inline int fk_kx_bin(int lgk, int p)
+{
+    const int T = (1 << lgk) / 16;
+    return fft16_bin(lgk, p % T, p / T);
+}
+
 // Device-side error bits (written with atomicOr into a per-launch word).
 enum DevErr : int { kErrTimeout = 1, kErrWindow = 2, kErrConfig = 4 };
 
@@ -189,7 +199,9 @@ struct FkJob {
     float2 *spec;         // [nt/2][nk] migrated spectrum, rows Kz bin q = 1 .. nt/2
     float *img;           // [ne][ns] magnitude image
     unsigned *maxbits;    // image maximum (float bits) for the log stage, or null
-    const float *beta;    // [na][ne] pi x_i sin(theta_a) / (nt dz): lateral phase per time bin
+    // [na][ne] lateral phase per time bin: pi x_i sin(theta_a) / (nt dz); for
+    // launch_fkmig16 without the pi (half turns)
+    const float *beta;
     // the mapping, decided on the host in double precision: per (angle, Kz bin
     // q = 1 .. nt/2, Kx bin) the temporal bin i0 below the mapped position (-1:
     // the point takes nothing from this angle) and (interpolation weight of
@@ -198,6 +210,11 @@ struct FkJob {
     const float2 *map_aw; // [na][nt/2][nk]
     const float2 *tw_t;   // [nt] exp(-2 pi i k / nt)
     const float2 *tw_k;   // [nk] exp(-2 pi i k / nk)
+    // launch_fkmig16: the level twiddles; E [na][nk][fk_pitch(nt)] the spectra after the
+    // lateral transforms, Kx bins in the order of fk_kx_bin; the mapping tables are
+    // [na][nk][nt/2] in that order, and spec is [ne][nt/2]
+    const float2 *ptw;
+    float2 *E;
     int na, ne, ns, nt, lgt, nk, lgk;
 };
 
@@ -254,7 +271,9 @@ cudaError_t launch_demod16(const DemodJob *jobs_dev, const int *blk_prefix_dev, 
                            int total_blocks, bool big, cudaStream_t stream);
 // Units (a frame's row pairs, a frame pair's rows) one CTA of launch_demod16 takes.
 __host__ __device__ constexpr int demod_units_per_block(int lg) { return lg >= 12 ? 1 : 4096 >> lg; }
-// f-k migration launches (bf_kernels.cu), in order on `stream`.
+// f-k migration launches, in order on `stream`: transforms of 32 points and more along
+// both axes (bf_fk.cu), and the others (bf_kernels.cu).
+cudaError_t launch_fkmig16(const FkJob &job, cudaStream_t stream);
 cudaError_t launch_fkmig(const FkJob &job, cudaStream_t stream);
 // nf: frames per job (1, 2 or 4, with 4 on two-row tiles only; the frames of
 // one job share the delays; DAS / DMAS variants of the RF precisions, or the
@@ -267,6 +286,7 @@ cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, i
                             int total_blocks, bool big, cudaStream_t stream);
 // Column pairs one CTA of launch_envelope takes.
 __host__ __device__ constexpr int envelope_pairs_per_block(int lg) { return lg >= 12 ? 1 : 4096 >> lg; }
+cudaError_t launch_log_one(const LogJob &job, float dynamic_range_db, cudaStream_t stream);
 cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int njobs,
                        int total_blocks, float dynamic_range_db, cudaStream_t stream);
 // Jobs of solo plans (bf_solo.cu; RF precisions, any RF combiners), all of one split.

@@ -1494,19 +1494,12 @@ __global__ void __launch_bounds__(256) fk_depth_kernel(const FkJob J)
 
 constexpr int kLogPerBlock = 4096;
 
-__global__ void __launch_bounds__(256) log_kernel(const LogJob *__restrict__ jobs,
-                                                  const int *__restrict__ blk_prefix, int njobs,
-                                                  float dr)
+// Pixels of block blk of one image (launched as a programmatic dependent of the kernel
+// that writes the envelope: the block may start while that grid's last CTAs still
+// run, and waits here until the grid has completed and its results are visible).
+__device__ __forceinline__ void log_block(const LogJob &J, int blk, float dr)
 {
-    // blocks in launch order: the envelope kernels walk a batch's images in
-    // reverse, so the envelopes written last (still in L2) are read first
-    const int blk = blockIdx.x;
-    const int jb = find_job(blk_prefix, njobs, blk);
-    const LogJob J = jobs[jb];
-    const size_t base = (size_t)(blk - __ldg(blk_prefix + jb)) * kLogPerBlock;
-    // Launched as a programmatic dependent of the envelope kernel: this block
-    // may start while that grid's last CTAs still run, and waits here until
-    // the grid has completed and its envelopes and maxima are visible.
+    const size_t base = (size_t)blk * kLogPerBlock;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const float peak = __uint_as_float(__ldcg(J.maxbits));
     // 20 log10(e / peak) = (20 log10 2) (log2 e - log2 peak), the logarithm on the
@@ -1541,6 +1534,24 @@ __global__ void __launch_bounds__(256) log_kernel(const LogJob *__restrict__ job
             break;
         J.out[p] = db(__ldg(J.env + p));
     }
+}
+
+__global__ void __launch_bounds__(256) log_kernel(const LogJob *__restrict__ jobs,
+                                                  const int *__restrict__ blk_prefix, int njobs,
+                                                  float dr)
+{
+    // blocks in launch order: the envelope kernels walk a batch's images in
+    // reverse, so the envelopes written last (still in L2) are read first
+    const int blk = blockIdx.x;
+    const int jb = find_job(blk_prefix, njobs, blk);
+    const LogJob J = jobs[jb];
+    log_block(J, blk - __ldg(blk_prefix + jb), dr);
+}
+
+// One image, its job by value (no list to send).
+__global__ void __launch_bounds__(256) log_one_kernel(const LogJob J, float dr)
+{
+    log_block(J, blockIdx.x, dr);
 }
 
 template <int PREC, bool DMAS, bool CF, bool PDAS, int ROWS, int NF = 1>
@@ -1743,6 +1754,20 @@ cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int nj
     return cudaLaunchKernelEx(&cfg, log_kernel, jobs_dev, blk_prefix_dev, njobs, dynamic_range_db);
 }
 
+cudaError_t launch_log_one(const LogJob &job, float dynamic_range_db, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)log_blocks(job.n));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, log_one_kernel, job, dynamic_range_db);
+}
+
 int log_blocks(long long pixels) { return (int)((pixels + kLogPerBlock - 1) / kLogPerBlock); }
 
 cudaError_t kernel_setup(const void *k, size_t smem, int threads, bool max_carveout, int *sms,
@@ -1811,6 +1836,11 @@ cudaError_t launch_fkmig(const FkJob &J, cudaStream_t st)
         e = kernel_setup((const void *)fk_rows_kernel, s_rows, 256, false, &sms, nullptr);
     if (e != cudaSuccess)
         return e;
+    if (J.maxbits) {
+        e = cudaMemsetAsync(J.maxbits, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess)
+            return e;
+    }
     const int nf = J.nt / 2 + 1, half = J.nt / 2;
     fk_time_kernel<<<J.na * J.ne, 256, s_nt, st>>>(J);
     const int drows = J.na * nf;

@@ -240,11 +240,9 @@ void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, i
     }
 }
 
-void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
-                       const std::vector<double> &sc, bool stolt, std::vector<int> &i0,
-                       std::vector<float> &aw)
+void fk_mapping_tables(int nt, int nk, double pitch, double dz, const std::vector<double> &sc,
+                       bool stolt, int lgk, std::vector<int> &i0, std::vector<float> &aw)
 {
-    (void)ne;
     const int na = (int)sc.size() / 2, half = nt / 2;
     const size_t npts = (size_t)half * nk;
     i0.assign((size_t)na * npts, -1);
@@ -256,7 +254,8 @@ void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
         const double bet = std::sqrt(1.0 + ct - 0.5 * st * st);  // Stolt: depth scale
         parallel_for(half, [&](int qi) {
             const double Q = (double)(qi + 1);
-            for (int m = 0; m < nk; ++m) {
+            for (int p = 0; p < nk; ++p) {
+                const int m = lgk ? fk_kx_bin(lgk, p) : p;
                 const double X = (double)(m < nk / 2 ? m : m - nk) * r;
                 double pos, w;
                 bool ok;
@@ -280,7 +279,7 @@ void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
                 if (!ok)
                     continue;
                 const double fl = std::floor(pos);
-                const size_t t = (size_t)a * npts + (size_t)qi * nk + m;
+                const size_t t = (size_t)a * npts + (lgk ? (size_t)p * half + qi : (size_t)qi * nk + p);
                 i0[t] = (int)fl;
                 aw[2 * t] = (float)(pos - fl);
                 aw[2 * t + 1] = (float)w;

@@ -57,10 +57,10 @@ void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, i
 // taken), aw [na][nt/2][nk][2] its interpolation weight toward i0 + 1 and the
 // spectral weight.  sc: sin, cos of each angle.  stolt: Stolt's mapping of the
 // exploding-reflector fit instead of the exact plane-wave mapping.  Double
-// precision, evaluated in the order the definitions are written.
-void fk_mapping_tables(int ne, int nt, int nk, double pitch, double dz,
-                       const std::vector<double> &sc, bool stolt, std::vector<int> &i0,
-                       std::vector<float> &aw);
+// precision, evaluated in the order the definitions are written.  lgk > 0: transposed,
+// [na][nk][nt/2], Kx bins in the order of fk_kx_bin.
+void fk_mapping_tables(int nt, int nk, double pitch, double dz, const std::vector<double> &sc,
+                       bool stolt, int lgk, std::vector<int> &i0, std::vector<float> &aw);
 // exp(-2 pi i k / n) for k < n, interleaved.
 void fft_twiddles(int n, std::vector<float> &tw);
 // The level twiddles of every Fft16 transform (layout: bf_fft16.cuh), interleaved.

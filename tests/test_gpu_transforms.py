@@ -61,3 +61,25 @@ def test_static_stage_depths(torch, nz, band):  # noqa: F811
     err = 4.4e-6 * np.linalg.norm(y, axis=1, keepdims=True)
     tol = 8.686 * err / np.maximum(env, 10 ** (-3.5) * peak) + 8.686 * err.max() / peak + 1e-4
     assert np.all(np.abs(got[0] - oracle.log_compress(env)) <= tol)
+
+
+@pytest.mark.parametrize("ne,ns,na", [(2, 2, 1), (9, 15, 2), (8, 16, 1), (16, 15, 1), (16, 16, 2), (17, 100, 1),
+                                      (33, 513, 3), (64, 1024, 1), (65, 2049, 2), (300, 64, 1),
+                                      (3, 4096, 1)])
+@pytest.mark.parametrize("stolt", [False, True])
+def test_fk_sizes(torch, ne, ns, na, stolt):  # noqa: F811
+    """Both transform families around their boundary (32 points along either axis) and
+    odd channel counts; tolerance of test_gpu_fk (2e-5 of the image's norm)."""
+    rng = np.random.default_rng(ne * 5000 + ns)
+    angles = np.deg2rad(np.linspace(-6.0, 6.0, na)) if na > 1 else np.array([0.0])
+    rf = rng.integers(-20000, 20000, (na, ne, ns), dtype=np.int16)
+    h = bf.bf_create(ne, 0.3e-3, 1.5, (8, 8, -1e-3, 1e-3, 5e-3, 6e-3), 20e6, 5e6, 1540.0)
+    try:
+        out = torch.full((ne, ns), float("nan"), device="cuda")
+        bf.bf_fkmig(h, torch.from_numpy(rf).cuda(), ns, angles, bf.BF_FK_STOLT if stolt else 0, out)
+        bf.bf_sync(h)
+    finally:
+        bf.bf_destroy(h)
+    ref = (oracle.fk_stolt if stolt else oracle.fk_migrate)(rf, 0.3e-3, angles, 20e6, 1540.0)
+    got = out.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 2e-5 * np.linalg.norm(ref)
