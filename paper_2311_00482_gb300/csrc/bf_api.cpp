@@ -291,15 +291,14 @@ static int angle_tables_dev(bf_handle *h, PlanKey key, std::shared_ptr<AngleTabl
         out = it->second;
         return BF_OK;
     }
-    PlanHost ph;
+    PlanHost<int16_t> ph;
     angle_tables(h->g, h->geo, key.ns, key.angles, ph);
-    const std::vector<int16_t> valid(ph.valid.begin(), ph.valid.end());  // rows are below 2^15
     auto t = std::make_shared<AngleTablesDev>();
     int rc = t->colK.upload(ph.colK.data(), ph.colK.size() * sizeof(int));
     if (!rc) rc = t->colF.upload(ph.colF.data(), ph.colF.size() * sizeof(float));
     if (!rc) rc = t->rowK.upload(ph.rowK.data(), ph.rowK.size() * sizeof(int));
     if (!rc) rc = t->rowF.upload(ph.rowF.data(), ph.rowF.size() * sizeof(float));
-    if (!rc) rc = t->valid.upload(valid.data(), valid.size() * sizeof(int16_t));
+    if (!rc) rc = t->valid.upload(ph.valid.data(), ph.valid.size() * sizeof(int16_t));
     if (rc)
         return rc;
     h->angle_tabs.emplace(std::move(key), t);
@@ -1582,7 +1581,7 @@ BF_API int bf_host_tables(const bf_geometry *geom, const bf_grid *grid, double f
     g.c = c_mps;
     GeometryHost geo;
     geometry_tables(g, geo);
-    PlanHost ph;
+    PlanHost<int> ph;
     angle_tables(g, geo, n_samples, std::vector<double>(angles_rad, angles_rad + n_angles),
                  ph);
     const int nxp = pad_cols(g.nx);

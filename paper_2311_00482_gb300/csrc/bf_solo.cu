@@ -587,8 +587,8 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
     }
 }
 
-// Records of a solo plan: one CTA per (tile, angle group), one thread per (angle,
-// channel) of a channel group.  Per step: for every row band the channels that
+// Records of a solo plan: one CTA per (tile, angle group, channel group), one thread
+// per (angle, channel).  Per step: for every row band the channels that
 // all its pixels count for all the group's angles, and those that only some do;
 // per (angle, run of channels) the first staged pair of the run's windows.
 __global__ void __launch_bounds__(128) solo_plan_kernel(const PlanJob J, int *__restrict__ err)
@@ -602,78 +602,76 @@ __global__ void __launch_bounds__(128) solo_plan_kernel(const PlanJob J, int *__
     const int amax = (J.na + J.ang_groups - 1) / J.ang_groups;
     const int G = J.group, ngroups = (J.ne + G - 1) / G, runs = G / J.run;
     const int words = solo_record_words(amax, runs);
-    for (int g = 0; g < ngroups; ++g) {
-        const int k = threadIdx.x / G, c = threadIdx.x - k * G, i = g * G + c;
-        if (k < an) {
-            int lo = INT_MAX, hi = INT_MIN;
-            unsigned any = 0, full = (1u << J.bands) - 1;
-            const int a = a0 + k;
-            for (int w = 0; w < kTileCols && i < J.ne; ++w) {
-                const int ix = tx * kTileCols + w;
-                if (ix >= J.nx)
-                    break;
-                const short2 vr = J.valid[((size_t)a * J.ne + i) * J.nxp + ix];
-                for (int b = 0; b < J.bands; ++b) {
-                    const int b0 = tz0 + b * J.rows, b1 = min(b0 + J.rows - 1, J.nz - 1);
-                    if (b0 > b1)
-                        continue;  // band below the grid: nothing to store there
-                    if (vr.x <= b1 && vr.y >= b0)
-                        any |= 1u << b;
-                    if (!(vr.x <= b0 && vr.y >= b1))
-                        full &= ~(1u << b);
-                }
-                const int r0 = max((int)vr.x, tz0), r1 = min((int)vr.y, tz_last);
-                if (r0 > r1)
-                    continue;
-                const float d2 = J.dx2[(size_t)i * J.nxp + ix];
-                const int kb = J.colK[a * J.nx + ix];
-                const float fb = J.colF[a * J.nx + ix];
-                const int k0 = kb + J.rowK[a * J.nz + r0] +
-                               __float2int_rd(fb + J.rowF[a * J.nz + r0] + rx_excess(d2, J.rowZ[r0]));
-                const int k1 = kb + J.rowK[a * J.nz + r1] +
-                               __float2int_rd(fb + J.rowF[a * J.nz + r1] + rx_excess(d2, J.rowZ[r1]));
-                lo = min(lo, min(k0, k1));
-                hi = max(hi, max(k0, k1));
+    const int g = blockIdx.z;
+    const int k = threadIdx.x / G, c = threadIdx.x - k * G, i = g * G + c;
+    if (k < an) {
+        int lo = INT_MAX, hi = INT_MIN;
+        unsigned any = 0, full = (1u << J.bands) - 1;
+        const int a = a0 + k;
+        for (int w = 0; w < kTileCols && i < J.ne; ++w) {
+            const int ix = tx * kTileCols + w;
+            if (ix >= J.nx)
+                break;
+            const short2 vr = J.valid[((size_t)a * J.ne + i) * J.nxp + ix];
+            for (int b = 0; b < J.bands; ++b) {
+                const int b0 = tz0 + b * J.rows, b1 = min(b0 + J.rows - 1, J.nz - 1);
+                if (b0 > b1)
+                    continue;  // band below the grid: nothing to store there
+                if (vr.x <= b1 && vr.y >= b0)
+                    any |= 1u << b;
+                if (!(vr.x <= b0 && vr.y >= b1))
+                    full &= ~(1u << b);
             }
-            kmin[k][c] = lo;
-            kmax[k][c] = hi;
-            flags[k][c] = lo > hi ? 0u : any | ((full & any) << 8);
+            const int r0 = max((int)vr.x, tz0), r1 = min((int)vr.y, tz_last);
+            if (r0 > r1)
+                continue;
+            const float d2 = J.dx2[(size_t)i * J.nxp + ix];
+            const int kb = J.colK[a * J.nx + ix];
+            const float fb = J.colF[a * J.nx + ix];
+            const int k0 = kb + J.rowK[a * J.nz + r0] +
+                           __float2int_rd(fb + J.rowF[a * J.nz + r0] + rx_excess(d2, J.rowZ[r0]));
+            const int k1 = kb + J.rowK[a * J.nz + r1] +
+                           __float2int_rd(fb + J.rowF[a * J.nz + r1] + rx_excess(d2, J.rowZ[r1]));
+            lo = min(lo, min(k0, k1));
+            hi = max(hi, max(k0, k1));
         }
-        __syncthreads();
-        int *rec = J.wtab + ((size_t)(ag * ngroups + g) * ntiles + tile) * words;
-        if (threadIdx.x < kWarps) {
-            const int b = threadIdx.x;
-            unsigned mf = 0, mp = 0;
-            for (int ch = 0; ch < G; ++ch) {
-                bool all = true, some = false;
-                for (int q = 0; q < an; ++q) {
-                    all = all && ((flags[q][ch] >> (8 + b)) & 1u);
-                    some = some || ((flags[q][ch] >> b) & 1u);
-                }
-                if (all)
-                    mf |= 1u << ch;
-                else if (some)
-                    mp |= 1u << ch;
+        kmin[k][c] = lo;
+        kmax[k][c] = hi;
+        flags[k][c] = lo > hi ? 0u : any | ((full & any) << 8);
+    }
+    __syncthreads();
+    int *rec = J.wtab + ((size_t)(ag * ngroups + g) * ntiles + tile) * words;
+    if (threadIdx.x < kWarps) {
+        const int b = threadIdx.x;
+        unsigned mf = 0, mp = 0;
+        for (int ch = 0; ch < G; ++ch) {
+            bool all = true, some = false;
+            for (int q = 0; q < an; ++q) {
+                all = all && ((flags[q][ch] >> (8 + b)) & 1u);
+                some = some || ((flags[q][ch] >> b) & 1u);
             }
-            rec[b] = (int)mf;
-            rec[kWarps + b] = (int)mp;
-        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + amax * runs) {
-            const int q = (threadIdx.x - 32) / runs, c0 = (threadIdx.x - 32 - q * runs) * J.run;
-            int lo = INT_MAX, hi = INT_MIN;
-            for (int ch = c0; ch < c0 + J.run && q < an; ++ch) {
-                lo = min(lo, kmin[q][ch]);
-                hi = max(hi, kmax[q][ch]);
-            }
-            int w0 = kNoWindow;
-            if (lo <= hi) {
-                // pairs lo + kPadL .. hi + kPadL, two pairs of margin on either side
-                w0 = (lo + kPadL - 2) & ~(J.align - 1);
-                if (hi + kPadL + 2 - w0 + 1 > J.wmax)
-                    atomicOr(err, kErrWindow);
-            }
-            rec[2 * kWarps + threadIdx.x - 32] = w0;
+            if (all)
+                mf |= 1u << ch;
+            else if (some)
+                mp |= 1u << ch;
         }
-        __syncthreads();
+        rec[b] = (int)mf;
+        rec[kWarps + b] = (int)mp;
+    } else if (threadIdx.x >= 32 && threadIdx.x < 32 + amax * runs) {
+        const int q = (threadIdx.x - 32) / runs, c0 = (threadIdx.x - 32 - q * runs) * J.run;
+        int lo = INT_MAX, hi = INT_MIN;
+        for (int ch = c0; ch < c0 + J.run && q < an; ++ch) {
+            lo = min(lo, kmin[q][ch]);
+            hi = max(hi, kmax[q][ch]);
+        }
+        int w0 = kNoWindow;
+        if (lo <= hi) {
+            // pairs lo + kPadL .. hi + kPadL, two pairs of margin on either side
+            w0 = (lo + kPadL - 2) & ~(J.align - 1);
+            if (hi + kPadL + 2 - w0 + 1 > J.wmax)
+                atomicOr(err, kErrWindow);
+        }
+        rec[2 * kWarps + threadIdx.x - 32] = w0;
     }
 }
 
@@ -735,7 +733,8 @@ size_t solo_smem_bytes(int wmax, int group, int prec, int ang, int split, int va
 
 cudaError_t launch_solo_plan(const PlanJob &job, int *err_dev, cudaStream_t stream)
 {
-    solo_plan_kernel<<<dim3(job.tiles_x * job.tiles_z, job.ang_groups), 128, 0, stream>>>(job, err_dev);
+    const dim3 grid(job.tiles_x * job.tiles_z, job.ang_groups, (job.ne + job.group - 1) / job.group);
+    solo_plan_kernel<<<grid, 128, 0, stream>>>(job, err_dev);
     return cudaGetLastError();
 }
 

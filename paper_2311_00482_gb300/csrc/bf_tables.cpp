@@ -107,8 +107,9 @@ void geometry_tables(const GeomHost &g, GeometryHost &out)
     });
 }
 
+template <class Row>
 void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
-                  const std::vector<double> &angles, PlanHost &out)
+                  const std::vector<double> &angles, PlanHost<Row> &out)
 {
     const double kappa = g.fs / g.c;
     const int na = (int)angles.size();
@@ -159,12 +160,17 @@ void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
                 hi = -1;
             }
             size_t o = (((size_t)a * g.ne + i) * nxp + ix) * 2;
-            out.valid[o] = lo;
-            out.valid[o + 1] = hi;
+            out.valid[o] = (Row)lo;
+            out.valid[o + 1] = (Row)hi;
         }
     });
     out.nsp = (ns + kPadL + 7) / 8 * 8;
 }
+
+template void angle_tables(const GeomHost &, const GeometryHost &, int, const std::vector<double> &,
+                           PlanHost<int> &);
+template void angle_tables(const GeomHost &, const GeometryHost &, int, const std::vector<double> &,
+                           PlanHost<int16_t> &);
 
 void tile_window(const GeomHost &g, const std::vector<double> &angles, int prec, int tile_rows,
                  int run, int &wmax, int &box_out)

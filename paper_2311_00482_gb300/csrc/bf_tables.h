@@ -26,11 +26,12 @@ struct GeometryHost {
     std::vector<float> dx2;        // [ne][nxp] (kappa (x_p - x_i))^2, columns padded
 };
 
-// Tables of one angle set and sample count.
+// Tables of one angle set and sample count.  Row: the type rows are stored in.
+template <class Row>
 struct PlanHost {
     std::vector<int> colK, rowK;
     std::vector<float> colF, rowF;
-    std::vector<int> valid;        // [na][ne][nxp][2] first / last counted row (padding: none)
+    std::vector<Row> valid;        // [na][ne][nxp][2] first / last counted row (padding: none)
     int nsp = 0;
 };
 
@@ -47,8 +48,10 @@ void geometry_tables(const GeomHost &g, GeometryHost &out);
 // channels, and the width of the tensor copies it is fetched in.
 void tile_window(const GeomHost &g, const std::vector<double> &angles, int prec, int tile_rows,
                  int run, int &wmax, int &box);
+// (Row: int16_t for the device, whose grids are below 2^15 rows, or int)
+template <class Row>
 void angle_tables(const GeomHost &g, const GeometryHost &geo, int ns,
-                  const std::vector<double> &angles, PlanHost &out);
+                  const std::vector<double> &angles, PlanHost<Row> &out);
 // Channels per pipeline stage whose sample windows take stage_bytes.
 int stage_channels(int wmax, int prec, int rows_per_thread, int stage_bytes, int ne);
 void bandpass_bins(int nz, double z0, double z1, double c, double f0, int &lo, int &hi);
