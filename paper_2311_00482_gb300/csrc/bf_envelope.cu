@@ -36,6 +36,7 @@
 #include "bf_envelope_pairs.cuh"
 #include "bf_fft16.cuh"
 #include "bf_internal.h"
+#include "bf_launch.cuh"
 
 namespace bfi {
 namespace {
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(32 * kEnvWarps, 2)
     extern __shared__ __align__(16) float2 esm[];
     // the log stage's blocks may be scheduled as this grid's CTAs finish (they
     // wait for the whole grid before reading its results)
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {
         // [16][kPitch]: W_N^(k1 n2) from the job's table exp(-2 pi i k / N), k < N
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(32 * kEnvWarps, 2)
         }
     }
     __syncthreads();
+    wait_for_producer();  // the beamformed images
     const uint32_t twa = smem_addr(esm);
     const uint32_t buf = smem_addr(esm + (1 + warp) * kR * kPitch);  // this warp's transposes
     // this warp's holding area, [r][lane]: at most one transform's registers and
@@ -282,12 +284,13 @@ __global__ void __launch_bounds__(BIG ? kEnvBigThreads : kEnvThreads, BIG ? 1 : 
     const int blk = gridDim.x - 1 - blockIdx.x;
     // the log stage's blocks may be scheduled as this grid's CTAs finish (they
     // wait for the whole grid before reading its results)
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     const int jb = find_pair_job(blk_prefix, njobs, blk);
     const EnvJob &J = jobs[jb];
     const int first = blk - __ldg(blk_prefix + jb);
     const uint32_t bufs = smem_addr(esm);
     const uint32_t hold = bufs + (uint32_t)(THREADS * 17 * 8);
+    wait_for_producer();  // the beamformed images
     float lmax = 0.f;
     auto run = [&](auto lg, auto conv) {
         constexpr int LG = decltype(lg)::value;
@@ -344,7 +347,7 @@ cudaError_t launch_envelope_warp(const EnvJob *jobs_dev, const int *pair_prefix_
 {
     if (njobs <= 0 || total_pairs <= 0)
         return cudaSuccess;
-    const size_t smem = envelope_warp_smem_bytes();
+    size_t smem = envelope_warp_smem_bytes();
     int sms = 0, occ = 0;
     cudaError_t e = kernel_setup((const void *)envelope_warp_kernel, smem, 32 * kEnvWarps, false,
                                  &sms, &occ);
@@ -352,9 +355,15 @@ cudaError_t launch_envelope_warp(const EnvJob *jobs_dev, const int *pair_prefix_
         return e;
     const int cap = sms * (occ > 0 ? occ : 1);
     const int want = (total_pairs + kEnvWarps - 1) / kEnvWarps;
-    envelope_warp_kernel<<<want < cap ? want : cap, 32 * kEnvWarps, smem, stream>>>(
-        jobs_dev, pair_prefix_dev, njobs, total_pairs);
-    return cudaGetLastError();
+    const bool dependent = want <= sms;
+    if (dependent) {
+        smem = spread_smem(smem, want, sms);
+        e = kernel_setup((const void *)envelope_warp_kernel, smem, 32 * kEnvWarps, false, &sms, nullptr);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return launch_kernel(envelope_warp_kernel, dim3((unsigned)(want < cap ? want : cap)), 32 * kEnvWarps,
+                         smem, dependent, stream, jobs_dev, pair_prefix_dev, njobs, total_pairs);
 }
 
 template <bool BIG>
@@ -362,14 +371,20 @@ static cudaError_t launch_envelope_t(const EnvJob *jobs_dev, const int *blk_pref
                                      int total_blocks, cudaStream_t stream)
 {
     constexpr int threads = BIG ? kEnvBigThreads : kEnvThreads;
-    const size_t smem = (size_t)threads * (17 + 16) * sizeof(float2);
+    size_t smem = (size_t)threads * (17 + 16) * sizeof(float2);
     const void *k = (const void *)envelope_kernel<BIG>;
     int sms = 0;
     cudaError_t e = kernel_setup(k, smem, threads, true, &sms, nullptr);
     if (e != cudaSuccess)
         return e;
-    envelope_kernel<BIG><<<total_blocks, threads, smem, stream>>>(jobs_dev, blk_prefix_dev, njobs);
-    return cudaGetLastError();
+    const bool dependent = total_blocks <= sms;
+    if (dependent) {
+        smem = spread_smem(smem, total_blocks, sms);
+        e = kernel_setup(k, smem, threads, true, &sms, nullptr);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return launch_kernel(envelope_kernel<BIG>, dim3((unsigned)total_blocks), threads, smem, dependent, stream, jobs_dev, blk_prefix_dev, njobs);
 }
 
 cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,

@@ -19,6 +19,7 @@
 // transforms and a synchronous upload took 59 us per call, these 29 us.
 #include "bf_fft16.cuh"
 #include "bf_internal.h"
+#include "bf_launch.cuh"
 
 namespace bfi {
 namespace {
@@ -31,16 +32,6 @@ struct FkShape {
     static constexpr int T = (1 << LG) / 16;
     static constexpr int threads(int least) { return T > least ? T : least; }
 };
-
-__device__ __forceinline__ void dependents_may_start()
-{
-    asm volatile("griddepcontrol.launch_dependents;");
-}
-
-__device__ __forceinline__ void wait_for_producer()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
 
 template <int LG, int THREADS>
 __global__ void __launch_bounds__(THREADS) fk_time16_kernel(const FkJob J)
@@ -256,17 +247,7 @@ cudaError_t launch_after(void (*k)(Params...), dim3 blocks, int threads, size_t 
     cudaError_t e = kernel_setup((const void *)k, smem, threads, true, &sms, nullptr);
     if (e != cudaSuccess)
         return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = blocks;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, args...);
+    return launch_kernel(k, blocks, threads, smem, dependent, st, args...);
 }
 
 template <int LG>

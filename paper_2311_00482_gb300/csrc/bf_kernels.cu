@@ -34,6 +34,7 @@
 #include "bf_device.cuh"
 #include "bf_fft.cuh"
 #include "bf_internal.h"
+#include "bf_launch.cuh"
 
 namespace bfi {
 namespace {
@@ -153,6 +154,7 @@ template <int PREC>
 __global__ void __launch_bounds__(256) ingest_kernel(const IngestJob *__restrict__ jobs,
                                                      const int *__restrict__ blk_prefix, int njobs)
 {
+    dependents_may_start();
     const int jb = find_job(blk_prefix, njobs, blockIdx.x);
     const IngestJob J = jobs[jb];
     const int local = blockIdx.x - __ldg(blk_prefix + jb);
@@ -1500,7 +1502,7 @@ constexpr int kLogPerBlock = 4096;
 __device__ __forceinline__ void log_block(const LogJob &J, int blk, float dr)
 {
     const size_t base = (size_t)blk * kLogPerBlock;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_producer();
     const float peak = __uint_as_float(__ldcg(J.maxbits));
     // 20 log10(e / peak) = (20 log10 2) (log2 e - log2 peak), the logarithm on the
     // special-function unit (absolute error ~1e-6 of a unit of log2: ~1e-5 dB)
@@ -1741,31 +1743,12 @@ cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int nj
     // programmatic stream serialization: the blocks may be scheduled before the
     // envelope kernel ends (the kernel's griddepcontrol.wait orders the reads),
     // which hides this launch behind that kernel's last CTAs
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)total_blocks);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, log_kernel, jobs_dev, blk_prefix_dev, njobs, dynamic_range_db);
+    return launch_kernel(log_kernel, dim3((unsigned)total_blocks), 256, 0, true, stream, jobs_dev, blk_prefix_dev, njobs, dynamic_range_db);
 }
 
 cudaError_t launch_log_one(const LogJob &job, float dynamic_range_db, cudaStream_t stream)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)log_blocks(job.n));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, log_one_kernel, job, dynamic_range_db);
+    return launch_kernel(log_one_kernel, dim3((unsigned)log_blocks(job.n)), 256, 0, true, stream, job, dynamic_range_db);
 }
 
 int log_blocks(long long pixels) { return (int)((pixels + kLogPerBlock - 1) / kLogPerBlock); }

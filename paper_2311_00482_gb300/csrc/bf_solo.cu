@@ -32,6 +32,7 @@
 #include "../../include/bf.h"
 #include "bf_device.cuh"
 #include "bf_internal.h"
+#include "bf_launch.cuh"
 
 namespace bfi {
 namespace {
@@ -206,6 +207,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
     constexpr int EX = solo_exchange_bytes(SPLIT, DMAS, CF, PDAS);
     auto stage_base = [&](int st) { return smem + kSoloHeaderBytes + EX + (size_t)st * stage_stride; };
 
+    dependents_may_start();
     if (threadIdx.x == 0) {
         for (int st = 0; st < kSoloStages; ++st) {
             mbar_init(&sh.full[st], 1);
@@ -222,6 +224,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
         // the header, its tables and windows by tensor copies.  A copy costs the
         // issuing warp about 65 cycles, so one copy brings the windows of a run of
         // (up to four) adjacent channels, which start at the same pair.
+        wait_for_producer();  // the staged pairs (and the deadlines start here)
         unsigned r = 0;
         for (int tg = blockIdx.x; tg < total_tiles; tg += gridDim.x) {
             const unsigned long long deadline = global_ns() + kWaitNs;
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
     }
 
     // ================= consumer warps
+    wait_for_producer();  // so that their deadlines do not run while the pairs are made
     const int band = warp % BANDS, part = warp / BANDS;
     constexpr int NV = solo_sums(DMAS, CF, PDAS);
     // sums handed over by warp part > 0 of this band: value v at ex(part) + 256 v
@@ -687,8 +691,16 @@ cudaError_t launch_t(const BfJob *jobs, const int *prefix, int njobs, int tiles,
     const int grid = std::max(1, std::min(tiles, std::max(occ, 1) * sms));
     const int stride = (int)((smem - kSoloHeaderBytes - solo_exchange_bytes(SPLIT, DMAS, CF, PDAS)) /
                              kSoloStages);
-    k<<<grid, kThreads + 32, smem, st>>>(jobs, prefix, njobs, tiles, stride, err);
-    return cudaGetLastError();
+    // a launch of one wave starts under the ingest kernel's last CTAs (in larger ones
+    // the early CTAs would take the SMs from the kernel they wait for)
+    const bool dependent = tiles <= std::max(occ, 1) * sms;
+    if (dependent) {
+        smem = spread_smem(smem, grid, sms);
+        e = kernel_setup((const void *)k, smem, kThreads + 32, true, &sms, nullptr);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return launch_kernel(k, dim3((unsigned)grid), kThreads + 32, smem, dependent, st, jobs, prefix, njobs, tiles, stride, err);
 }
 
 template <int PREC, int SPLIT>

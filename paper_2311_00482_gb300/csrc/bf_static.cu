@@ -23,6 +23,7 @@
 #include "bf_envelope_pairs.cuh"
 #include "bf_fft.cuh"
 #include "bf_internal.h"
+#include "bf_launch.cuh"
 
 namespace bfi {
 namespace {
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(256, 2)
                              float *__restrict__ env, float *__restrict__ maxima)
 {
     extern __shared__ __align__(16) float2 sbuf[];
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     float2 *tab = sbuf + 256 * (17 + 16);
     fft16_fill_shared<LG>(tab);
     __syncthreads();
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(256) static_envelope_kernel(const float *__res
                                                               int kb_hi, float *__restrict__ env,
                                                               float *__restrict__ maxima)
 {
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     extern __shared__ __align__(16) float2 sbuf[];
     const int m = nz, lgm = 31 - __clz(m);
     const int C = m >= 2048 ? 1 : 2048 / m;  // complex columns: pairs of image columns
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict
                                                          const float *__restrict__ maxima, int nmax,
                                                          float *__restrict__ out, float dr)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the envelope kernel has completed
+    wait_for_producer();
     __shared__ float red[8];
     float peak = 0.f;
     for (int k = threadIdx.x; k < nmax; k += blockDim.x)
@@ -341,16 +342,7 @@ extern "C" BF_API int bf_logdb_static(const float *y_dev, int32_t nx, int32_t nz
         return cuda_fail(e, "envelope launch");
     const int n = nx * nz;
     const int vec4 = n % 4 == 0 && (reinterpret_cast<uintptr_t>(db_dev) & 15) == 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((n + kStaticLogPixels - 1) / kStaticLogPixels));
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];  // scheduled while the envelope kernel's last CTAs run
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, static_log_kernel, (const float *)env, n, vec4, (const float *)maxima,
-                           blocks, db_dev, 70.0f);
+    e = launch_kernel(static_log_kernel, dim3((unsigned)((n + kStaticLogPixels - 1) / kStaticLogPixels)), 256,
+                      0, true, st, (const float *)env, n, vec4, (const float *)maxima, blocks, db_dev, 70.0f);
     return e == cudaSuccess ? BF_OK : cuda_fail(e, "log launch");
 }
