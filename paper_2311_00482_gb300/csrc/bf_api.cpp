@@ -761,7 +761,8 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
             j.box = box_nf;
         const int combiners = j.modes & (BF_DMAS | BF_CF | BF_PDAS);
         const int variant =
-            (((p->split * 8 + nf) * 16 + p->rows) * 4 + f.prec) * 16 + combiners;
+            ((((p->split * 2 + (p->ang > 1 ? 1 : 0)) * 8 + nf) * 16 + p->rows) * 4 + f.prec) * 16 +
+            combiners;
         groups[variant].push_back(j);
         const size_t sm = p->split
                               ? solo_smem_bytes(p->wmax, p->group, f.prec, p->ang, p->split, combiners)
@@ -771,7 +772,8 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
     }
     for (auto &kv : groups) {
         HostLaunch::Group g;
-        g.split = kv.first / (8 * 16 * 4 * 16);
+        g.split = kv.first / (2 * 8 * 16 * 4 * 16);
+        g.ang = kv.first / (8 * 16 * 4 * 16) % 2 ? kSoloAngles : 1;
         g.nf = (kv.first / (16 * 4 * 16)) % 8;
         g.rows = (kv.first / 64) % 16;
         g.prec = (kv.first / 16) % 4;
@@ -1079,7 +1081,7 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
         const BfJob *jobs = dl.jobs + g.first;
         const int *prefix = dl.tile_prefix + g.prefix_first;
         e = g.split ? launch_solo(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant, g.split,
-                                  (int *)dl.err.p, st)
+                                  g.ang, (int *)dl.err.p, st)
                     : launch_beamform(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant,
                                       g.rows, g.nf, (int *)dl.err.p, st);
         if (e != cudaSuccess)

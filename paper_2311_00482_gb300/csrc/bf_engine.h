@@ -138,7 +138,7 @@ struct FramePrep {
 
 struct HostLaunch {
     struct Group {  // one beamforming launch (split > 0: solo jobs)
-        int prec, variant, rows, nf, split, first, count, prefix_first, tiles;
+        int prec, variant, rows, nf, split, ang, first, count, prefix_first, tiles;
         size_t smem;
     };
     struct IGroup {  // one ingest launch

@@ -289,9 +289,10 @@ __host__ __device__ constexpr int envelope_pairs_per_block(int lg) { return lg >
 cudaError_t launch_log_one(const LogJob &job, float dynamic_range_db, cudaStream_t stream);
 cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int njobs,
                        int total_blocks, float dynamic_range_db, cudaStream_t stream);
-// Jobs of solo plans (bf_solo.cu; RF precisions, any RF combiners), all of one split.
+// Jobs of solo plans (bf_solo.cuh; RF precisions, any RF combiners), all of one split,
+// with one angle per stage each (ang 1) or more.
 cudaError_t launch_solo(const BfJob *jobs_dev, const int *tile_prefix_dev, int njobs, int total_tiles,
-                        size_t smem_bytes, int prec, int variant, int split, int *err_dev,
+                        size_t smem_bytes, int prec, int variant, int split, int ang, int *err_dev,
                         cudaStream_t stream);
 cudaError_t launch_solo_plan(const PlanJob &job, int *err_dev, cudaStream_t stream);
 // ang: angles of a stage; split: warps per row pair.
