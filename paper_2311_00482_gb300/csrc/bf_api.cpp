@@ -791,6 +791,9 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         g.tiles = acc;
         hl.groups.push_back(g);
     }
+    // the largest launches first: the others fill in as their last CTAs leave
+    std::stable_sort(hl.groups.begin(), hl.groups.end(),
+                     [](const HostLaunch::Group &a, const HostLaunch::Group &b) { return a.tiles > b.tiles; });
     std::map<int, std::vector<IngestJob>> ig;
     // IQ frames: one demodulation job per frame, or per frame pair of a
     // multi-frame job (into the lead's interleaved array)
@@ -1077,16 +1080,33 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     e = mark(1);
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
-    for (const HostLaunch::Group &g : hl.groups) {
+    // in a capture with a branch, launches after the first go to its work streams
+    const int spread = branch ? std::min<int>((int)hl.groups.size() - 1, MarkBranch::kWork) : 0;
+    if (spread > 0)
+        e = cudaEventRecord(branch->work_fork, st);
+    for (int w = 0; w < spread && e == cudaSuccess; ++w)
+        e = cudaStreamWaitEvent(branch->work[w], branch->work_fork, 0);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "cudaEventRecord (fork)");
+    for (size_t k = 0; k < hl.groups.size(); ++k) {
+        const HostLaunch::Group &g = hl.groups[k];
+        const cudaStream_t to = spread > 0 && k > 0 ? branch->work[(k - 1) % spread] : st;
         const BfJob *jobs = dl.jobs + g.first;
         const int *prefix = dl.tile_prefix + g.prefix_first;
         e = g.split ? launch_solo(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant, g.split,
-                                  g.ang, (int *)dl.err.p, st)
+                                  g.ang, (int *)dl.err.p, to)
                     : launch_beamform(jobs, prefix, g.count, g.tiles, g.smem, g.prec, g.variant,
-                                      g.rows, g.nf, (int *)dl.err.p, st);
+                                      g.rows, g.nf, (int *)dl.err.p, to);
         if (e != cudaSuccess)
             return cuda_fail(e, "beamform launch");
     }
+    for (int w = 0; w < spread && e == cudaSuccess; ++w) {
+        e = cudaEventRecord(branch->work_join[w], branch->work[w]);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(st, branch->work_join[w], 0);
+    }
+    if (e != cudaSuccess)
+        return cuda_fail(e, "cudaStreamWaitEvent (join)");
     e = mark(2);
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
@@ -1787,6 +1807,13 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
             e = cudaEventCreateWithFlags(&f, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&br.join, cudaEventDisableTiming);
+    if (e == cudaSuccess)
+        e = cudaEventCreateWithFlags(&br.work_fork, cudaEventDisableTiming);
+    for (int w = 0; w < MarkBranch::kWork && e == cudaSuccess; ++w) {
+        e = cudaStreamCreateWithFlags(&br.work[w], cudaStreamNonBlocking);
+        if (e == cudaSuccess)
+            e = cudaEventCreateWithFlags(&br.work_join[w], cudaEventDisableTiming);
+    }
     for (auto &m : b->marks)
         if (e == cudaSuccess)
             e = cudaEventCreate(&m);
@@ -1819,6 +1846,14 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
             cudaEventDestroy(f);
     if (br.join)
         cudaEventDestroy(br.join);
+    if (br.work_fork)
+        cudaEventDestroy(br.work_fork);
+    for (int w = 0; w < MarkBranch::kWork; ++w) {
+        if (br.work_join[w])
+            cudaEventDestroy(br.work_join[w]);
+        if (br.work[w])
+            cudaStreamDestroy(br.work[w]);
+    }
     if (br.side)
         cudaStreamDestroy(br.side);
     if (rc)

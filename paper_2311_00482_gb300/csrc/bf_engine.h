@@ -301,6 +301,11 @@ struct MarkBranch {
     cudaStream_t side = nullptr;
     cudaEvent_t fork[4] = {nullptr, nullptr, nullptr, nullptr};
     cudaEvent_t join = nullptr;
+    // further beamforming launches run beside the first (their CTAs fill the SMs as its
+    // last ones leave): streams to capture them on, forked after the ingest
+    static constexpr int kWork = 3;
+    cudaStream_t work[kWork] = {nullptr, nullptr, nullptr};
+    cudaEvent_t work_fork = nullptr, work_join[kWork] = {nullptr, nullptr, nullptr};
 };
 // marks (optional, 4 events): recorded before the ingest, before and after the
 // beamforming launches, and after the last launch; in line on st, or (branch,
