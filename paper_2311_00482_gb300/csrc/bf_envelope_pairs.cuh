@@ -119,6 +119,9 @@ __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, flo
         }
         f.inverse(v);
         if (it == 0) {  // the band-passed columns kept, their Hilbert spectrum next
+            // the second inverse writes its first level's addresses, which other threads
+            // read in the last level of this one
+            f.sync();
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 const float2 t = lds2(slot + 8u * THREADS * q);

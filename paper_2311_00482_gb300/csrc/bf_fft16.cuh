@@ -12,8 +12,11 @@
 //
 // Between two levels the sixteen values go through shared memory once: every
 // level writes the addresses its thread read, so one barrier per exchange is
-// enough and one buffer serves both directions.  Element p lies at p + p / 16
-// (float2): every level's accesses of a half warp then fall on distinct banks.
+// enough and one buffer serves both directions.  That holds from a transform to
+// the next one, too, if the next runs the other way (it starts at the level the
+// first ended with); two transforms one after the other in the same direction, or
+// anything else stored in the buffer, need a barrier (sync) between them.  Element
+// p lies at p + p / 16 (float2): every level's accesses of a half warp then fall on distinct banks.
 #pragma once
 
 #include <cuda_runtime.h>

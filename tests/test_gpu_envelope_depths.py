@@ -44,3 +44,26 @@ def test_envelope_depth(nz):
     for k in range(2):
         ref = oracle.envelope(y[k], bandpass=k == 1, dz=dz, c=1540.0, f0=5e6)
         assert np.linalg.norm(env[k] - ref) <= 4.4e-6 * np.linalg.norm(y[k])
+
+
+@pytest.mark.parametrize("nz", (300, 800, 1024, 1750, 3000))
+def test_band_passed_envelope_repeats(nz):
+    """The band-passed image takes two inverse transforms one after the other in the same
+    exchange buffer: on a full chip every pass gives the same bits."""
+    import torch
+
+    nx, ne, ns = 2048, 4, 512
+    grid = (nx, nz, -2e-3, 2e-3, 5e-3, 5e-3 + 40e-6 * (nz - 1))
+    rng = np.random.default_rng(nz)
+    rf = torch.from_numpy(rng.integers(-3000, 3000, (1, ne, ns), dtype=np.int16)).cuda()
+    h = bf.bf_create(ne, 0.3e-3, 1.5, grid, 20e6, 5e6, 1540.0)
+    try:
+        env = [torch.full((1, nx, nz), -1.0, device="cuda") for _ in range(30)]
+        torch.cuda.synchronize()
+        for e in env:
+            bf.bf_beamform(h, rf, ns, [0.0], bf.BF_DMAS | bf.BF_OUT_ENV, e)
+        bf.bf_sync(h)
+    finally:
+        bf.bf_destroy(h)
+    for e in env[1:]:
+        assert torch.equal(e, env[0])
