@@ -85,6 +85,15 @@ __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *map, int x,
         : "memory");
 }
 
+// Before the first copy through a tensor map that lies where an earlier launch had
+// another one (the job lists' maps): its descriptor is read again.
+__device__ __forceinline__ void map_acquire(const CUtensorMap *map)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(
+                     reinterpret_cast<uint64_t>(map))
+                 : "memory");
+}
+
 __device__ __forceinline__ float rsqrt_approx(float x)
 {
     float y;

@@ -772,6 +772,7 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
     if (warp == kWarps) {
         // ================= producer warp: TMA copies of every step's stage
         unsigned r = 0;
+        int mapped = -1;  // the job whose map was acquired last
         for (int tg = blockIdx.x; tg < total_tiles; tg += gridDim.x) {
             const unsigned long long deadline = global_ns() + kWaitNs;
             const int jb = find_job(tile_prefix, njobs, tg);
@@ -784,6 +785,9 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
             const int *__restrict__ wtab = J->wtab;
             const int *__restrict__ btab = J->btab;
             const CUtensorMap *rf_map = J->rf_map;
+            if (jb != mapped)
+                map_acquire(rf_map);
+            mapped = jb;
             const CUtensorMap *valid_map = J->valid_map;
             const CUtensorMap *dx2_map = J->dx2_map;
             const int box = J->box;
