@@ -853,10 +853,10 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
                 ij.maxbits_more[q] = g.stage != BF_OUT_RF ? g.maxbits : nullptr;
             }
         }
-        // threads per record row: one per 8 pairs and frame (per frame pair for
-        // FP32 multi-frame jobs)
-        const int units = (f.prec == kPrecF32 && ij.nf > 1) ? ij.nf / 2 : ij.nf;
-        ij.chunks = (units * ((ij.nsp + 7) / 8) + 255) / 256;
+        // nsp is a multiple of 8: units of sixteen bytes, or of eight pairs of a frame pair
+        const bool frames_f32 = f.prec == kPrecF32 && ij.nf > 1;
+        ij.units = ij.nsp / 8 * (frames_f32 ? ij.nf / 2 : ij.nf * pair_bytes(f.prec) / 2);
+        ij.per = 1;
         ig[f.prec].push_back(ij);
     }
     for (auto &kv : ig) {
@@ -865,13 +865,19 @@ int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
         g.first = (int)hl.ingest.size();
         g.count = (int)kv.second.size();
         g.prefix_first = (int)hl.ingest_prefix.size();
+        long long single = 0;
+        for (const IngestJob &j : kv.second)
+            single += ingest_blocks(j);
+        g.wide = single >= kIngestWide;
         int acc = 0;
-        for (const IngestJob &j : kv.second) {
+        for (IngestJob &j : kv.second) {
+            if (g.wide && (j.nf == 1 || g.prec != kPrecF32))
+                j.per = ingest_units(j.nf);
             hl.ingest_prefix.push_back(acc);  // first CTA of the job
-            acc += j.rows * j.chunks;
+            acc += ingest_blocks(j);
             hl.ingest.push_back(j);
         }
-        g.rows = acc;
+        g.blocks = acc;
         hl.igroups.push_back(g);
     }
     long long blks = 0;
@@ -1063,9 +1069,8 @@ int enqueue(const std::vector<FramePrep> &frames, const HostLaunch &hl, DeviceLa
     if (e != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord (mark)");
     for (const HostLaunch::IGroup &g : hl.igroups) {
-        e = launch_ingest(dl.ingest + g.first,
-                          dl.ingest_prefix + g.prefix_first, g.count, g.rows, g.prec,
-                          st);
+        e = launch_ingest(dl.ingest + g.first, dl.ingest_prefix + g.prefix_first, g.count, g.blocks,
+                          g.prec, g.wide, st);
         if (e != cudaSuccess)
             return cuda_fail(e, "ingest launch");
     }

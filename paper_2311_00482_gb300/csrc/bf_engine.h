@@ -142,7 +142,8 @@ struct HostLaunch {
         size_t smem;
     };
     struct IGroup {  // one ingest launch
-        int prec, first, count, prefix_first, rows;  // rows: the launch's CTAs
+        int prec, first, count, prefix_first, blocks;
+        bool wide;  // several units per thread
     };
     std::vector<BfJob> jobs;        // rf_map: index into maps until the upload
     std::vector<CUtensorMap> maps;  // over the jobs' sample pairs

@@ -163,7 +163,7 @@ struct IngestJob {
     // the other frames of a multi-frame beamforming job (nf > 1): their records
     // and maxima; pair j of frame f lands at [row][j][f]
     int nf;
-    int chunks;           // CTAs per record row: nf * nsp / 8 threads of 256 per CTA
+    int units, per;       // units of a row of pairs; per thread
     const int16_t *rf_more[kMaxFramesPerJob - 1];
     unsigned *maxbits_more[kMaxFramesPerJob - 1];
 };
@@ -260,9 +260,16 @@ cudaError_t kernel_setup(const void *k, size_t smem, int threads, bool max_carve
 // (all its jobs must share them, the precision and the rows per thread);
 // BF_PDAS adds the p-th-root combiner.
 cudaError_t launch_plan(const PlanJob &job, int *err_dev, cudaStream_t stream);
-// total_blocks: the jobs' rows x chunks (blk_prefix_dev: each job's first CTA).
+// Records to sample pairs; blk_prefix_dev: each job's first CTA.  wide: launches of so many
+// CTAs (kIngestWide, of one unit per thread: eight of the largest residency) that each thread may
+// take several units, which
+// ingest_units gives for a job of nf frames; in smaller ones that leaves SMs without work
+// (1024 x 1024, 7 angles, FP16, 3591 such CTAs: 9.1 us, 10.9 us with eight units per thread).
+__host__ __device__ constexpr int ingest_units(int nf) { return nf == 1 ? 8 : 4; }
+constexpr int kIngestWide = 8 * 8 * 152;
+int ingest_blocks(const IngestJob &job);
 cudaError_t launch_ingest(const IngestJob *jobs_dev, const int *blk_prefix_dev, int njobs,
-                          int total_blocks, int prec, cudaStream_t stream);
+                          int total_blocks, int prec, bool wide, cudaStream_t stream);
 // Demodulation of records below 32 samples, one row (or frame pair's row) per CTA.
 cudaError_t launch_demod(const DemodJob *jobs_dev, const int *row_prefix_dev, int njobs,
                          int total_rows, cudaStream_t stream);

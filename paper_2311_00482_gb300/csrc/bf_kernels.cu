@@ -95,14 +95,11 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanJob J, int *__restr
 
 // ---------------------------------------------------------------- ingest --
 
-// Pairs j0 .. j0 + 7 of one record row: mid point and difference of samples
-// k = j - kPadL and k + 1 (zero outside the record), FP32 or scaled by 2^-15 to
-// FP16 / BF16 (two 16-bit halves: sample k low, k + 1 high).
+// Pairs j0 .. j0 + 7 of one record row in FP32 (see ingest_kernel).
 // vec: the row starts 16-byte aligned (samples j0 .. j0 + 7 in one 16-byte
 // load, j0 - 2 and j0 - 1 in one 4-byte load when all lie inside the record).
-template <int PREC>
 __device__ __forceinline__ void row_pairs(const int16_t *__restrict__ u, int ns, int j0, bool vec,
-                                          float2 *f, unsigned *h)
+                                          float2 *f)
 {
     static_assert(kPadL == 2, "the vector path loads two samples before j0");
     int s[9];
@@ -122,101 +119,145 @@ __device__ __forceinline__ void row_pairs(const int16_t *__restrict__ u, int ns,
             s[q] = (k >= 0 && k < ns) ? (int)__ldg(u + k) : 0;
         }
     }
-    if (PREC == kPrecF32) {
-        // v = mid + (alpha - 1/2) * diff (exact for int16)
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            f[q] = make_float2(0.5f * (float)(s[q] + s[q + 1]), (float)(s[q + 1] - s[q]));
-    } else {
-        const float sc = 1.0f / 32768.0f;
-        unsigned b[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            if (PREC == kPrecF16)
-                b[q] = __half_as_ushort(__float2half_rn((float)s[q] * sc));
-            else
-                b[q] = __bfloat16_as_ushort(__float2bfloat16_rn((float)s[q] * sc));
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            h[q] = b[q] | (b[q + 1] << 16);
-    }
+    for (int q = 0; q < 8; ++q)
+        f[q] = make_float2(0.5f * (float)(s[q] + s[q + 1]), (float)(s[q + 1] - s[q]));
 }
 
-// Record rows to sample pairs.  A job's CTAs take its rows in order, `chunks`
-// CTAs per row.  nf = 1 writes [row][nsp] (thread g: pairs 8 g .. 8 g + 7).
-// A multi-frame job (nf = 2, 4) writes its frames interleaved per pair index:
-// FP32 as frame pairs, pair j of frames 2q, 2q + 1 at [row][j][q] as
-// (mid_2q, mid_2q+1, diff_2q, diff_2q+1) (thread g: frame pair g % (nf / 2),
-// pairs 8 (g / (nf / 2)) .. + 7); FP16 / BF16 as one 4-byte pair per frame at
-// [row][j][f] (thread g: frame g % nf, pairs 8 (g / nf) .. + 7).
-template <int PREC>
+// Record rows to sample pairs, sixteen output bytes per unit, the units of a job in
+// the order of its pairs array: a warp's stores are contiguous.  A CTA takes J.per units
+// per thread, 256 apart, whose samples are loaded before any is used.  nf = 1 writes
+// [row][nsp]: FP32 two pairs per unit, (mid, diff) each with v = mid + (alpha - 1/2) *
+// diff (exact for int16), FP16 / BF16 four (samples k low and k + 1 high, scaled by
+// 2^-15).  A multi-frame job (nf = 2, 4) writes its frames interleaved per pair index:
+// FP32 as frame pairs, pair j of frames 2q, 2q + 1 at [row][j][q] as (mid_2q,
+// mid_2q+1, diff_2q, diff_2q+1); FP16 / BF16 as one 4-byte pair per frame at
+// [row][j][f].  Pair j holds the samples k = j - kPadL and k + 1, zero outside the
+// record.
+// Bound: memory, mostly the pairs' writes (32 uneven FP32 frames, 50 MB of records to
+// 200 MB of pairs, 79 us with eight pairs per thread, whose stores lay 64 bytes apart;
+// 56 us with four units per thread, 53 us with eight, 85 us with one).  FP32 frame pairs
+// keep eight pairs per thread: a sector is written by two adjacent lanes at once, and
+// one unit's samples come in two loads (64 frames 24.9 -> 24.4 us in CTAs that run on
+// from row to row; 30 us in units of one pair).  64 FP16 frames in fours 25.3 -> 23.6 us.
+// WIDE: several units per thread.
+template <int PREC, bool WIDE>
 __global__ void __launch_bounds__(256) ingest_kernel(const IngestJob *__restrict__ jobs,
                                                      const int *__restrict__ blk_prefix, int njobs)
 {
     dependents_may_start();
     const int jb = find_job(blk_prefix, njobs, blockIdx.x);
-    const IngestJob J = jobs[jb];
+    const IngestJob &J = jobs[jb];
     const int local = blockIdx.x - __ldg(blk_prefix + jb);
-    const int row = local / J.chunks, chunk = local - row * J.chunks;
-    if (row == 0 && chunk == 0 && threadIdx.x < 4) {  // before any later kernel takes a maximum
+    const int nf = J.nf;  // 1, 2 or 4
+    if (local == 0 && threadIdx.x < 4) {  // before any later kernel takes a maximum
         if (J.maxbits)
             J.maxbits[threadIdx.x] = 0u;
-        for (int f = 1; f < J.nf; ++f) {
-            unsigned *m = jobs[jb].maxbits_more[f - 1];
-            if (m)
-                m[threadIdx.x] = 0u;
-        }
+        for (int f = 1; f < nf; ++f)
+            if (J.maxbits_more[f - 1])
+                J.maxbits_more[f - 1][threadIdx.x] = 0u;
     }
-    const int nf = J.nf;  // 1, 2 or 4
-    const int g = chunk * blockDim.x + threadIdx.x;
-    // the other frames' pointers come from the job in global memory: a runtime
-    // index into the local copy J would put it on the stack
-    auto record = [&](int f) { return f == 0 ? J.rf : jobs[jb].rf_more[f - 1]; };
-    auto vec_ok = [&](const int16_t *rf) {
-        return (J.ns & 7) == 0 && (reinterpret_cast<unsigned long long>(rf) & 15) == 0;
-    };
-    float2 fp[8];
-    unsigned hp[8];
-    if (PREC == kPrecF32 && nf > 1) {
-        const int npair = nf / 2;
-        const int q = g % npair, j0 = (g / npair) * 8;
-        if (j0 >= J.nsp)
-            return;
-        float2 fq[8];
-        const int16_t *ra = record(2 * q), *rb = record(2 * q + 1);
-        row_pairs<PREC>(ra + (size_t)row * J.ns, J.ns, j0, vec_ok(ra), fp, hp);
-        row_pairs<PREC>(rb + (size_t)row * J.ns, J.ns, j0, vec_ok(rb), fq, hp);
-        float4 *o = reinterpret_cast<float4 *>(J.pairs) + ((size_t)row * J.nsp + j0) * npair + q;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            o[(size_t)k * npair] = make_float4(fp[k].x, fq[k].x, fp[k].y, fq[k].y);
-        return;
-    }
-    const int f = g & (nf - 1), j0 = (g / nf) * 8;
-    if (j0 >= J.nsp)
-        return;
-    const int16_t *__restrict__ rf = record(f);
-    const int16_t *__restrict__ u = rf + (size_t)row * J.ns;
-    row_pairs<PREC>(u, J.ns, j0, vec_ok(rf), fp, hp);
-    const size_t at = ((size_t)row * J.nsp + j0) * nf + f;  // slot of pair j0
-    if (PREC == kPrecF32) {
-        float2 *o = reinterpret_cast<float2 *>(J.pairs) + at;
-#pragma unroll
-        for (int k = 0; k < 8; k += 2)  // nf == 1: 16-byte stores of two pairs
-            reinterpret_cast<float4 *>(o)[k / 2] =
-                make_float4(fp[k].x, fp[k].y, fp[k + 1].x, fp[k + 1].y);
+    const int ns = J.ns;
+    const unsigned upr = J.units;  // per row
+    const unsigned long long first = (unsigned long long)local * (256u * (unsigned)J.per) + threadIdx.x;
+    unsigned row0, c0;
+    if ((first >> 32) == 0) {
+        row0 = (unsigned)first / upr;
+        c0 = (unsigned)first - row0 * upr;
     } else {
-        unsigned *o = reinterpret_cast<unsigned *>(J.pairs) + at;
-        if (nf == 1) {
-            reinterpret_cast<uint4 *>(o)[0] = make_uint4(hp[0], hp[1], hp[2], hp[3]);
-            reinterpret_cast<uint4 *>(o)[1] = make_uint4(hp[4], hp[5], hp[6], hp[7]);
-        } else {
+        row0 = (unsigned)(first / upr);
+        c0 = (unsigned)(first - (unsigned long long)row0 * upr);
+    }
+    if constexpr (PREC == kPrecF32) {
+        if (nf > 1) {  // one unit: eight pairs of a frame pair
+            const int npair = nf / 2, q = (int)(c0 % (unsigned)npair), j0 = (int)(c0 / (unsigned)npair) * 8;
+            if (row0 >= (unsigned)J.rows)
+                return;
+            float2 fa[8], fb[8];
+            const int16_t *ra = q == 0 ? J.rf : J.rf_more[2 * q - 1], *rb = J.rf_more[2 * q];
+            auto vec_ok = [&](const int16_t *rf) {
+                return (ns & 7) == 0 && (reinterpret_cast<unsigned long long>(rf) & 15) == 0;
+            };
+            row_pairs(ra + (size_t)row0 * ns, ns, j0, vec_ok(ra), fa);
+            row_pairs(rb + (size_t)row0 * ns, ns, j0, vec_ok(rb), fb);
+            float4 *o = reinterpret_cast<float4 *>(J.pairs) + ((size_t)row0 * J.nsp + j0) * npair + q;
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                o[(size_t)k * nf] = hp[k];
+                o[(size_t)k * npair] = make_float4(fa[k].x, fb[k].x, fa[k].y, fb[k].y);
+            return;
         }
     }
+    auto units = [&](auto nf_c) {
+        constexpr int NF = decltype(nf_c)::value;
+        constexpr bool F32 = PREC == kPrecF32;
+        constexpr int FR = F32 ? 1 : NF, NP = F32 ? 2 : 4 / NF;  // frames of a unit, pairs of each
+        constexpr int U = WIDE ? ingest_units(NF) : 1;
+        int s[U][FR][NP + 1];
+        unsigned row = row0, c = c0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c >= upr) {
+                const unsigned q = c / upr;
+                row += q;
+                c -= q * upr;
+            }
+            const bool in = row < (unsigned)J.rows;
+            const int j = (int)c * NP;
+#pragma unroll
+            for (int f = 0; f < FR; ++f) {
+                const int16_t *rec = f == 0 ? J.rf : J.rf_more[f - 1];
+                const int16_t *__restrict__ x = rec + (size_t)row * ns;
+#pragma unroll
+                for (int p = 0; p <= NP; ++p) {
+                    const int k = j - kPadL + p;
+                    s[u][f][p] = in && (unsigned)k < (unsigned)ns ? (int)__ldg(x + k) : 0;
+                }
+            }
+            c += 256;
+        }
+        row = row0, c = c0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c >= upr) {
+                const unsigned q = c / upr;
+                row += q;
+                c -= q * upr;
+            }
+            uint4 o;
+            if constexpr (F32) {
+                const int (&a)[NP + 1] = s[u][0];
+                o = make_uint4(__float_as_uint(0.5f * (float)(a[0] + a[1])),
+                               __float_as_uint((float)(a[1] - a[0])),
+                               __float_as_uint(0.5f * (float)(a[1] + a[2])),
+                               __float_as_uint((float)(a[2] - a[1])));
+            } else {
+                unsigned w[4];
+#pragma unroll
+                for (int f = 0; f < FR; ++f) {
+                    unsigned h[NP + 1];
+#pragma unroll
+                    for (int p = 0; p <= NP; ++p) {
+                        const float x = (float)s[u][f][p] * (1.0f / 32768.0f);
+                        h[p] = PREC == kPrecF16 ? __half_as_ushort(__float2half_rn(x))
+                                                : __bfloat16_as_ushort(__float2bfloat16_rn(x));
+                    }
+#pragma unroll
+                    for (int p = 0; p < NP; ++p)
+                        w[p * NF + f] = h[p] | (h[p + 1] << 16);
+                }
+                o = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            if (row < (unsigned)J.rows)
+                reinterpret_cast<uint4 *>(J.pairs)[(size_t)row * upr + c] = o;
+            c += 256;
+        }
+    };
+    if (PREC == kPrecF32 || nf == 1)
+        units(std::integral_constant<int, 1>());
+    else if (nf == 2)
+        units(std::integral_constant<int, PREC == kPrecF32 ? 1 : 2>());
+    else
+        units(std::integral_constant<int, PREC == kPrecF32 ? 1 : 4>());
 }
 
 // ------------------------------------------------------------- beamform --
@@ -1641,18 +1682,26 @@ cudaError_t launch_plan(const PlanJob &job, int *err_dev, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+int ingest_blocks(const IngestJob &job)
+{
+    const long long per = 256 * job.per;
+    return (int)(((long long)job.rows * job.units + per - 1) / per);
+}
+
 cudaError_t launch_ingest(const IngestJob *jobs_dev, const int *blk_prefix_dev, int njobs,
-                          int total_blocks, int prec, cudaStream_t stream)
+                          int total_blocks, int prec, bool wide, cudaStream_t stream)
 {
     if (njobs <= 0 || total_blocks <= 0)
         return cudaSuccess;
+    auto go = [&](auto k) {
+        k<<<total_blocks, 256, 0, stream>>>(jobs_dev, blk_prefix_dev, njobs);
+        return cudaGetLastError();
+    };
     if (prec == kPrecF32)
-        ingest_kernel<kPrecF32><<<total_blocks, 256, 0, stream>>>(jobs_dev, blk_prefix_dev, njobs);
-    else if (prec == kPrecF16)
-        ingest_kernel<kPrecF16><<<total_blocks, 256, 0, stream>>>(jobs_dev, blk_prefix_dev, njobs);
-    else
-        ingest_kernel<kPrecBF16><<<total_blocks, 256, 0, stream>>>(jobs_dev, blk_prefix_dev, njobs);
-    return cudaGetLastError();
+        return wide ? go(ingest_kernel<kPrecF32, true>) : go(ingest_kernel<kPrecF32, false>);
+    if (prec == kPrecF16)
+        return wide ? go(ingest_kernel<kPrecF16, true>) : go(ingest_kernel<kPrecF16, false>);
+    return wide ? go(ingest_kernel<kPrecBF16, true>) : go(ingest_kernel<kPrecBF16, false>);
 }
 
 cudaError_t launch_demod(const DemodJob *jobs_dev, const int *row_prefix_dev, int njobs,
