@@ -258,39 +258,48 @@ void fk_mapping_tables(int nt, int nk, double pitch, double dz, const std::vecto
     for (int a = 0; a < na; ++a) {
         const double st = sc[2 * a], ct = sc[2 * a + 1];
         const double bet = std::sqrt(1.0 + ct - 0.5 * st * st);  // Stolt: depth scale
-        parallel_for(half, [&](int qi) {
+        auto point = [&](int qi, int p, size_t t) {
             const double Q = (double)(qi + 1);
-            for (int p = 0; p < nk; ++p) {
-                const int m = lgk ? fk_kx_bin(lgk, p) : p;
-                const double X = (double)(m < nk / 2 ? m : m - nk) * r;
-                double pos, w;
-                bool ok;
-                if (!stolt) {
-                    // exact plane-wave mapping k = (Kx^2 + Kz^2) / (2 (Kx sin + Kz cos))
-                    const double den = X * st + Q * ct;
-                    const double num = X * X + Q * Q;
-                    pos = num / den;
-                    w = (Q * den - 0.5 * num * ct) / (den * den);
-                    ok = den > 0.0 && std::fabs(2.0 * X - pos * st) <= pos && pos >= 0.0 &&
-                         pos < (double)half;
-                } else {
-                    // Stolt's mapping of the exploding reflector at velocity c / bet,
-                    // sheared and scaled back onto the native grid
-                    const double Qp = (Q - st * X) / bet;
-                    const double rad = std::sqrt(X * X + Qp * Qp);
-                    pos = (2.0 / bet) * rad;
-                    w = Qp / (bet * bet * rad);
-                    ok = Qp > 0.0 && pos >= 0.0 && pos < (double)half;
-                }
-                if (!ok)
-                    continue;
-                const double fl = std::floor(pos);
-                const size_t t = (size_t)a * npts + (lgk ? (size_t)p * half + qi : (size_t)qi * nk + p);
-                i0[t] = (int)fl;
-                aw[2 * t] = (float)(pos - fl);
-                aw[2 * t + 1] = (float)w;
+            const int m = lgk ? fk_kx_bin(lgk, p) : p;
+            const double X = (double)(m < nk / 2 ? m : m - nk) * r;
+            double pos, w;
+            bool ok;
+            if (!stolt) {
+                // exact plane-wave mapping k = (Kx^2 + Kz^2) / (2 (Kx sin + Kz cos))
+                const double den = X * st + Q * ct;
+                const double num = X * X + Q * Q;
+                pos = num / den;
+                w = (Q * den - 0.5 * num * ct) / (den * den);
+                ok = den > 0.0 && std::fabs(2.0 * X - pos * st) <= pos && pos >= 0.0 &&
+                     pos < (double)half;
+            } else {
+                // Stolt's mapping of the exploding reflector at velocity c / bet,
+                // sheared and scaled back onto the native grid
+                const double Qp = (Q - st * X) / bet;
+                const double rad = std::sqrt(X * X + Qp * Qp);
+                pos = (2.0 / bet) * rad;
+                w = Qp / (bet * bet * rad);
+                ok = Qp > 0.0 && pos >= 0.0 && pos < (double)half;
             }
-        });
+            if (!ok)
+                return;
+            const double fl = std::floor(pos);
+            i0[t] = (int)fl;
+            aw[2 * t] = (float)(pos - fl);
+            aw[2 * t + 1] = (float)w;
+        };
+        // every thread writes rows of its own
+        const size_t base = (size_t)a * npts;
+        if (lgk)
+            parallel_for(nk, [&](int p) {
+                for (int qi = 0; qi < half; ++qi)
+                    point(qi, p, base + (size_t)p * half + qi);
+            });
+        else
+            parallel_for(half, [&](int qi) {
+                for (int p = 0; p < nk; ++p)
+                    point(qi, p, base + (size_t)qi * nk + p);
+            });
     }
 }
 
