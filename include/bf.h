@@ -355,7 +355,8 @@ BF_API int bf_host_tables(const bf_geometry *geometry, const bf_grid *grid, doub
  * staged pair of every (angle, tile, channel) window, INT32_MIN when no pixel
  * of the tile counts that channel.  Pair j of a record holds samples j - 2
  * and j - 1.  Tiles are 32 columns wide and 8 * rows deep, numbered across
- * first. */
+ * first.  These are the tiles of frames that share their plan with others; an RF
+ * frame that shares it with none may run on tiles of its own. */
 BF_API int bf_plan_info(bf_handle *h, int32_t n_samples, const double *angles_rad,
                         int32_t n_angles, uint32_t mode_and_flags, int32_t *info8, int32_t *wtab,
                         size_t wtab_entries);

@@ -21,8 +21,8 @@ LIB = os.path.join(HERE, "libbf.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["bf_kernels.cu", "bf_solo.cu", "bf_solo_f16.cu", "bf_solo_bf16.cu", "bf_envelope.cu", "bf_demod.cu", "bf_fk.cu",
-              "bf_static.cu"]
+CU_SOURCES = ["bf_kernels.cu", "bf_solo.cu", "bf_solo_f16.cu", "bf_solo_bf16.cu", "bf_envelope.cu",
+              "bf_demod.cu", "bf_fk.cu", "bf_static.cu"]
 CPP_SOURCES = ["bf_api.cpp", "bf_engine.cpp", "bf_tables.cpp"]
 
 

@@ -257,8 +257,9 @@ static PlanKey tuned_key(PlanKey k)
 // Configuration of a workload (of kTileConfigs, or a solo one): BF_TILE_ROWS, else
 // what bf_autotune measured fastest for it, else by the frames that share it.
 // Beamforming time per 512 x 512 frame, 32 frames in a batch, DAS + DMAS of one
-// angle / DMAS of three: alone (solo) 13.7 / 22.3 us, in pairs on 32-row tiles 7.4 /
-// 21.0 us, in fours on 16-row tiles 5.9 / 16.2 us.
+// angle / DMAS of three: alone (solo, measured before its one-angle registers, which
+// take a lone frame of one angle from 24.9 to 18.7 us) 13.7 / 22.3 us, in pairs on
+// 32-row tiles 7.4 / 21.0 us, in fours on 16-row tiles 5.9 / 16.2 us.
 static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w, bool narrow_ok)
 {
     const int forced = forced_cfg();

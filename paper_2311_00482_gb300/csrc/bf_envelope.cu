@@ -384,7 +384,8 @@ static cudaError_t launch_envelope_t(const EnvJob *jobs_dev, const int *blk_pref
         if (e != cudaSuccess)
             return e;
     }
-    return launch_kernel(envelope_kernel<BIG>, dim3((unsigned)total_blocks), threads, smem, dependent, stream, jobs_dev, blk_prefix_dev, njobs);
+    return launch_kernel(envelope_kernel<BIG>, dim3((unsigned)total_blocks), threads, smem, dependent,
+                         stream, jobs_dev, blk_prefix_dev, njobs);
 }
 
 cudaError_t launch_envelope(const EnvJob *jobs_dev, const int *blk_prefix_dev, int njobs,

@@ -62,8 +62,8 @@ __device__ __forceinline__ float magnitude(float q, float a, float b)
 // inverse's 1 / M in them: one forward transform and one inverse, or two for the
 // band-passed image, serve two columns.  (Bluestein's four transforms per single
 // column, which this replaced: 39.4 us of a 64 x 1750 image's pass, 732 us of the
-// pass of 32 uneven images of 64-1024 rows; measured now by the whole passes,
-// 47.7 -> 30.7 us and 3345 -> 2712 us.)  Bound: latency of the exchanges at small
+// pass of 32 uneven images of 64-1024 rows; by the whole passes 47.7 -> 30.7 us
+// and 3345 -> 2712 us.)  Bound: latency of the exchanges at small
 // image counts, shared-memory traffic and FP32 issue about equally at large ones.
 template <int LG, bool CONV, int THREADS, bool TAB_SHARED, class Factors>
 __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, float *__restrict__ env,

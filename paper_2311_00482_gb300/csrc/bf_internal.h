@@ -260,11 +260,11 @@ cudaError_t kernel_setup(const void *k, size_t smem, int threads, bool max_carve
 // (all its jobs must share them, the precision and the rows per thread);
 // BF_PDAS adds the p-th-root combiner.
 cudaError_t launch_plan(const PlanJob &job, int *err_dev, cudaStream_t stream);
-// Records to sample pairs; blk_prefix_dev: each job's first CTA.  wide: launches of so many
-// CTAs (kIngestWide, of one unit per thread: eight of the largest residency) that each thread may
-// take several units, which
-// ingest_units gives for a job of nf frames; in smaller ones that leaves SMs without work
-// (1024 x 1024, 7 angles, FP16, 3591 such CTAs: 9.1 us, 10.9 us with eight units per thread).
+// Records to sample pairs; blk_prefix_dev: each job's first CTA.  wide: launches of so
+// many CTAs (kIngestWide, of one unit per thread: eight of the largest residency) that
+// each thread may take several units, which ingest_units gives for a job of nf frames; in
+// smaller ones that leaves SMs without work (1024 x 1024, 7 angles, FP16, 3591 such CTAs:
+// 9.1 us, 10.9 us with eight units per thread).
 __host__ __device__ constexpr int ingest_units(int nf) { return nf == 1 ? 8 : 4; }
 constexpr int kIngestWide = 8 * 8 * 152;
 int ingest_blocks(const IngestJob &job);

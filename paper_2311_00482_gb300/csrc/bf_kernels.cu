@@ -11,7 +11,7 @@
 //                    consumer warp, `ROWS` contiguous rows per thread).  Per
 //                    angle and channel group a producer warp has the tensor
 //                    memory accelerator (cp.async.bulk.tensor) copy, into a
-//                    3-stage shared-memory ring tracked by mbarriers, the
+//                    shared-memory ring tracked by mbarriers, the
 //                    group's window of every channel's record plus the tile's
 //                    per-(channel, column) tables; delays are formed in
 //                    registers, samples interpolated linearly and combined
@@ -20,7 +20,8 @@
 //                    frames of one plan (their pairs interleaved by frame):
 //                    every delay (and for IQ-DAS / BB-DMAS, Eq. (4), the
 //                    carrier phase) serves all of them, and a storer warp
-//                    writes the staged tile images with bulk copies
+//                    writes the staged tile images with bulk copies.  (RF
+//                    frames that share their plan with no other: bf_solo.cuh)
 //   log_kernel       20 log10(env / max) clipped to the -70 dB range of Fig. 3
 #include <limits.h>
 
@@ -1421,6 +1422,8 @@ __global__ void __launch_bounds__(256) plain_kernel(const BfJob J, const int16_t
 
 // ------------------------------------------------------------ f-k migration --
 
+// Transforms of fewer than 32 points along time or across the elements only; bf_fk.cu
+// has the others.
 // Per channel record: transform along time (zero-padded to nt), then the
 // transmit's lateral delay removed per bin, written to D[a][b][i].
 __global__ void __launch_bounds__(256) fk_time_kernel(const FkJob J)
@@ -1796,12 +1799,14 @@ cudaError_t launch_log(const LogJob *jobs_dev, const int *blk_prefix_dev, int nj
     // programmatic stream serialization: the blocks may be scheduled before the
     // envelope kernel ends (the kernel's griddepcontrol.wait orders the reads),
     // which hides this launch behind that kernel's last CTAs
-    return launch_kernel(log_kernel, dim3((unsigned)total_blocks), 256, 0, true, stream, jobs_dev, blk_prefix_dev, njobs, dynamic_range_db);
+    return launch_kernel(log_kernel, dim3((unsigned)total_blocks), 256, 0, true, stream, jobs_dev,
+                         blk_prefix_dev, njobs, dynamic_range_db);
 }
 
 cudaError_t launch_log_one(const LogJob &job, float dynamic_range_db, cudaStream_t stream)
 {
-    return launch_kernel(log_one_kernel, dim3((unsigned)log_blocks(job.n)), 256, 0, true, stream, job, dynamic_range_db);
+    return launch_kernel(log_one_kernel, dim3((unsigned)log_blocks(job.n)), 256, 0, true, stream, job,
+                         dynamic_range_db);
 }
 
 int log_blocks(long long pixels) { return (int)((pixels + kLogPerBlock - 1) / kLogPerBlock); }

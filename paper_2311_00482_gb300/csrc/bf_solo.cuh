@@ -17,13 +17,17 @@
 // tiles run with SPLIT = 2 or 4: that many times the tiles, each with fewer
 // channels per warp, so a small image still fills the chip.
 //
-// Bound: FP32 / integer issue (62-64 % of the issue slots, 15.5 instructions per
-// active (pixel, channel, angle) for DAS and 18.2 for DMAS of 1-11 angles, 19.9 and
-// 24.3 before) and, between a sample's address and its value, shared-memory latency.
+// Bound: latency, with no unit saturated: 15.5 instructions per active (pixel, channel,
+// angle) for DAS and 18.2 for DMAS of 1-11 angles (19.9 and 24.3 before) fill 59-63 % of
+// the issue slots, the FMA pipe 42-46 %, special functions 33 % (DAS) to 54 % (DMAS),
+// shared memory 34-45 %, with 23-24 warps per SM.  Scalar instead of paired sums (13 %
+// more instructions), or the receive distance as a polynomial without special functions,
+// take the same time or longer.
 // Measured against the tiles of beamform_kernel that these frames used: whole passes
-// of 32 uneven frames 2712 -> 1844 us, of one 1024 x 1024 x 128 x 7-angle frame with
-// DAS + DMAS + CF in FP16 403 -> 270 us, of a 300 x 384 pDAS frame 73.8 -> 45.6 us;
-// a 512 x 512 frame of one angle 22.1 -> 18.7 us of beamforming.
+// of 32 uneven frames 2712 -> 1844 us (1659 with the launches side by side and the ingest
+// of today), of one 1024 x 1024 x 128 x 7-angle frame with DAS + DMAS + CF in FP16
+// 403 -> 272 us, of a 300 x 384 pDAS frame 73.8 -> 45.6 us (43.1 with dependent
+// launches); a 512 x 512 frame of one angle 22.1 -> 18.7 us of beamforming.
 #pragma once
 
 #include <limits.h>
@@ -629,7 +633,8 @@ cudaError_t launch_t(const BfJob *jobs, const int *prefix, int njobs, int tiles,
         if (e != cudaSuccess)
             return e;
     }
-    return launch_kernel(k, dim3((unsigned)grid), kThreads + 32, smem, dependent, st, jobs, prefix, njobs, tiles, stride, err);
+    return launch_kernel(k, dim3((unsigned)grid), kThreads + 32, smem, dependent, st, jobs, prefix, njobs,
+                         tiles, stride, err);
 }
 
 template <int PREC, int SPLIT, int NA>
