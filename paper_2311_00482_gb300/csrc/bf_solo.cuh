@@ -24,9 +24,9 @@
 // more instructions), or the receive distance as a polynomial without special functions,
 // take the same time or longer.
 // Measured against the tiles of beamform_kernel that these frames used: whole passes
-// of 32 uneven frames 2712 -> 1844 us (1659 with the launches side by side and the ingest
+// of 32 uneven frames 2712 -> 1844 us (1647 with the launches side by side and the ingest
 // of today), of one 1024 x 1024 x 128 x 7-angle frame with DAS + DMAS + CF in FP16
-// 403 -> 272 us, of a 300 x 384 pDAS frame 73.8 -> 45.6 us (43.1 with dependent
+// 403 -> 260 us, of a 300 x 384 pDAS frame 73.8 -> 45.6 us (43.1 with dependent
 // launches); a 512 x 512 frame of one angle 22.1 -> 18.7 us of beamforming.
 #pragma once
 
@@ -61,11 +61,11 @@ struct SoloHeader {
 };
 constexpr int kSoloHeaderBytes = (int)(sizeof(SoloHeader) + 127) / 128 * 128;
 
-// Sums a warp hands to the others of its row pair: per angle T1, T2 (DMAS) and P1
-// (pDAS); S1 and the squares (CF).  Row pairs, one per lane.
+// Sums a warp hands to the others of its row pair: per angle T1 (DMAS) and P1 (pDAS);
+// T2 (DMAS), S1 and the squares (CF).  Row pairs, one per lane.
 __host__ __device__ constexpr int solo_sums(int na, bool dmas, bool cf, bool pdas)
 {
-    return na * ((dmas ? 2 : 0) + (pdas ? 1 : 0)) + 1 + (cf ? 1 : 0);
+    return na * ((dmas ? 1 : 0) + (pdas ? 1 : 0)) + (dmas ? 1 : 0) + 1 + (cf ? 1 : 0);
 }
 __host__ __device__ constexpr int solo_exchange_bytes(int split, int na, bool dmas, bool cf, bool pdas)
 {
@@ -130,7 +130,8 @@ struct SoloAcc {
     // sample pair's address
     f32x2_t M[NA];
     f32x2_t S1, Su2;
-    f32x2_t T1[NA], T2[NA], P1[NA];
+    f32x2_t T1[NA], P1[NA];
+    f32x2_t T2;  // of all the group's angles, which only enter the image as their sum
     f32x2_t Yd, Yp;
 };
 
@@ -162,6 +163,7 @@ __device__ __forceinline__ void solo_channels(SoloAcc<NA> &A, const int4 (&E)[NC
         upk2(add2(r, A.Z), a, b);
         const f32x2_t R = pk2(rcp_approx(a), rcp_approx(b));
         const int ent[4] = {E[c].x, E[c].y, E[c].z, E[c].w};
+        f32x2_t squares = 0;
 #pragma unroll
         for (int k = 0; k < AN; ++k) {
             const f32x2_t x = fma2(D2, R, A.F[k]);
@@ -186,25 +188,31 @@ __device__ __forceinline__ void solo_channels(SoloAcc<NA> &A, const int4 (&E)[NC
                 const f32x2_t q = pk2(copysignf(sqrt_approx(fabsf(v0)), v0),
                                       copysignf(sqrt_approx(fabsf(v1)), v1));
                 A.T1[k] = add2(A.T1[k], q);
-                A.T2[k] = fma2(q, q, A.T2[k]);
+                // a channel's angles first, so that T2 is no longer a sum than per angle
+                squares = AN == 1 ? fma2(q, q, A.T2) : k == 0 ? mul2(q, q) : fma2(q, q, squares);
             }
             if (CF)
                 A.Su2 = fma2(v, v, A.Su2);
             if (PDAS)
                 A.P1[k] = add2(A.P1[k], pk2(pdas_root(v0, inv_p, square), pdas_root(v1, inv_p, square)));
         }
+        if (DMAS)
+            A.T2 = AN == 1 ? squares : add2(A.T2, squares);
     }
 }
 
 // Resident CTAs per SM the register budget is sized for.  (One angle, 512 x 512 DAS +
 // DMAS: 19.5 / 18.7 / 20.7 us at two / three / four; while these jobs ran with the
-// registers of four angles, which spilled at three, 24.9.)
+// registers of four angles, which spilled at three, 24.9.  1024 x 1024 x 128 elements, 7
+// angles, DAS + DMAS + CF in FP16, whole pass: 269.5 us at two, 259.5 at three; with a T2
+// per angle, which left room for two only, 272.  32 uneven frames 1667 us at two
+// throughout, 1647 now, 1660 with a T2 per angle.)
 template <bool DMAS, bool CF, bool PDAS, int NA>
 constexpr int solo_min_blocks()
 {
     if (NA == 1)
         return 3;
-    return (PDAS && (DMAS || CF)) || (DMAS && CF) ? 2 : 3;
+    return PDAS && (DMAS || CF) ? 2 : 3;
 }
 
 // NA: angles of a stage, 1 (jobs of one angle) or kSoloAngles.
@@ -380,10 +388,10 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                        wstep = (uint32_t)G * wbytes;
         const f32x2_t zero2 = pk2(0.f, 0.f);
         SoloAcc<NA> A;
-        A.Z = A.S1 = A.Su2 = A.Yd = A.Yp = zero2;
+        A.Z = A.S1 = A.T2 = A.Su2 = A.Yd = A.Yp = zero2;
 #pragma unroll
         for (int k = 0; k < NA; ++k) {
-            A.F[k] = A.M[k] = A.T1[k] = A.T2[k] = A.P1[k] = zero2;
+            A.F[k] = A.M[k] = A.T1[k] = A.P1[k] = zero2;
         }
         bool dead = false;
         int g = 0, ag = 0;
@@ -398,6 +406,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                 return;  // warp-uniform: a bounded wait ran out (error bit set)
             if (!dead) {
                 if (g == 0) {  // the angle group's delay tables
+                    A.T2 = zero2;
                     A.Z = pk2(sh.tZ[st][2 * band], sh.tZ[st][2 * band + 1]);
 #pragma unroll
                     for (int k = 0; k < NA; ++k)
@@ -408,7 +417,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                             const float *tf = &sh.tF[st][k][kTileCols + 2 * band];
                             A.M[k] = pk2(__int_as_float(ck + tk[0]), __int_as_float(ck + tk[1]));
                             A.F[k] = pk2(cf + tf[0] - 0.5f, cf + tf[1] - 0.5f);
-                            A.T1[k] = A.T2[k] = A.P1[k] = zero2;
+                            A.T1[k] = A.P1[k] = zero2;
                         }
                 }
                 const uint32_t base = smem_u32(stage_base(st));
@@ -513,13 +522,13 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                         };
 #pragma unroll
                         for (int k = 0; k < NA; ++k) {
-                            if (DMAS) {
+                            if (DMAS)
                                 put(A.T1[k]);
-                                put(A.T2[k]);
-                            }
                             if (PDAS)
                                 put(A.P1[k]);
                         }
+                        if (DMAS)
+                            put(A.T2);
                         put(A.S1);
                         if (CF)
                             put(A.Su2);
@@ -537,13 +546,13 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                             };
 #pragma unroll
                             for (int k = 0; k < NA; ++k) {
-                                if (DMAS) {
+                                if (DMAS)
                                     get(A.T1[k]);
-                                    get(A.T2[k]);
-                                }
                                 if (PDAS)
                                     get(A.P1[k]);
                             }
+                            if (DMAS)
+                                get(A.T2);
                             if (last) {
                                 get(A.S1);
                                 if (CF)
@@ -555,11 +564,11 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
                 }
             }
             if (DMAS) {
+                A.Yd = fma2(pk2(-0.5f, -0.5f), A.T2, A.Yd);
 #pragma unroll
                 for (int k = 0; k < NA; ++k)
                     if (k < an)
-                        A.Yd = fma2(mul2(pk2(0.5f, 0.5f), A.T1[k]), A.T1[k],
-                                    fma2(pk2(-0.5f, -0.5f), A.T2[k], A.Yd));
+                        A.Yd = fma2(mul2(pk2(0.5f, 0.5f), A.T1[k]), A.T1[k], A.Yd);
             }
             if (PDAS) {  // Eq. (3) per angle, then the coherent sum
 #pragma unroll
