@@ -18,9 +18,9 @@
 // channels per warp, so a small image still fills the chip.
 //
 // Bound: latency, with no unit saturated: 15.5 instructions per active (pixel, channel,
-// angle) for DAS and 18.2 for DMAS of 1-11 angles (19.9 and 24.3 before) fill 59-63 % of
-// the issue slots, the FMA pipe 42-46 %, special functions 33 % (DAS) to 54 % (DMAS),
-// shared memory 34-45 %, with 23-24 warps per SM.  Scalar instead of paired sums (13 %
+// angle) for DAS and 18.2 for DMAS of 1-11 angles (19.9 and 24.3 before) fill 59-65 % of
+// the issue slots, the FMA pipe 42-48 %, special functions 33 % (DAS) to 55 % (DMAS),
+// shared memory 19-45 %, with 23-24 warps per SM.  Scalar instead of paired sums (13 %
 // more instructions), or the receive distance as a polynomial without special functions,
 // take the same time or longer.
 // Measured against the tiles of beamform_kernel that these frames used: whole passes
