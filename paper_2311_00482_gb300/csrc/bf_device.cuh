@@ -85,13 +85,21 @@ __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *map, int x,
         : "memory");
 }
 
-// Before the first copy through a tensor map that lies where an earlier launch had
-// another one (the job lists' maps): its descriptor is read again.
+// Before a job's first copies: a tensor map in global memory may lie where an earlier
+// launch had another one (the job lists are rewritten, and a plan's maps may get the
+// address of a destroyed handle's), so its descriptor is read again.
 __device__ __forceinline__ void map_acquire(const CUtensorMap *map)
 {
     asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(
                      reinterpret_cast<uint64_t>(map))
                  : "memory");
+}
+
+__device__ __forceinline__ void maps_acquire(const BfJob *J)
+{
+    map_acquire(J->rf_map);
+    map_acquire(J->valid_map);
+    map_acquire(J->dx2_map);
 }
 
 __device__ __forceinline__ float rsqrt_approx(float x)

@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
     if (warp == kWarps) {
         // ================= producer warp: TMA copies of every step's stage
         unsigned r = 0;
-        int mapped = -1;  // the job whose map was acquired last
+        int mapped = -1;  // the job whose maps were acquired last
         for (int tg = blockIdx.x; tg < total_tiles; tg += gridDim.x) {
             const unsigned long long deadline = global_ns() + kWaitNs;
             const int jb = find_job(tile_prefix, njobs, tg);
@@ -827,11 +827,11 @@ __global__ void __launch_bounds__(beamform_threads<NF>(),
             const int *__restrict__ wtab = J->wtab;
             const int *__restrict__ btab = J->btab;
             const CUtensorMap *rf_map = J->rf_map;
-            if (jb != mapped)
-                map_acquire(rf_map);
-            mapped = jb;
             const CUtensorMap *valid_map = J->valid_map;
             const CUtensorMap *dx2_map = J->dx2_map;
+            if (jb != mapped)
+                maps_acquire(J);
+            mapped = jb;
             const int box = J->box;
             const unsigned meta_bytes = (unsigned)G * kTileCols * 8;
             // window start and band flags of this lane's channel at step s

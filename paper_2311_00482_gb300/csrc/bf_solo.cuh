@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
         // (up to four) adjacent channels, which start at the same pair.
         wait_for_producer();  // the staged pairs (and the deadlines start here)
         unsigned r = 0;
-        int mapped = -1;  // the job whose map was acquired last
+        int mapped = -1;  // the job whose maps were acquired last
         for (int tg = blockIdx.x; tg < total_tiles; tg += gridDim.x) {
             const unsigned long long deadline = global_ns() + kWaitNs;
             const int jb = find_job(tile_prefix, njobs, tg);
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kThreads + 32, (solo_min_blocks<DMAS, CF, PDAS
             const int amax = (na + ngr - 1) / ngr, box = J->box, run = J->run;
             const CUtensorMap *rf_map = J->rf_map;
             if (jb != mapped)
-                map_acquire(rf_map);
+                maps_acquire(J);
             mapped = jb;
             // this lane's run of channels and angle, its word of the step's record
             const int runs = G / run, kq = lane / runs, cq = lane - kq * runs;
