@@ -1755,13 +1755,12 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
 
 // ------------------------------------------------------------------ batch --
 
-// Whether two frames of a batch can share a beamforming job (see shareable).
-static bool same_job(const bf_frame &a, const bf_frame &b)
+// What frames of a batch have in common that can share a beamforming job (see shareable).
+using JobKey = std::tuple<const bf_handle *, int, uint32_t, std::vector<double>>;
+static JobKey job_key(const bf_frame &f)
 {
-    const uint32_t m = BF_MODE_MASK | BF_IQ_MASK | BF_PREC_MASK;
-    return a.h == b.h && a.n_samples == b.n_samples && a.n_angles == b.n_angles &&
-           (a.mode_and_flags & m) == (b.mode_and_flags & m) && a.n_angles > 0 && a.angles_rad &&
-           b.angles_rad && std::equal(a.angles_rad, a.angles_rad + a.n_angles, b.angles_rad);
+    return JobKey(f.h, f.n_samples, f.mode_and_flags & (BF_MODE_MASK | BF_IQ_MASK | BF_PREC_MASK),
+                  std::vector<double>(f.angles_rad, f.angles_rad + f.n_angles));
 }
 
 BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
@@ -1772,6 +1771,9 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
     auto b = std::make_unique<bf_batch>();
     b->scratch.resize(n);
     b->frames.resize(n);
+    // frames of the batch with the same plan and combiners; every frame's arguments are
+    // checked before its angles are read
+    std::map<JobKey, int> peers;
     int dev = -1;
     for (int i = 0; i < n; ++i) {
         const bf_frame &f = frames[i];
@@ -1784,12 +1786,17 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
         cudaSetDevice(dev);
         if (!is_device_pointer(f.rf_dev) || !is_device_pointer(f.out_dev))
             return fail(BF_EINVAL, "frame %d: batches need device pointers", i);
-        int peers = 0;  // frames of the batch with the same plan and combiners
-        for (int j = 0; j < n; ++j)
-            peers += same_job(f, frames[j]) ? 1 : 0;
+        int rc = check_frame_args(f.h, f.n_samples, f.angles_rad, f.n_angles, f.mode_and_flags);
+        if (rc)
+            return fail(rc, "frame %d: %s", i, g_err.c_str());
+        peers[job_key(f)] += 1;
+    }
+    for (int i = 0; i < n; ++i) {
+        const bf_frame &f = frames[i];
+        const int same = peers[job_key(f)];
         int rc = prepare_frame(f.h, f.rf_dev, f.n_samples, f.angles_rad, f.n_angles,
                                f.mode_and_flags, f.out_dev, b->scratch[i], b->frames[i],
-                               peers > 1 ? kMaxFramesPerJob : 1, PlanWish{-1, peers});
+                               same > 1 ? kMaxFramesPerJob : 1, PlanWish{-1, same});
         if (rc)
             return fail(rc, "frame %d: %s", i, g_err.c_str());
     }
