@@ -46,9 +46,14 @@ struct MaskFactors {
 // Magnitude where the sum of squares leaves the range it can be formed in.
 __device__ __noinline__ float hypot_far(float a, float b) { return hypotf(a, b); }
 
+// The root of the sum of squares: the special-function unit's reciprocal root and one
+// Newton step with the residual in a fused multiply-add, about half a unit in the last place.
 __device__ __forceinline__ float magnitude(float q, float a, float b)
 {
-    return (q > 1e-36f && q < 3e38f) ? sqrt_fast(q) : hypot_far(a, b);
+    if (!(q > 1e-36f && q < 3e38f))
+        return hypot_far(a, b);
+    const float y = rsqrtf(q), s = q * y;
+    return fmaf(fmaf(-s, s, q), 0.5f * y, s);
 }
 
 // Envelopes of the column pairs pair0, pair0 + 1, ... of one image, one pair per
