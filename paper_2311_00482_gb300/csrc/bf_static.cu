@@ -153,11 +153,11 @@ __global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict
 #pragma unroll
     for (int w = 0; w < 8; ++w)
         peak = fmaxf(peak, red[w]);
-    // 20 log10(e / peak) = (20 log10 2) (log2 e - log2 peak), as log_kernel
-    const float lp = peak > 0.f ? __log2f(peak) : 0.f;
+    // of the quotient, so that the image's scale cancels exactly and images of any scale
+    // lose nothing (a difference of two fast logarithms: 1e-5 dB at a scale of one, 1e-4 dB
+    // at 2^-100)
     auto db = [&](float e) {
-        return (e > 0.f && peak > 0.f) ? fminf(fmaxf(6.0205999132796239f * (__log2f(e) - lp), -dr), 0.f)
-                                       : -dr;
+        return (e > 0.f && peak > 0.f) ? fminf(fmaxf(20.f * log10f(e / peak), -dr), 0.f) : -dr;
     };
     const int base = blockIdx.x * kStaticLogPixels;
     if (vec4) {
