@@ -38,6 +38,17 @@ static __device__ __constant__ float2 kW32[16] = {
     {-7.071067812e-01f, 7.071067812e-01f}, {-8.314696123e-01f, 5.555702330e-01f},
     {-9.238795325e-01f, 3.826834324e-01f}, {-9.807852804e-01f, 1.950903220e-01f}};
 
+// What rounding took from them.
+static __device__ __constant__ float2 kW32Lo[16] = {
+    {0.000000000e+00f, 0.000000000e+00f}, {2.973947311e-08f, -1.670471539e-09f},
+    {2.830748969e-08f, 6.223350724e-09f}, {1.687026341e-08f, -1.176952136e-08f},
+    {1.210161749e-08f, 1.210161749e-08f}, {-1.176952136e-08f, 1.687026341e-08f},
+    {6.223350724e-09f, 2.830748969e-08f}, {-1.670471428e-09f, 2.973947311e-08f},
+    {0.000000000e+00f, 0.000000000e+00f}, {1.670471539e-09f, 2.973947311e-08f},
+    {-6.223350724e-09f, 2.830748969e-08f}, {1.176952136e-08f, 1.687026341e-08f},
+    {-1.210161749e-08f, 1.210161749e-08f}, {-1.687026341e-08f, -1.176952136e-08f},
+    {-2.830748969e-08f, 6.223351168e-09f}, {-2.973947311e-08f, -1.670471095e-09f}};
+
 // Complex add / subtract as one paired FP32 instruction (Blackwell f32x2):
 // the real and imaginary parts of a float2 sit in a register pair.
 static __device__ __forceinline__ float2 c_add(float2 a, float2 b)
@@ -97,9 +108,19 @@ static __device__ __forceinline__ float2 c_sfma(float s, float2 a, float2 b)
     return c;
 }
 
+// a * (w + l): a twiddle in two parts, w rounded to FP32 and l what the rounding took.
+// The rounding of the twiddles is half of a transform's error; with l the product keeps
+// only its own.
+static __device__ __forceinline__ float2 cmul_fine(float2 a, float2 w, float2 l)
+{
+    const float cr = fmaf(a.x, l.x, -a.y * l.y), ci = fmaf(a.x, l.y, a.y * l.x);
+    return make_float2(fmaf(a.x, w.x, fmaf(-a.y, w.y, cr)), fmaf(a.x, w.y, fmaf(a.y, w.x, ci)));
+}
+
 // b * W_32^e (INV: conjugate), W_32 = exp(-2 pi i / 32), 0 <= e < 32; e is a
-// compile-time constant wherever this is used (quarter turns are swaps).
-template <bool INV>
+// compile-time constant wherever this is used (quarter turns are swaps).  FINE: the
+// factor in two parts.
+template <bool INV, bool FINE = false>
 static __device__ __forceinline__ float2 w32mul(float2 b, int e)
 {
     if (e >= 16) {  // W_32^16 = -1
@@ -112,6 +133,9 @@ static __device__ __forceinline__ float2 w32mul(float2 b, int e)
         return INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
     const float2 w = kW32[e];
     const float s = INV ? w.y : -w.y;
+    if constexpr (FINE)
+        return cmul_fine(b, make_float2(w.x, s),
+                         make_float2(kW32Lo[e].x, INV ? kW32Lo[e].y : -kW32Lo[e].y));
     return make_float2(b.x * w.x - b.y * s, b.x * s + b.y * w.x);
 }
 
@@ -146,7 +170,7 @@ static __device__ __forceinline__ void dft4_half(float2 &a, float2 &b, float2 &c
 // W_16^(n k) (INV: conjugate exponent, no scaling), as 4 x 4 with n = n1 + 4 n2
 // and k = 4 k1 + k2: DFTs over n2, twiddles W_16^(n1 k2), DFTs over n1, and a
 // transposed read-out (register renaming only).  HALF: x[8 .. 15] are zero.
-template <bool INV, bool HALF = false>
+template <bool INV, bool HALF = false, bool FINE = false>
 static __device__ __forceinline__ void dft16(float2 (&x)[16])
 {
     if constexpr (HALF) {
@@ -161,15 +185,15 @@ static __device__ __forceinline__ void dft16(float2 (&x)[16])
         dft4<INV>(x[2], x[6], x[10], x[14]);
         dft4<INV>(x[3], x[7], x[11], x[15]);
     }
-    x[5] = w32mul<INV>(x[5], 2);  // W_16^(n1 k2) = W_32^(2 n1 k2)
-    x[9] = w32mul<INV>(x[9], 4);
-    x[13] = w32mul<INV>(x[13], 6);
-    x[6] = w32mul<INV>(x[6], 4);
-    x[10] = w32mul<INV>(x[10], 8);
-    x[14] = w32mul<INV>(x[14], 12);
-    x[7] = w32mul<INV>(x[7], 6);
-    x[11] = w32mul<INV>(x[11], 12);
-    x[15] = w32mul<INV>(x[15], 18);
+    x[5] = w32mul<INV, FINE>(x[5], 2);  // W_16^(n1 k2) = W_32^(2 n1 k2)
+    x[9] = w32mul<INV, FINE>(x[9], 4);
+    x[13] = w32mul<INV, FINE>(x[13], 6);
+    x[6] = w32mul<INV, FINE>(x[6], 4);
+    x[10] = w32mul<INV, FINE>(x[10], 8);
+    x[14] = w32mul<INV, FINE>(x[14], 12);
+    x[7] = w32mul<INV, FINE>(x[7], 6);
+    x[11] = w32mul<INV, FINE>(x[11], 12);
+    x[15] = w32mul<INV, FINE>(x[15], 18);
     dft4<INV>(x[0], x[1], x[2], x[3]);  // -> X[4 k1 + k2] at 4 k2 + k1
     dft4<INV>(x[4], x[5], x[6], x[7]);
     dft4<INV>(x[8], x[9], x[10], x[11]);
@@ -184,7 +208,7 @@ static __device__ __forceinline__ void dft16(float2 (&x)[16])
 }
 
 // R-point DFTs (R = 2, 4, 8) of consecutive registers, natural order in and out.
-template <int R, bool INV>
+template <int R, bool INV, bool FINE>
 static __device__ __forceinline__ void dft_runs(float2 (&v)[16])
 {
 #pragma unroll
@@ -202,7 +226,7 @@ static __device__ __forceinline__ void dft_runs(float2 (&v)[16])
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 e[k] = v[s + 2 * k];
-                o[k] = w32mul<INV>(v[s + 2 * k + 1], 4 * k);
+                o[k] = w32mul<INV, FINE>(v[s + 2 * k + 1], 4 * k);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -233,36 +257,10 @@ static __device__ __forceinline__ void sts2(uint32_t a, float2 v)
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
-// Shared-memory twiddles of one length: level L's entries start here, after those of
-// the levels above it; fft16_tab_shared(lg, below the last level) is their number.
-__host__ __device__ constexpr int fft16_tab_shared(int lg, int L)
-{
-    int n = 0;
-    for (int l = lg; l > L && l > 4; l -= 4)
-        n += 6 << (l - 4);
-    return n;
-}
-
-// Fill them (all threads of the CTA; a barrier must follow).
-template <int LG>
-static __device__ __forceinline__ void fft16_fill_shared(float2 *tab)
-{
-#pragma unroll
-    for (int l = LG; l > 4; l -= 4) {
-        const int S = 1 << (l - 4);
-        for (int t = threadIdx.x; t < 6 * S; t += blockDim.x) {
-            const int i = t / S, e = i < 4 ? i + 1 : 4 * (i - 2);  // exponents 1, 2, 3, 4, 8, 12
-            float sn, cs;
-            sincospif(-2.0f * (float)((t - i * S) * e) / (float)(1 << l), &sn, &cs);
-            tab[fft16_tab_shared(LG, l) + t] = make_float2(cs, sn);
-        }
-    }
-}
-
-// buf: the transform's exchange buffer; tab: the twiddle table (fft16_tw_at's layout;
-// TAB_SHARED: in shared memory, the levels of this length only, fft16_tab_shared);
-// bar: a named barrier (1 .. 15) of the transform's T threads, used where T > 32.
-template <int LG, bool TAB_SHARED = false>
+// buf: the transform's exchange buffer; tab: the twiddle table (fft16_tw_at's layout; what
+// the rounding took from the entries lies kFft16TwLo entries on); bar: a named barrier
+// (1 .. 15) of the transform's T threads, used where T > 32.  FINE: twiddles in two parts.
+template <int LG, bool FINE = false>
 struct Fft16 {
     static constexpr int M = 1 << LG, T = M / 16;
     static constexpr int kLast = (LG - 1) % 4 + 1;  // log2 length of the last level
@@ -316,49 +314,29 @@ struct Fft16 {
     __device__ __forceinline__ void twiddle(float2 (&v)[16]) const
     {
         constexpr int S = 1 << (L - 4);
-        float2 w[16];
-        if constexpr (TAB_SHARED) {
-            const uint32_t t = smem_addr(tab) + 8u * (uint32_t)(fft16_tab_shared(LG, L) + (u & (S - 1)));
-            w[1] = lds2(t);
-            w[2] = lds2(t + 8u * S);
-            w[3] = lds2(t + 16u * S);
-            w[4] = lds2(t + 24u * S);
-            w[8] = lds2(t + 32u * S);
-            w[12] = lds2(t + 40u * S);
-        } else {
-            const float2 *__restrict__ t = tab + fft16_tw_at(L) + (u & (S - 1));
-            w[1] = __ldg(t);
-            w[2] = __ldg(t + S);
-            w[3] = __ldg(t + 2 * S);
-            w[4] = __ldg(t + 3 * S);
-            w[8] = __ldg(t + 4 * S);
-            w[12] = __ldg(t + 5 * S);
-        }
-        if (INV) {
+        const float2 *__restrict__ t = tab + fft16_tw_at(L) + (u & (S - 1));
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                const int e = k < 4 ? k + 1 : 4 * (k - 2);
-                w[e].y = -w[e].y;
+        for (int k = 1; k < 16; ++k) {
+            float2 w = __ldg(t + (k - 1) * S);
+            if (INV)
+                w.y = -w.y;
+            if constexpr (FINE) {
+                float2 l = __ldg(t + kFft16TwLo + (k - 1) * S);
+                if (INV)
+                    l.y = -l.y;
+                v[k] = cmul_fine(v[k], w, l);
+            } else {
+                v[k] = cmul(v[k], w);
             }
         }
-#pragma unroll
-        for (int hi = 0; hi < 16; hi += 4)
-#pragma unroll
-            for (int lo = 0; lo < 4; ++lo) {
-                if (hi + lo == 0)
-                    continue;
-                if (hi && lo)
-                    w[hi + lo] = cmul(w[hi], w[lo]);
-                v[hi + lo] = cmul(v[hi + lo], w[hi + lo]);
-            }
     }
     template <int L, bool HALF>
     __device__ __forceinline__ void down(float2 (&v)[16]) const
     {
         if constexpr (L < 4) {
-            dft_runs<(1 << L), false>(v);
+            dft_runs<(1 << L), false, FINE>(v);
         } else {
-            dft16<false, HALF>(v);
+            dft16<false, HALF, FINE>(v);
             if constexpr (L > 4) {
                 twiddle<L, false>(v);
                 put<L>(v);
@@ -376,7 +354,7 @@ struct Fft16 {
             sync();
             get<L + 4>(v);
             twiddle<L + 4, true>(v);
-            dft16<true>(v);
+            dft16<true, false, FINE>(v);
             up<L + 4>(v);
         }
     }
@@ -390,9 +368,9 @@ struct Fft16 {
     __device__ __forceinline__ void inverse(float2 (&v)[16]) const
     {
         if constexpr (kLast < 4)
-            dft_runs<(1 << kLast), true>(v);
+            dft_runs<(1 << kLast), true, FINE>(v);
         else
-            dft16<true>(v);
+            dft16<true, false, FINE>(v);
         up<kLast>(v);
     }
 };

@@ -37,7 +37,7 @@ template <int LG, int THREADS>
 __global__ void __launch_bounds__(THREADS) fk_time16_kernel(const FkJob J)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    using F = Fft16<LG>;
+    using F = Fft16<LG, true>;
     constexpr int T = F::T, M = F::M;
     dependents_may_start();
     if (blockIdx.x == 0 && threadIdx.x == 0 && J.maxbits)

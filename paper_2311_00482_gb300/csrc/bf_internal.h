@@ -62,11 +62,13 @@ constexpr int kMaxFramesPerJob = 4;
 enum Prec : int { kPrecF32 = 0, kPrecF16 = 1, kPrecBF16 = 2, kPrecIQ = 3 };
 
 // Layout of the Fft16 transforms (bf_fft16.cuh), shared with the host tables.
-// Twiddles of a level of length 2^L, S = 2^(L-4): exponents 1, 2, 3, 4, 8, 12 of
-// W_(2^L)^t, each a run of S entries, levels L = 5, 6, ... back to back (one
-// table serves every transform length; the other powers are single products).
+// Twiddles of a level of length 2^L, S = 2^(L-4): exponents 1 .. 15 of W_(2^L)^t, each a
+// run of S entries, levels L = 5, 6, ... back to back (one table serves every transform
+// length).  Every power has an entry of its own: as products of two entries (six runs a
+// level) nine of the fifteen carried two entries' roundings and their own.
 constexpr int kFft16MaxLg = 13;
-__host__ __device__ constexpr int fft16_tw_at(int L) { return 6 * ((1 << (L - 4)) - 2); }
+__host__ __device__ constexpr int fft16_tw_at(int L) { return 15 * ((1 << (L - 4)) - 2); }
+constexpr int kFft16TwLo = fft16_tw_at(kFft16MaxLg + 1);
 // Bin held by register q of thread u after the forward transform.
 __host__ __device__ inline int fft16_bin(int lg, int u, int q)
 {

@@ -31,9 +31,11 @@ namespace {
 constexpr size_t kStaticPixels = (size_t)1 << 20;  // largest nx * nz accepted
 constexpr int kMaxDevices = 64;
 
-// [0, kStaticPixels): envelope image; from kStaticPixels: the envelope CTAs' maxima.
+// [0, kStaticPixels): envelope image; from kStaticPixels: the envelope CTAs' maxima; from
+// kStaticTw: the level twiddles (fft16_twiddles), written by a device's first call.
 constexpr int kStaticMaxima = 512;
-__device__ __align__(256) float g_static_scratch[kStaticPixels + kStaticMaxima];
+constexpr size_t kStaticTw = kStaticPixels + kStaticMaxima, kStaticTwFloats = (size_t)kFft16TwLo * 4;
+__device__ __align__(256) float g_static_scratch[kStaticTw + kStaticTwFloats];
 
 // The CTA's largest value into its slot of the maxima.
 __device__ __forceinline__ void block_max(float v, float *__restrict__ slot)
@@ -55,8 +57,8 @@ __device__ __forceinline__ void block_max(float v, float *__restrict__ slot)
     }
 }
 
-// Depths of 32 rows and more: the envelope kernel's transforms, with twiddles and
-// masks computed here.  512 x 512 with the band-pass: 17.5 us as radix-4 passes over
+// Depths of 32 rows and more: the envelope kernel's transforms, with the static twiddles
+// (in two parts) and masks computed here.  512 x 512 with the band-pass: 17.5 us as radix-4 passes over
 // shared memory by 64 CTAs of eight columns; a CTA now holds T-thread transforms of
 // 4096 points in all.
 template <int LG>
@@ -66,12 +68,10 @@ __global__ void __launch_bounds__(256, 2)
 {
     extern __shared__ __align__(16) float2 sbuf[];
     dependents_may_start();
-    float2 *tab = sbuf + 256 * (17 + 16);
-    fft16_fill_shared<LG>(tab);
-    __syncthreads();
     const uint32_t bufs = smem_addr(sbuf);
     const float v = envelope_pairs<LG, false, 256, true>(
-        y, env, nx, 1 << LG, blockIdx.x * envelope_pairs_per_block(LG), band != 0, tab,
+        y, env, nx, 1 << LG, blockIdx.x * envelope_pairs_per_block(LG), band != 0,
+        reinterpret_cast<const float2 *>(g_static_scratch + kStaticTw),
         MaskFactors<LG>{kb_lo, kb_hi, band != 0}, bufs, bufs + 256 * 17 * 8);
     block_max(v, maxima + blockIdx.x);
 }
@@ -179,7 +179,7 @@ template <int LG>
 cudaError_t launch_static16(const float *y, int nx, int band, int lo, int hi, float *env,
                             float *maxima, int *blocks, cudaStream_t st)
 {
-    const size_t smem = (256 * (17 + 16) + fft16_tab_shared(LG, 4)) * sizeof(float2);
+    const size_t smem = 256 * (17 + 16) * sizeof(float2);
     int sms = 0;
     cudaError_t e = kernel_setup((const void *)static_envelope16_kernel<LG>, smem, 256, true, &sms,
                                  nullptr);
@@ -193,10 +193,13 @@ cudaError_t launch_static16(const float *y, int nx, int band, int lo, int hi, fl
 
 std::mutex g_static_mu;
 float *g_static_ptr[kMaxDevices] = {};
+bool g_static_tw[kMaxDevices] = {};  // twiddles written
 
 // Device address of the scratch array on the current device, looked up once
-// per device (the array's name is only a host-side stand-in in host code).
-int static_scratch(float **out)
+// per device (the array's name is only a host-side stand-in in host code); a device's
+// first call also sends the twiddles ahead of its kernels (every call into a capture
+// does, until one outside has: a captured copy runs with its graph only).
+int static_scratch(float **out, cudaStream_t st)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -211,6 +214,21 @@ int static_scratch(float **out)
         if (e != cudaSuccess)
             return cuda_fail(e, "cudaGetSymbolAddress (static scratch)");
         g_static_ptr[dev] = static_cast<float *>(p);
+    }
+    if (!g_static_tw[dev]) {
+        static const std::vector<float> tw = [] {
+            std::vector<float> t;
+            fft16_twiddles(t);
+            return t;
+        }();
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(st, &cap);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(g_static_ptr[dev] + kStaticTw, tw.data(), tw.size() * sizeof(float),
+                                cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess)
+            return cuda_fail(e, "cudaMemcpyAsync (static twiddles)");
+        g_static_tw[dev] = cap == cudaStreamCaptureStatusNone;
     }
     *out = g_static_ptr[dev];
     return BF_OK;
@@ -304,7 +322,7 @@ extern "C" BF_API int bf_logdb_static(const float *y_dev, int32_t nx, int32_t nz
     if (!(z1_m >= z0_m) || !(c_mps > 0.0) || !(f0_hz > 0.0))
         return fail(BF_EINVAL, "bad depth range or acquisition parameters");
     float *scratch = nullptr;
-    int rc = static_scratch(&scratch);
+    int rc = static_scratch(&scratch, (cudaStream_t)cuda_stream);
     if (rc)
         return rc;
     int kb_lo = 1, kb_hi = 0;

@@ -315,16 +315,17 @@ void fft_twiddles(int n, std::vector<float> &tw)
 
 void fft16_twiddles(std::vector<float> &tw)
 {
-    const int e[6] = {1, 2, 3, 4, 8, 12};
-    tw.resize((size_t)fft16_tw_at(kFft16MaxLg + 1) * 2);
+    tw.resize((size_t)kFft16TwLo * 4);
     for (int L = 5; L <= kFft16MaxLg; ++L) {
         const int S = 1 << (L - 4);
-        for (int i = 0; i < 6; ++i)
+        for (int i = 0; i < 15; ++i)
             for (int t = 0; t < S; ++t) {
-                const double ang = -2.0 * kPi * (double)(t * e[i]) / (double)(1 << L);
-                float *w = &tw[2 * ((size_t)fft16_tw_at(L) + i * S + t)];
+                const double ang = -2.0 * kPi * (double)(t * (i + 1)) / (double)(1 << L);
+                float *w = &tw[2 * ((size_t)fft16_tw_at(L) + i * S + t)], *l = w + 2 * kFft16TwLo;
                 w[0] = (float)std::cos(ang);
                 w[1] = (float)std::sin(ang);
+                l[0] = (float)(std::cos(ang) - (double)w[0]);
+                l[1] = (float)(std::sin(ang) - (double)w[1]);
             }
     }
 }
