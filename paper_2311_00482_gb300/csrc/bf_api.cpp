@@ -1433,7 +1433,7 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         rc = ce == cudaSuccess ? BF_OK : cuda_fail(ce, "cudaStreamSynchronize");
     }
     if (!rc && rebuild)
-        rc = h->fk_beta.ensure((size_t)n_angles * ne * sizeof(float));
+        rc = h->fk_beta.ensure((size_t)n_angles * ne * (regs ? 2 : 1) * sizeof(float));
     if (!rc && rebuild)
         rc = h->fk_i0.ensure((size_t)n_angles * npts * sizeof(int));
     if (!rc && rebuild)
@@ -1441,7 +1441,7 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     if (rc)
         return rc;
     if (rebuild) {
-        std::vector<float> beta((size_t)n_angles * ne);
+        std::vector<float> beta;
         std::vector<double> sc((size_t)2 * n_angles);
         for (int a = 0; a < n_angles; ++a) {
             sc[2 * a] = std::sin(angles_rad[a]);
@@ -1449,7 +1449,9 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
             for (int i = 0; i < ne; ++i) {
                 const double x = ((double)i - 0.5 * (double)(ne - 1)) * pitch;
                 const double turns = x * sc[2 * a] / ((double)nt * dz);  // half turns per bin
-                beta[(size_t)a * ne + i] = (float)(regs ? turns : kPi * turns);
+                beta.push_back((float)(regs ? turns : kPi * turns));
+                if (regs)
+                    beta.push_back((float)(turns - (double)beta.back()));
             }
         }
         std::vector<int> i0;

@@ -202,7 +202,7 @@ struct FkJob {
     float *img;           // [ne][ns] magnitude image
     unsigned *maxbits;    // image maximum (float bits) for the log stage, or null
     // [na][ne] lateral phase per time bin: pi x_i sin(theta_a) / (nt dz); for
-    // launch_fkmig16 without the pi (half turns)
+    // launch_fkmig16 without the pi (half turns), in two parts (float2)
     const float *beta;
     // the mapping, decided on the host in double precision: per (angle, Kz bin
     // q = 1 .. nt/2, Kx bin) the temporal bin i0 below the mapped position (-1:

@@ -2,7 +2,10 @@
 import numpy as np
 import pytest
 
+import oracle
 import paper_2311_00482_gb300 as bf
+import synth
+from test_gpu_fk import run_fk
 from test_gpu_parity import torch  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -86,3 +89,16 @@ def test_band_passed_envelope_is_no_further_off_than_radix_4(torch, seed):  # no
 
     ours = 10 ** (db / 20) * peak
     assert error((ours[::2], ours[1::2])) <= error(four)
+
+
+def test_fk_phases_of_long_delays(torch):  # noqa: F811
+    """A transmit of 20 degrees over 128 elements: lateral delays of up to 85 samples, 43
+    half turns at the last bin, 21 at the pulse's.  A phase formed in one FP32 product is
+    off by 21 pi 2^-25 = 2e-6 rms, the image with it; without that the transforms (42
+    radix-2 equivalents of 0.6 u each, as a random walk 2.3e-7) and the tabulated weights
+    (u / sqrt(12) each, twice) are left.  Tolerance: twice their sum."""
+    acq = synth.CYST_WIRES_512.with_(n_elements=128, n_samples=2048, angles_deg=(20.0,))
+    rf, _ = synth.cyst_wires_frame(acq)
+    got = run_fk(torch, acq, rf)
+    ref = oracle.fk_migrate(rf, acq.pitch_m, acq.angles_rad, acq.fs_hz, acq.c_mps)
+    assert np.linalg.norm(got - ref) <= 2 * (2.3e-7 + 0.4e-7) * np.linalg.norm(ref)
