@@ -65,7 +65,9 @@ __device__ __forceinline__ float magnitude(float q, float a, float b)
 // way the spectrum is multiplied by real tables (gr: the band-passed column, a
 // real even response; gh: i gh its Hilbert transform, a real odd one), with the
 // inverse's 1 / M in them: one forward transform and one inverse, or two for the
-// band-passed image, serve two columns.  (Bluestein's four transforms per single
+// band-passed image, serve two columns.  Convolved columns are brought to one magnitude
+// first (pair_down), so that a quiet column keeps its own precision beside a loud one;
+// power-of-two depths share as they are, like the warp kernel.  (Bluestein's four transforms per single
 // column, which this replaced: 39.4 us of a 64 x 1750 image's pass, 732 us of the
 // pass of 32 uneven images of 64-1024 rows; by the whole passes 47.7 -> 30.7 us
 // and 3345 -> 2712 us.)  Bound: latency of the exchanges at small
@@ -100,10 +102,31 @@ __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, flo
                 v[j].y = __ldcs(yb + n);
         }
     }
+    uint2 top = make_uint2(0u, 0u);
+    if constexpr (CONV) {
+#pragma unroll
+        for (int j = 0; j < JN; ++j) {
+            top.x = max(top.x, __float_as_uint(fabsf(v[j].x)));
+            top.y = max(top.y, __float_as_uint(fabsf(v[j].y)));
+        }
+        top = f.pair_max(top.x, top.y);
+        const float da = pair_down(top.x), db = pair_down(top.y);
+#pragma unroll
+        for (int j = 0; j < JN; ++j)
+            v[j] = make_float2(v[j].x * da, v[j].y * db);
+    }
+    const float ua = CONV ? pair_up(top.x) : 1.f, ub = CONV ? pair_up(top.y) : 1.f;
+    // a column with infinities or NaNs has no transform, and takes no part in its neighbour's
+    const bool bad_a = CONV && top.x >= 0x7f800000u, bad_b = CONV && top.y >= 0x7f800000u;
     if (!band) {
 #pragma unroll
         for (int j = 0; j < JN; ++j)
             sts2(slot + 8u * THREADS * j, v[j]);  // the columns themselves
+    }
+    if (bad_a || bad_b) {
+#pragma unroll
+        for (int j = 0; j < JN; ++j)
+            v[j] = make_float2(bad_a ? 0.f : v[j].x, bad_b ? 0.f : v[j].y);
     }
     f.template forward<CONV>(v);
 #pragma unroll 1
@@ -146,12 +169,12 @@ __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, flo
         if (CONV && n >= nz)
             continue;
         if (has_a) {
-            const float e = magnitude(q.x, r.x, v[j].x);
+            const float e = bad_a ? hypot_far(r.x, __int_as_float(0x7fffffff)) : magnitude(q.x, r.x, v[j].x) * ua;
             __stcg(oa + n, e);
             lmax = fmaxf(lmax, e);
         }
         if (has_b) {
-            const float e = magnitude(q.y, r.y, v[j].y);
+            const float e = bad_b ? hypot_far(r.y, __int_as_float(0x7fffffff)) : magnitude(q.y, r.y, v[j].y) * ub;
             __stcg(ob + n, e);
             lmax = fmaxf(lmax, e);
         }

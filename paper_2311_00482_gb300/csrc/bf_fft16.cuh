@@ -257,6 +257,25 @@ static __device__ __forceinline__ void sts2(uint32_t a, float2 v)
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
+// Two real sequences that share a complex transform leak each other's rounding errors:
+// both are scaled to one magnitude first, by powers of two (exact), so that each keeps
+// an error relative to its own.  m: the bits of a sequence's largest magnitude (finite);
+// a sequence of zeros comes back as zeros.
+static __device__ __forceinline__ unsigned pair_exponent(unsigned m)
+{
+    return min(max(m >> 23, 1u), 253u);
+}
+
+static __device__ __forceinline__ float pair_down(unsigned m)  // to [1, 2)
+{
+    return __uint_as_float((254u - pair_exponent(m)) << 23);
+}
+
+static __device__ __forceinline__ float pair_up(unsigned m)  // and back
+{
+    return m ? __uint_as_float(pair_exponent(m) << 23) : 0.f;
+}
+
 // buf: the transform's exchange buffer; tab: the twiddle table (fft16_tw_at's layout; what
 // the rounding took from the entries lies kFft16TwLo entries on); bar: a named barrier
 // (1 .. 15) of the transform's T threads, used where T > 32.  FINE: twiddles in two parts.
@@ -274,6 +293,35 @@ struct Fft16 {
             __syncwarp();
         else
             asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(T) : "memory");
+    }
+    // Largest of the T threads' ma and mb (magnitudes, as their bits).  The warps' results
+    // go through elements of the buffer that no exchange uses (every seventeenth), so no
+    // barrier stands before the transform that follows.  Once per kernel.
+    __device__ __forceinline__ uint2 pair_max(unsigned ma, unsigned mb) const
+    {
+        if constexpr (T < 32) {
+#pragma unroll
+            for (int off = 1; off < T; off <<= 1) {
+                ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, off));
+                mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, off));
+            }
+        } else {
+            ma = __reduce_max_sync(0xffffffffu, ma);
+            mb = __reduce_max_sync(0xffffffffu, mb);
+            if constexpr (T > 32) {
+                auto at = [&](int w) { return buf + 8u * (uint32_t)(17 * w + 16); };
+                if (u % 32 == 0)
+                    sts2(at(u / 32), make_float2(__uint_as_float(ma), __uint_as_float(mb)));
+                sync();
+#pragma unroll
+                for (int w = 0; w < T / 32; ++w) {
+                    const float2 m = lds2(at(w));
+                    ma = max(ma, __float_as_uint(m.x));
+                    mb = max(mb, __float_as_uint(m.y));
+                }
+            }
+        }
+        return make_uint2(ma, mb);
     }
     // Address of this thread's element 0 at a level, and element j's offset.
     template <int L>
