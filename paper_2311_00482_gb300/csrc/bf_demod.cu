@@ -38,6 +38,24 @@ __device__ __forceinline__ void demod_units(const DemodJob &J, int unit0, uint32
     for (int j = 0; j < 16; ++j)
         v[j] = make_float2(has_a ? (float)__ldg(ua + f.u + j * T) : 0.f,
                            has_b ? (float)__ldg(ub + f.u + j * T) : 0.f);
+    // Two rows of one frame each keep their own precision (a dead channel's stays zero);
+    // the two frames of a pair share a row as they are.
+    float ha = 1.f, hb = 1.f;
+    if (J.nf == 1) {
+        unsigned ma = 0u, mb = 0u;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            ma = max(ma, __float_as_uint(fabsf(v[j].x)));
+            mb = max(mb, __float_as_uint(fabsf(v[j].y)));
+        }
+        const uint2 m = f.pair_max(ma, mb);
+        const float da = pair_down(m.x), db = pair_down(m.y);
+        ha = pair_up(m.x);
+        hb = pair_up(m.y);
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            v[j] = make_float2(v[j].x * da, v[j].y * db);
+    }
     f.template forward<false>(v);
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
@@ -50,7 +68,7 @@ __device__ __forceinline__ void demod_units(const DemodJob &J, int unit0, uint32
     auto at = [&](int n) { return f.buf + 8u * (uint32_t)(n + (n >> 4)); };
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-        sts2(at(f.u + j * T), v[j]);
+        sts2(at(f.u + j * T), make_float2(v[j].x * ha, v[j].y * hb));
     f.sync();
     // pair j: samples k = j - kPadL and k + 1, mid = (A + B) / 2 and diff = B - A with
     // A = a[k], B = a[k + 1] rot (zero outside the record)
@@ -89,7 +107,7 @@ __device__ __forceinline__ void demod_units(const DemodJob &J, int unit0, uint32
 }
 
 template <bool BIG>
-__global__ void __launch_bounds__(BIG ? kDemodBigThreads : kDemodThreads, BIG ? 1 : 3)
+__global__ void __launch_bounds__(BIG ? kDemodBigThreads : kDemodThreads, BIG ? 1 : 2)
     demod16_kernel(const DemodJob *__restrict__ jobs, const int *__restrict__ blk_prefix, int njobs)
 {
     constexpr int THREADS = BIG ? kDemodBigThreads : kDemodThreads;
