@@ -153,6 +153,10 @@ __device__ __forceinline__ void solo_channels(SoloAcc<NA> &A, const int4 (&E)[NC
                                               const SoloCheck &K, float inv_p, bool square)
 {
     constexpr uint32_t PB = PairIO<PREC>::kBytes;
+    // Channels walked together are added up before they enter the running sums, which so
+    // take half or a quarter of the roundings (one angle: sixteen for 64 channels).
+    constexpr bool FIRST = NCH > 1;
+    f32x2_t sum = 0, roots[AN], proots[AN];
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
         const f32x2_t D2 = pk2(D[c], D[c]);
@@ -183,21 +187,42 @@ __device__ __forceinline__ void solo_channels(SoloAcc<NA> &A, const int4 (&E)[NC
                 v1 = (unsigned)(K.r_first + 1 - vr.x) <= span ? v1 : 0.f;
             }
             const f32x2_t v = pk2(v0, v1);
-            A.S1 = add2(A.S1, v);
+            if (FIRST)
+                sum = c == 0 && k == 0 ? v : add2(sum, v);
+            else
+                A.S1 = add2(A.S1, v);
             if (DMAS) {
                 const f32x2_t q = pk2(copysignf(sqrt_approx(fabsf(v0)), v0),
                                       copysignf(sqrt_approx(fabsf(v1)), v1));
-                A.T1[k] = add2(A.T1[k], q);
+                if (FIRST)
+                    roots[k] = c == 0 ? q : add2(roots[k], q);
+                else
+                    A.T1[k] = add2(A.T1[k], q);
                 // a channel's angles first, so that T2 is no longer a sum than per angle
                 squares = AN == 1 ? fma2(q, q, A.T2) : k == 0 ? mul2(q, q) : fma2(q, q, squares);
             }
             if (CF)
                 A.Su2 = fma2(v, v, A.Su2);
-            if (PDAS)
-                A.P1[k] = add2(A.P1[k], pk2(pdas_root(v0, inv_p, square), pdas_root(v1, inv_p, square)));
+            if (PDAS) {
+                const f32x2_t q = pk2(pdas_root(v0, inv_p, square), pdas_root(v1, inv_p, square));
+                if (FIRST)
+                    proots[k] = c == 0 ? q : add2(proots[k], q);
+                else
+                    A.P1[k] = add2(A.P1[k], q);
+            }
         }
         if (DMAS)
             A.T2 = AN == 1 ? squares : add2(A.T2, squares);
+    }
+    if (FIRST) {
+        A.S1 = add2(A.S1, sum);
+#pragma unroll
+        for (int k = 0; k < AN; ++k) {
+            if (DMAS)
+                A.T1[k] = add2(A.T1[k], roots[k]);
+            if (PDAS)
+                A.P1[k] = add2(A.P1[k], proots[k]);
+        }
     }
 }
 
