@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(BIG ? kEnvBigThreads : kEnvThreads, BIG ? 1 : 
     auto run = [&](auto lg, auto conv) {
         constexpr int LG = decltype(lg)::value;
         constexpr bool CONV = decltype(conv)::value != 0;
-        lmax = envelope_pairs<LG, CONV, THREADS, false>(
+        lmax = envelope_pairs<LG, CONV, THREADS, Twiddles::kProducts>(
             J.y, J.env, J.nx, J.nz, first * envelope_pairs_per_block(LG), J.band != 0, J.ptw,
             TableFactors<Fft16<LG>::T>{J.gr, J.gh}, bufs, hold);
     };

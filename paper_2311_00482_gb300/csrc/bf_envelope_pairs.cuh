@@ -72,13 +72,13 @@ __device__ __forceinline__ float magnitude(float q, float a, float b)
 // pass of 32 uneven images of 64-1024 rows; by the whole passes 47.7 -> 30.7 us
 // and 3345 -> 2712 us.)  Bound: latency of the exchanges at small
 // image counts, shared-memory traffic and FP32 issue about equally at large ones.
-template <int LG, bool CONV, int THREADS, bool FINE, class Factors>
+template <int LG, bool CONV, int THREADS, Twiddles TW, class Factors>
 __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, float *__restrict__ env,
                                                 int nx, int nz_in, int pair0, bool band,
                                                 const float2 *tab, const Factors &G, uint32_t bufs,
                                                 uint32_t hold)
 {
-    using F = Fft16<LG, FINE>;
+    using F = Fft16<LG, TW>;
     constexpr int T = F::T;
     const int grp = threadIdx.x / T;
     const F f{bufs + (uint32_t)(grp * fft16_buf_bytes(LG)), tab, (int)threadIdx.x % T, 1 + grp};

@@ -278,9 +278,17 @@ static __device__ __forceinline__ float pair_up(unsigned m)  // and back
 
 // buf: the transform's exchange buffer; tab: the twiddle table (fft16_tw_at's layout; what
 // the rounding took from the entries lies kFft16TwLo entries on); bar: a named barrier
-// (1 .. 15) of the transform's T threads, used where T > 32.  FINE: twiddles in two parts.
-template <int LG, bool FINE = false>
+// (1 .. 15) of the transform's T threads, used where T > 32.
+//
+// How a level's fifteen twiddles come about: six entries and nine products of two (the
+// envelopes and the demodulation, whose launches wait for these loads: with fifteen
+// entries sixteen served frames took 1346 us instead of 1300); an entry each; or an entry
+// and what its rounding took (two parts), where the transform's error shows.
+enum class Twiddles { kProducts, kEntries, kTwoParts };
+
+template <int LG, Twiddles TW = Twiddles::kProducts>
 struct Fft16 {
+    static constexpr bool FINE = TW == Twiddles::kTwoParts;
     static constexpr int M = 1 << LG, T = M / 16;
     static constexpr int kLast = (LG - 1) % 4 + 1;  // log2 length of the last level
     uint32_t buf;
@@ -363,18 +371,36 @@ struct Fft16 {
     {
         constexpr int S = 1 << (L - 4);
         const float2 *__restrict__ t = tab + fft16_tw_at(L) + (u & (S - 1));
+        auto entry = [&](int k) {
+            const float2 w = __ldg(t + (k - 1) * S);
+            return make_float2(w.x, INV ? -w.y : w.y);
+        };
+        if constexpr (TW == Twiddles::kProducts) {
+            float2 w[16];
 #pragma unroll
-        for (int k = 1; k < 16; ++k) {
-            float2 w = __ldg(t + (k - 1) * S);
-            if (INV)
-                w.y = -w.y;
-            if constexpr (FINE) {
-                float2 l = __ldg(t + kFft16TwLo + (k - 1) * S);
-                if (INV)
-                    l.y = -l.y;
-                v[k] = cmul_fine(v[k], w, l);
-            } else {
-                v[k] = cmul(v[k], w);
+            for (int k = 0; k < 6; ++k) {
+                const int e = k < 4 ? k + 1 : 4 * (k - 2);
+                w[e] = entry(e);
+            }
+#pragma unroll
+            for (int hi = 0; hi < 16; hi += 4)
+#pragma unroll
+                for (int lo = 0; lo < 4; ++lo) {
+                    if (hi + lo == 0)
+                        continue;
+                    if (hi && lo)
+                        w[hi + lo] = cmul(w[hi], w[lo]);
+                    v[hi + lo] = cmul(v[hi + lo], w[hi + lo]);
+                }
+        } else {
+#pragma unroll
+            for (int k = 1; k < 16; ++k) {
+                if constexpr (FINE) {
+                    const float2 l = __ldg(t + kFft16TwLo + (k - 1) * S);
+                    v[k] = cmul_fine(v[k], entry(k), make_float2(l.x, INV ? -l.y : l.y));
+                } else {
+                    v[k] = cmul(v[k], entry(k));
+                }
             }
         }
     }

@@ -49,7 +49,7 @@ template <int LG, int THREADS>
 __global__ void __launch_bounds__(THREADS) fk_time16_kernel(const FkJob J)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    using F = Fft16<LG, true>;
+    using F = Fft16<LG, Twiddles::kTwoParts>;
     constexpr int T = F::T, M = F::M;
     dependents_may_start();
     if (blockIdx.x == 0 && threadIdx.x == 0 && J.maxbits)
@@ -100,7 +100,7 @@ template <int LG, int THREADS>
 __global__ void __launch_bounds__(THREADS) fk_rows16_kernel(const FkJob J)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    using F = Fft16<LG>;
+    using F = Fft16<LG, Twiddles::kEntries>;
     constexpr int T = F::T, M = F::M;
     dependents_may_start();
     const int grp = threadIdx.x / T, nb = J.nt / 2 + 1, a = blockIdx.y;
@@ -131,7 +131,7 @@ template <int LG>
 __global__ void __launch_bounds__(256) fk_map16_kernel(const FkJob J)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    using F = Fft16<LG>;
+    using F = Fft16<LG, Twiddles::kEntries>;
     constexpr int T = F::T, M = F::M, R = fk_map_rows(LG), STEP = 256 / R, NP = M / STEP;
     // rows' buffers one float2 apart modulo the banks: lanes along rows do not collide
     constexpr int ROW = fft16_buf_bytes(LG) + 8;
@@ -205,7 +205,7 @@ template <int LG, int THREADS>
 __global__ void __launch_bounds__(THREADS) fk_depth16_kernel(const FkJob J)
 {
     extern __shared__ __align__(16) float2 fsm[];
-    using F = Fft16<LG>;
+    using F = Fft16<LG, Twiddles::kEntries>;
     constexpr int T = F::T, M = F::M;
     dependents_may_start();
     const int grp = threadIdx.x / T;

@@ -64,8 +64,7 @@ enum Prec : int { kPrecF32 = 0, kPrecF16 = 1, kPrecBF16 = 2, kPrecIQ = 3 };
 // Layout of the Fft16 transforms (bf_fft16.cuh), shared with the host tables.
 // Twiddles of a level of length 2^L, S = 2^(L-4): exponents 1 .. 15 of W_(2^L)^t, each a
 // run of S entries, levels L = 5, 6, ... back to back (one table serves every transform
-// length).  Every power has an entry of its own: as products of two entries (six runs a
-// level) nine of the fifteen carried two entries' roundings and their own.
+// length), then as many entries that hold what the rounding took.
 constexpr int kFft16MaxLg = 13;
 __host__ __device__ constexpr int fft16_tw_at(int L) { return 15 * ((1 << (L - 4)) - 2); }
 constexpr int kFft16TwLo = fft16_tw_at(kFft16MaxLg + 1);

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256, 2)
     extern __shared__ __align__(16) float2 sbuf[];
     dependents_may_start();
     const uint32_t bufs = smem_addr(sbuf);
-    const float v = envelope_pairs<LG, false, 256, true>(
+    const float v = envelope_pairs<LG, false, 256, Twiddles::kTwoParts>(
         y, env, nx, 1 << LG, blockIdx.x * envelope_pairs_per_block(LG), band != 0,
         reinterpret_cast<const float2 *>(g_static_scratch + kStaticTw),
         MaskFactors<LG>{kb_lo, kb_hi, band != 0}, bufs, bufs + 256 * 17 * 8);
