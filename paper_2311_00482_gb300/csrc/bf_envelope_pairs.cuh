@@ -158,6 +158,12 @@ __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, flo
             }
         }
     }
+    if (bad_a || bad_b) {
+        const float nan = __int_as_float(0x7fffffff);
+#pragma unroll
+        for (int j = 0; j < JN; ++j)
+            v[j] = make_float2(bad_a ? nan : v[j].x, bad_b ? nan : v[j].y);
+    }
     float lmax = 0.f;
     float *__restrict__ oa = env + (size_t)ca * nz;
     float *__restrict__ ob = oa + nz;
@@ -169,12 +175,12 @@ __device__ __forceinline__ float envelope_pairs(const float *__restrict__ y, flo
         if (CONV && n >= nz)
             continue;
         if (has_a) {
-            const float e = bad_a ? hypot_far(r.x, __int_as_float(0x7fffffff)) : magnitude(q.x, r.x, v[j].x) * ua;
+            const float e = magnitude(q.x, r.x, v[j].x) * ua;
             __stcg(oa + n, e);
             lmax = fmaxf(lmax, e);
         }
         if (has_b) {
-            const float e = bad_b ? hypot_far(r.y, __int_as_float(0x7fffffff)) : magnitude(q.y, r.y, v[j].y) * ub;
+            const float e = magnitude(q.y, r.y, v[j].y) * ub;
             __stcg(ob + n, e);
             lmax = fmaxf(lmax, e);
         }
