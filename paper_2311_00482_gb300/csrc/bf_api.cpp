@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/bf.h"
+#include "bf_choice.h"
 #include "bf_engine.h"
 
 namespace bfi {
@@ -255,11 +256,8 @@ static PlanKey tuned_key(PlanKey k)
 }
 
 // Configuration of a workload (of kTileConfigs, or a solo one): BF_TILE_ROWS, else
-// what bf_autotune measured fastest for it, else by the frames that share it.
-// Beamforming time per 512 x 512 frame, 32 frames in a batch, DAS + DMAS of one
-// angle / DMAS of three: alone (solo, measured before its one-angle registers, which
-// take a lone frame of one angle from 24.9 to 18.7 us) 13.7 / 22.3 us, in pairs on
-// 32-row tiles 7.4 / 21.0 us, in fours on 16-row tiles 5.9 / 16.2 us.
+// what bf_autotune measured fastest for it, else by the frames that share it
+// (bf_choice.h).
 static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w, bool narrow_ok)
 {
     const int forced = forced_cfg();
@@ -268,19 +266,8 @@ static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w,
     auto it = h->tuned.find(key);
     if (it != h->tuned.end())
         return it->second;
-    // Alone: split the channels of a row pair over four warps below 3/4 of a 16-row
-    // tile per SM, over two below 3/2 (152 SMs; splits 1 / 2 / 4, DMAS of three angles:
-    // 32 tiles 26.2 / 16.0 / 11.9 us, 112 tiles 20.4 / 16.0 / 13.9, 128 tiles 20.1 /
-    // 16.0 / 20.1, 220 tiles 28.3 / 24.2 / 32.4, 325 tiles 26.2 / 26.6 / 36.5, 512
-    // tiles 32.4 / 34.4 / 54.9).  The frame's own tiles decide, also in a batch: a
-    // frame's sums do not depend on what it is launched with.
-    if (w.alone && key.prec != kPrecIQ) {
-        const int tiles = (h->g.nx + kTileCols - 1) / kTileCols * ((h->g.nz + 15) / 16);
-        return kSoloConfig + (4 * tiles <= 3 * h->sms ? 2 : 2 * tiles <= 3 * h->sms ? 1 : 0);
-    }
-    if (w.peers >= kMaxFramesPerJob && narrow_ok)
-        return key.prec == kPrecIQ ? 4 : 6;
-    return 0;
+    return rule_config(key.prec, key.ns, (int)key.angles.size(), image_tiles(h->g.nx, h->g.nz), h->sms,
+                       w.alone, narrow_ok, w.peers);
 }
 
 // The angle tables of a plan key, shared by its tilings (the handle's lock is held).

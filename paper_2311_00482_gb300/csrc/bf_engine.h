@@ -258,7 +258,7 @@ namespace bfi {
 // What is known about a frame's launch when its plan is chosen.
 struct PlanWish {
     int cfg = -1;   // a configuration of kTileConfigs, or < 0: by the rules of choose_cfg
-    int peers = 1;  // frames of this plan and combiners submitted together (jobs of four)
+    int peers = 1;  // frames of this plan and combiners submitted together (see bf_choice.h)
     bool alone = false;  // the frame shares its plan with no other: RF frames take solo tiles
 };
 // Plan of a frame with these arguments (`flags`: its mode and precision bits).
