@@ -537,7 +537,8 @@ int prepare_frame(bf_handle *h, const int16_t *rf_dev, int ns, const double *ang
     const size_t img = (size_t)h->g.nx * h->g.nz;
     const int rows = na * h->g.ne;
     // room for the frames of a job this frame may lead (interleaved pairs)
-    const int cap = plan_frames_per_job(plan, modes, prec, nf_cap);
+    int cap = plan_frames_per_job(plan, modes, prec, nf_cap);
+    cap = wish.room > 0 ? std::min(cap, wish.room) : pairs_room(cap, wish.index, wish.peers, true);
     rc = s.pairs.ensure((size_t)cap * rows * plan->nsp * pair_bytes(prec));
     if (!rc && stage != BF_OUT_RF && !iq)  // IQ images are magnitudes already
         rc = s.y.ensure(nm * img * sizeof(float));
@@ -613,11 +614,6 @@ int job_frames_cap(const Plan *p, uint32_t flags, int cap)
     return plan_frames_per_job(p, (int)(flags & (BF_MODE_MASK | BF_IQ_MASK)), frame_prec(flags), cap);
 }
 
-static int max_frames_per_job(const FramePrep &a)
-{
-    return plan_frames_per_job(a.plan, a.modes, a.prec, a.nf_cap);
-}
-
 // Tensor map over the pairs of a job that frame f leads (nf frames interleaved, box
 // pairs per copy), encoded when the layout changed.
 static int job_map(const FramePrep &f, int nf, int box, CUtensorMap &out)
@@ -661,44 +657,75 @@ void use_solo_plans(std::vector<FramePrep> &frames)
     }
 }
 
+// The job of frame fi, the first that none has taken: its lead (whose pairs buffer holds
+// them all) and its partners.  Frames that can lead nothing are taken before those that
+// can, which are kept for further jobs.
+static std::vector<size_t> job_frames(const std::vector<FramePrep> &frames, const std::vector<char> &taken,
+                                      size_t fi)
+{
+    const FramePrep &f = frames[fi];
+    const size_t want = (size_t)plan_frames_per_job(f.plan, f.modes, f.prec, kMaxFramesPerJob);
+    std::vector<size_t> rest, leads;  // after fi, in order
+    for (size_t gi = fi + 1; gi < frames.size() && rest.size() + 1 < want && leads.size() < 2 * want; ++gi)
+        if (!taken[gi] && shareable(f, frames[gi]))
+            (frames[gi].nf_cap > 1 ? leads : rest).push_back(gi);
+    std::vector<size_t> job{fi};
+    if (f.nf_cap == 1) {
+        if (leads.empty())
+            return job;
+        auto most = std::max_element(leads.begin(), leads.end(), [&](size_t a, size_t b) {
+            return frames[a].nf_cap < frames[b].nf_cap;
+        });
+        job.insert(job.begin(), *most);
+        leads.erase(most);
+    }
+    rest.insert(rest.end(), leads.begin(), leads.end());
+    const size_t most = std::min({want, (size_t)frames[job[0]].nf_cap, job.size() + rest.size()});
+    const size_t nf = most >= 4 ? 4 : most >= 2 ? 2 : 1;
+    for (size_t q = 0; job.size() < nf; ++q)
+        job.push_back(rest[q]);
+    return job;
+}
+
 int build_launch(const std::vector<FramePrep> &frames, HostLaunch &hl)
 {
     hl = HostLaunch{};
     std::map<int, std::vector<BfJob>> groups;
     std::map<int, size_t> group_smem;
     std::vector<char> taken(frames.size(), 0);
-    // frames riding in another frame's job (the lead, the first of them, carries
-    // the job's ingest)
+    // frames riding in another frame's job (the lead carries the job's ingest)
     std::vector<char> member(frames.size(), 0);
     std::vector<std::vector<size_t>> partners(frames.size());
     for (size_t fi = 0; fi < frames.size(); ++fi) {
         if (taken[fi])
             continue;
-        const FramePrep &f = frames[fi];
-        taken[fi] = 1;
         // partner frames of the same plan, if any: all ride in one job (1, 2 or 4 frames)
-        const FramePrep *more[kMaxFramesPerJob - 1] = {};
-        const int cap = max_frames_per_job(f);
-        std::vector<size_t> cand;
-        for (size_t gi = fi + 1; gi < frames.size() && (int)cand.size() + 1 < cap; ++gi)
-            if (!taken[gi] && shareable(f, frames[gi]))
-                cand.push_back(gi);
-        const int avail = (int)cand.size() + 1;
-        int nf = avail >= 4 ? 4 : avail >= 2 ? 2 : 1;
-        const int box_nf = nf > 1 ? interleaved_box(f.plan->wmax, nf, f.prec) : 0;
+        std::vector<size_t> job = job_frames(frames, taken, fi);
+        int nf = (int)job.size();
+        int box_nf = 0;
         CUtensorMap map;
-        if (nf > 1 && job_map(f, nf, box_nf, map) != BF_OK)
-            nf = 1;  // no interleaved map: every frame alone
+        if (nf > 1) {
+            const FramePrep &l = frames[job[0]];
+            box_nf = interleaved_box(l.plan->wmax, nf, l.prec);
+            if (job_map(l, nf, box_nf, map) != BF_OK) {  // no interleaved map: every frame alone
+                job = {fi};
+                nf = 1;
+            }
+        }
+        const size_t lead = job[0];
+        const FramePrep &f = frames[lead];
         if (nf == 1) {
             int rc = job_map(f, 1, f.plan->box, map);
             if (rc)
                 return rc;
         }
+        const FramePrep *more[kMaxFramesPerJob - 1] = {};
+        taken[lead] = 1;
         for (int q = 0; q < nf - 1; ++q) {
-            more[q] = &frames[cand[q]];
-            taken[cand[q]] = 1;
-            member[cand[q]] = 1;
-            partners[fi].push_back(cand[q]);
+            more[q] = &frames[job[q + 1]];
+            taken[job[q + 1]] = 1;
+            member[job[q + 1]] = 1;
+            partners[lead].push_back(job[q + 1]);
         }
         const bf_handle *h = f.h;
         const Plan *p = f.plan;
@@ -1762,7 +1789,7 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
     b->frames.resize(n);
     // frames of the batch with the same plan and combiners; every frame's arguments are
     // checked before its angles are read
-    std::map<JobKey, int> peers;
+    std::map<JobKey, std::pair<int, int>> peers;  // (frames, of these prepared)
     int dev = -1;
     for (int i = 0; i < n; ++i) {
         const bf_frame &f = frames[i];
@@ -1778,14 +1805,15 @@ BF_API int bf_batch_create(const bf_frame *frames, int32_t n, bf_batch **out)
         int rc = check_frame_args(f.h, f.n_samples, f.angles_rad, f.n_angles, f.mode_and_flags);
         if (rc)
             return fail(rc, "frame %d: %s", i, g_err.c_str());
-        peers[job_key(f)] += 1;
+        peers[job_key(f)].first += 1;
     }
     for (int i = 0; i < n; ++i) {
         const bf_frame &f = frames[i];
-        const int same = peers[job_key(f)];
+        auto &p = peers[job_key(f)];
+        const int same = p.first, index = p.second++;
         int rc = prepare_frame(f.h, f.rf_dev, f.n_samples, f.angles_rad, f.n_angles,
                                f.mode_and_flags, f.out_dev, b->scratch[i], b->frames[i],
-                               same > 1 ? kMaxFramesPerJob : 1, PlanWish{-1, same});
+                               same > 1 ? kMaxFramesPerJob : 1, PlanWish{-1, same, false, index});
         if (rc)
             return fail(rc, "frame %d: %s", i, g_err.c_str());
     }

@@ -3,6 +3,8 @@
 // the rules can be checked on a machine without a GPU.
 #pragma once
 
+#include <algorithm>
+
 #include "bf_internal.h"
 
 namespace bfi {
@@ -49,6 +51,21 @@ inline int rule_config(int prec, int ns, int na, int tiles, int sms, bool alone,
     if (!iq && na == 1 && (peers == 6 || peers == 7))
         return 0;
     return iq ? 4 : 6;
+}
+
+// Frames the pairs buffer of frame `index` of `peers` (0 <= index < peers; < 0: not known)
+// has room for, in jobs of up to cap: the frame that leads a job holds the pairs of all of
+// it, so that cap frames need 2 cap - 1 rooms together instead of cap^2.  fixed: the launch
+// is made of just these frames in this order (a batch); otherwise (the serving engine) the
+// frames behind the last whole four, too few for one, and pairs may meet others.
+inline int pairs_room(int cap, int index, int peers, bool fixed)
+{
+    if (index < 0 || cap == 1 || (!fixed && (cap == 2 || peers < cap)))
+        return cap;
+    const int first = index / cap * cap, n = std::min(cap, peers - first);
+    if (n == cap)
+        return index == first ? cap : 1;
+    return !fixed || (n >= 2 && index == first) ? 2 : 1;
 }
 
 }  // namespace bfi

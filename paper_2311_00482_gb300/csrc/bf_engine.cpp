@@ -29,6 +29,7 @@
 #include <string>
 #include <thread>
 
+#include "bf_choice.h"
 #include "bf_engine.h"
 #include "bf_ptr.h"
 
@@ -336,10 +337,12 @@ public:
     // request gets its ticket but is queued by flush() once its copy is
     // enqueued.  Other sources are copied (and queued) at once.
     // dest (optional): where the batch delivers the result (see Request::dest).
+    // peers, index: the frames submitted together with this one, and its place among them.
     int submit(bf_handle *h, const int16_t *rf, int ns, const double *angles, int na,
                uint32_t flags, uint64_t *ticket, bool wait_copy = true,
                std::vector<Deferred> *defer = nullptr, float *dest = nullptr,
-               uint64_t dest_group = 0, const CopyRoute *dest_route = nullptr, int peers = 1);
+               uint64_t dest_group = 0, const CopyRoute *dest_route = nullptr, int peers = 1,
+               int index = -1);
     // a fresh id for the destinations of one bf_submit_many_into call
     uint64_t next_dest_group() { return next_group_.fetch_add(1) + 1; }
     int flush(std::vector<Deferred> &defer);
@@ -391,7 +394,7 @@ public:
 private:
     void loop();
     void launch(std::vector<std::shared_ptr<Request>> &reqs);
-    std::unique_ptr<Slot> take_slot();
+    std::unique_ptr<Slot> take_slot(size_t need);
     void put_free(std::unique_ptr<Slot> s);  // under mu_
 
     int device_;
@@ -417,14 +420,19 @@ private:
     ResPool res_pool_;
 };
 
-std::unique_ptr<Slot> Engine::take_slot()
+std::unique_ptr<Slot> Engine::take_slot(size_t need)
 {
     if (free_.empty())
         return std::make_unique<Slot>();
-    // the largest free slot (the least growth); sizes kept beside the list so
+    // the smallest free slot of at least `need` bytes, else the largest (the least growth):
+    // frames with room for a whole job's pairs keep theirs; sizes kept beside the list so
     // that the choice reads one contiguous array
-    const size_t i = (size_t)(std::max_element(free_bytes_.begin(), free_bytes_.end()) -
-                              free_bytes_.begin());
+    size_t i = 0;
+    for (size_t k = 1; k < free_bytes_.size(); ++k) {
+        const bool fits = free_bytes_[k] >= need, had = free_bytes_[i] >= need;
+        if (fits != had ? fits : (free_bytes_[k] < free_bytes_[i]) == fits && free_bytes_[k] != free_bytes_[i])
+            i = k;
+    }
     std::unique_ptr<Slot> s = std::move(free_[i]);
     free_[i] = std::move(free_.back());
     free_.pop_back();
@@ -441,7 +449,8 @@ void Engine::put_free(std::unique_ptr<Slot> s)
 
 int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles, int na,
                    uint32_t flags, uint64_t *ticket, bool wait_copy, std::vector<Deferred> *defer,
-                   float *dest, uint64_t dest_group, const CopyRoute *dest_route, int peers)
+                   float *dest, uint64_t dest_group, const CopyRoute *dest_route, int peers,
+                   int index)
 {
     int rc = check_frame_args(h, ns, angles, na, flags);
     if (rc)
@@ -462,53 +471,55 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
         std::lock_guard<std::mutex> lk(mu_);
         if (live_ >= max_live_)
             return fail(BF_EAGAIN, "%d requests in flight", live_);
-        req->slot = take_slot();
         live_ += 1;
     }
-    Slot &s = *req->slot;
-    const size_t before = s.device_bytes();
-    // admission by device memory: the slot may have to grow
     const int prec = frame_prec(flags);
     Plan *plan = nullptr;
     rc = handle_plan(h, ns, angles, na, flags, &plan,
                      PlanWish{-1, peers, !sharing_modes(flags)});
-    // staged pairs: room for the frames of a multi-frame job this frame may lead
-    const int cap = plan ? job_frames_cap(plan, flags, kMaxFramesPerJob) : 1;
-    size_t need = rf_bytes + out_bytes +
-                  (size_t)cap * na * h->g.ne * (plan ? plan->nsp : 0) * pair_bytes(prec);
-    if ((flags & BF_OUT_MASK) != BF_OUT_RF)
-        need += out_bytes * ((flags & BF_OUT_MASK) == BF_OUT_LOGDB ? 2 : 1);
-    auto give_back = [&](int code) {
+    if (rc) {
         std::lock_guard<std::mutex> lk(mu_);
-        used_ -= before;
-        used_ += s.device_bytes();
-        put_free(std::move(req->slot));
         live_ -= 1;
-        return code;
-    };
-    if (rc)
-        return give_back(rc);
+        return rc;
+    }
+    // admission by device memory: a slot, which may have to grow.  Staged pairs: room for
+    // the frames of a multi-frame job this frame may lead; a frame of a four leads a pair
+    // where there is no memory for the four.
+    int room = pairs_room(job_frames_cap(plan, flags, kMaxFramesPerJob), index, peers, false);
+    size_t base = rf_bytes + out_bytes;
+    if ((flags & BF_OUT_MASK) != BF_OUT_RF)
+        base += out_bytes * ((flags & BF_OUT_MASK) == BF_OUT_LOGDB ? 2 : 1);
+    const size_t frame_pairs = (size_t)na * h->g.ne * plan->nsp * pair_bytes(prec);
+    size_t before = 0, reserved = 0;
     {
         std::lock_guard<std::mutex> lk(mu_);
-        const size_t grow = need > before ? need - before : 0;
-        if (grow && used_ + grow > budget_) {
+        for (;; room = 2) {
+            const size_t need = base + (size_t)room * frame_pairs;
+            req->slot = take_slot(need);
+            before = req->slot->device_bytes();
+            reserved = need > before ? need - before : 0;
+            int refused = BF_OK;
+            if (reserved && used_ + reserved > budget_) {
+                refused = fail(BF_EAGAIN, "device memory budget reached (%zu of %zu bytes in use)", used_,
+                               budget_);
+            } else if (reserved) {
+                size_t fr = 0, tot = 0;
+                cudaSetDevice(device_);
+                if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || fr < reserved + ((size_t)256 << 20))
+                    refused = fail(BF_EAGAIN, "not enough free device memory for a request (%zu needed)",
+                                   reserved);
+            }
+            if (!refused)
+                break;
             put_free(std::move(req->slot));
-            live_ -= 1;
-            return fail(BF_EAGAIN, "device memory budget reached (%zu of %zu bytes in use)", used_,
-                        budget_);
-        }
-        if (grow) {
-            size_t fr = 0, tot = 0;
-            cudaSetDevice(device_);
-            if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || fr < grow + ((size_t)256 << 20)) {
-                put_free(std::move(req->slot));
+            if (room <= 2) {
                 live_ -= 1;
-                return fail(BF_EAGAIN, "not enough free device memory for a request (%zu needed)",
-                            grow);
+                return refused;
             }
         }
-        used_ += grow;  // reserved; corrected after allocation
+        used_ += reserved;  // corrected after allocation
     }
+    Slot &s = *req->slot;
     cudaSetDevice(device_);
     rc = s.rf.ensure(rf_bytes);
     if (!rc)
@@ -519,11 +530,11 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
         rc = fail(BF_ECUDA, "cudaEventCreate");
     if (!rc)
         rc = prepare_frame(h, (const int16_t *)s.rf.p, ns, angles, na, flags, (float *)s.out.p,
-                           s.scratch, req->fp, kMaxFramesPerJob, PlanWish{-1, peers}, peers == 1);
+                           s.scratch, req->fp, kMaxFramesPerJob, PlanWish{-1, peers, false, -1, room},
+                           peers == 1);
     if (rc) {
         std::lock_guard<std::mutex> lk(mu_);
-        const size_t grow = need > before ? need - before : 0;
-        used_ -= grow;
+        used_ -= reserved;
         used_ -= before;
         used_ += s.device_bytes();
         put_free(std::move(req->slot));
@@ -540,8 +551,7 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
         // copied with the call's other frames: registered now, queued by flush()
         {
             std::lock_guard<std::mutex> lk(mu_);
-            const size_t grow = need > before ? need - before : 0;
-            used_ -= grow;
+            used_ -= reserved;
             used_ -= before;
             used_ += s.device_bytes();
             req->ticket = next_ticket_++;
@@ -570,8 +580,7 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
         e = cudaEventSynchronize(s.h2d);
     {
         std::lock_guard<std::mutex> lk(mu_);
-        const size_t grow = need > before ? need - before : 0;
-        used_ -= grow;
+        used_ -= reserved;
         used_ -= before;
         used_ += s.device_bytes();
         if (e != cudaSuccess) {
@@ -1131,7 +1140,7 @@ static int submit_many(bf_handle *h, int32_t n, const int16_t *const *rf, int32_
             }
             rc = eng->submit(h, rf[k], n_samples, angles_rad, n_angles, flags, tickets_out + k,
                              false, &defer, outs ? outs[k] : nullptr, group,
-                             group ? &one_route : nullptr, n);
+                             group ? &one_route : nullptr, n, k);
             if (rc)
                 break;
         }

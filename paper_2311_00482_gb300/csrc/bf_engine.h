@@ -133,7 +133,7 @@ struct FramePrep {
     float *y = nullptr, *env = nullptr;
     unsigned *maxbits = nullptr;
     FrameScratch *scratch = nullptr;
-    int nf_cap = 1;  // frames of a job this frame may lead (its pairs buffer holds that many)
+    int nf_cap = 1;  // frames of a job this frame may lead: its pairs buffer holds that many
 };
 
 struct HostLaunch {
@@ -260,6 +260,8 @@ struct PlanWish {
     int cfg = -1;   // a configuration of kTileConfigs, or < 0: by the rules of choose_cfg
     int peers = 1;  // frames of this plan and combiners submitted together (see bf_choice.h)
     bool alone = false;  // the frame shares its plan with no other: RF frames take solo tiles
+    int index = -1;  // the frame's place among its peers, in a launch of just these (or < 0)
+    int room = 0;    // frames its pairs buffer holds at most (0: by pairs_room)
 };
 // Plan of a frame with these arguments (`flags`: its mode and precision bits).
 // BF_TILE_ROWS and bf_autotune's choice for the workload come before the rules; a
@@ -278,7 +280,8 @@ size_t frame_out_bytes(const bf_handle *h, uint32_t flags);
 int frame_prec(uint32_t flags);
 // nf_cap: frames of one plan a later build_launch may put in one job with
 // this frame (1: alone, as a single bf_beamform call); the frame's scratch
-// is sized for the multi-frame jobs its plan and combiners allow up to that.
+// is sized for the multi-frame jobs its plan and combiners allow up to that, or for what
+// its place among its peers asks for (PlanWish).
 // With nf_cap 1, or combiners no job shares, the plan is a solo plan where one
 // applies; late_solo: also find that plan for a frame that may turn out alone
 // (use_solo_plans).

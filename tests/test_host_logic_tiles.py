@@ -22,10 +22,16 @@ def choose(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-I" + CSRC, "-I" + inc,
                     os.path.join(ROOT, "tests", "tile_choice_check.cpp"), "-o", exe], check=True)
 
+    def rooms(cap, peers, fixed):
+        args = [str(int(x)) for x in (cap, peers, fixed)]
+        out = subprocess.run([exe, *args], check=True, capture_output=True, text=True).stdout
+        return [int(x) for x in out.split()]
+
     def run(prec, nx, nz, peers, ns=2048, na=1, sms=152, alone=False, shares=True):
         args = [str(int(x)) for x in (prec, ns, na, nx, nz, sms, alone, shares, peers)]
         return int(subprocess.run([exe, *args], check=True, capture_output=True, text=True).stdout)
 
+    run.rooms = rooms
     return run
 
 
@@ -61,3 +67,25 @@ def test_combiners_that_share_no_job(choose):
 @pytest.mark.parametrize("peers", [1, 16])
 def test_lone_frames_split_by_their_own_tiles(choose, nx, nz, split, peers):
     assert choose(F32, nx, nz, peers, alone=True) == SOLO + split
+
+
+@pytest.mark.parametrize("cap", [1, 2, 4])
+@pytest.mark.parametrize("peers", range(1, 14))
+def test_rooms_hold_the_jobs_of_a_batch(choose, cap, peers):
+    """Frames join jobs in order, fours, then pairs, then alone: the first of a job holds it."""
+    want, left = [], peers
+    while left:
+        nf = max(n for n in (1, 2, 4) if n <= min(cap, left))
+        want += [nf] + [1] * (nf - 1)
+        left -= nf
+    assert choose.rooms(cap, peers, True) == want
+
+
+@pytest.mark.parametrize("peers", range(4, 21))
+def test_rooms_of_served_frames(choose, peers):
+    """No more than two frames' pairs each on average, and a lead for every four."""
+    rooms = choose.rooms(4, peers, False)
+    assert sum(rooms) <= 2 * peers
+    assert rooms[:peers // 4 * 4] == [4, 1, 1, 1] * (peers // 4)
+    assert rooms[peers // 4 * 4:] == [2] * (peers % 4)
+    assert choose.rooms(2, peers, False) == [2] * peers
