@@ -1433,7 +1433,9 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
         rc = fft_tables(nk, tk);
     const size_t nf = (size_t)nt / 2 + 1, img = (size_t)ne * n_samples;
     if (!rc)
-        rc = h->fk_D.ensure((size_t)n_angles * nk * (nf + (regs ? fk_pitch(nt) : 0)) * sizeof(float2));
+        rc = h->fk_D.ensure((regs ? fk_angles(n_angles, nt, nk) * nf + (size_t)n_angles * fk_pitch(nt)
+                                  : n_angles * nf) *
+                            nk * sizeof(float2));
     if (!rc)
         rc = h->fk_spec.ensure((size_t)(nt / 2) * nk * sizeof(float2));
     if (!rc && stage == BF_OUT_LOGDB)
@@ -1495,7 +1497,7 @@ BF_API int bf_fkmig(bf_handle *h, const int16_t *rf_dev, int32_t n_samples,
     J.map_aw = (const float2 *)h->fk_aw.p;
     if (regs) {
         J.ptw = (const float2 *)tt->tw.p;
-        J.E = J.D + (size_t)n_angles * nf * nk;
+        J.E = J.D + (size_t)fk_angles(n_angles, nt, nk) * nf * nk;
     } else {
         J.tw_t = (const float2 *)tt->tw.p;
         J.tw_k = (const float2 *)tk->tw.p;

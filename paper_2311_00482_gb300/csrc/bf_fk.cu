@@ -307,9 +307,18 @@ cudaError_t launch_fkmig16(const FkJob &J, cudaStream_t st)
                                 map_t<9>, map_t<10>, map_t<11>, map_t<12>};
     static const Stage depth[] = {depth_t<5>, depth_t<6>, depth_t<7>, depth_t<8>, depth_t<9>,
                                   depth_t<10>, depth_t<11>, depth_t<12>, depth_t<13>};
-    cudaError_t e = time[J.lgt - 5](J, st);
-    if (e == cudaSuccess)
-        e = rows[J.lgk - 5](J, st);
+    cudaError_t e = cudaSuccess;
+    const int held = fk_angles(J.na, J.nt, J.nk);
+    for (int a = 0; a < J.na && e == cudaSuccess; a += held) {  // D is written anew for each
+        FkJob g = J;
+        g.na = J.na - a < held ? J.na - a : held;
+        g.rf += (size_t)a * J.ne * J.ns;
+        g.beta += (size_t)a * J.ne * 2;
+        g.E += (size_t)a * J.nk * fk_pitch(J.nt);
+        e = time[J.lgt - 5](g, st);
+        if (e == cudaSuccess)
+            e = rows[J.lgk - 5](g, st);
+    }
     if (e == cudaSuccess)
         e = map[J.lgk - 5](J, st);
     if (e == cudaSuccess)

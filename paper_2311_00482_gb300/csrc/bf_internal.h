@@ -91,6 +91,15 @@ __host__ __device__ inline int fk_kx_bin(int lgk, int p)
     return fft16_bin(lgk, p % T, p / T);
 }
 
+// Angles whose spectra before the lateral transforms are held at a time: 64 MB of them (they
+// then stay in L2 between the two launches), so that the spectra after them are the only
+// ones held of every angle.
+__host__ __device__ constexpr int fk_angles(int na, int nt, int nk)
+{
+    const size_t one = ((size_t)nt / 2 + 1) * nk * 8, n = ((size_t)64 << 20) / one;
+    return n < 1 ? 1 : n < (size_t)na ? (int)n : na;
+}
+
 // Device-side error bits (written with atomicOr into a per-launch word).
 enum DevErr : int { kErrTimeout = 1, kErrWindow = 2, kErrConfig = 4 };
 
@@ -196,7 +205,9 @@ struct DemodJob {
 // Plane-wave f-k migration of one frame (all its angles): see bf_fkmig.
 struct FkJob {
     const int16_t *rf;    // [na][ne][ns]
-    float2 *D;            // [na][nt/2 + 1][nk] per-angle spectra (time, then lateral transform)
+    // [na][nt/2 + 1][nk] per-angle spectra (time, then lateral transform); launch_fkmig16:
+    // of fk_angles angles at a time
+    float2 *D;
     float2 *spec;         // [nt/2][nk] migrated spectrum, rows Kz bin q = 1 .. nt/2
     float *img;           // [ne][ns] magnitude image
     unsigned *maxbits;    // image maximum (float bits) for the log stage, or null
