@@ -366,10 +366,14 @@ BF_API int bf_plan_info(bf_handle *h, int32_t n_samples, const double *angles_ra
  * this workload (grid of the handle, n_samples, angles, the combiner and
  * precision bits of mode_and_flags; the output stage is ignored) under each
  * tile configuration the library knows (rows per thread x channels per
- * pipeline stage), on synthetic zero records, and keeps the fastest: later
- * bf_beamform, bf_submit and bf_batch_create work on this workload uses it.
+ * pipeline stage), on synthetic zero records, and keeps the fastest for later
+ * bf_beamform, bf_submit and bf_batch_create work on this workload whose
+ * frames share jobs, and for IQ frames.  An RF frame that shares its plan with
+ * no other runs on tiles of its own (see bf_plan_info) and keeps them, unless
+ * frames is 1 or the combiners share no job (BF_CF, BF_PDAS): then these tiles
+ * are timed as well, and the fastest of all serves such frames.
  * Synchronous; allocates scratch for the frames while it runs.  Optional
- * outputs: the chosen rows per thread and stage bytes, and the median
+ * outputs: rows per thread and stage bytes of the fastest tile configuration, and the median
  * beamforming time in microseconds of every candidate (n_candidates
  * entries; -1 where a configuration does not fit).  Two-row tiles (16 rows,
  * up to four frames of one workload per job sharing every delay) serve DAS

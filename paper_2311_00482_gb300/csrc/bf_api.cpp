@@ -249,23 +249,32 @@ static int forced_cfg()
     return rows == 8 ? 3 : rows == 4 ? 0 : rows == 2 ? 6 : -1;
 }
 
-static PlanKey tuned_key(PlanKey k)
+// bf_autotune's choice for a workload, or -1.  lone: for RF frames that share their plan
+// with no other; two-row tiles only for frames that can take them.
+static int tuned_cfg(const bf_handle *h, PlanKey key, bool lone, bool narrow_ok)
 {
-    k.cfg = 0;
-    return k;
+    key.cfg = lone ? 1 : 0;
+    auto it = h->tuned.find(key);
+    if (it == h->tuned.end())
+        return -1;
+    const int c = it->second;
+    return c < kNumTileConfigs && kTileConfigs[c].rows == 2 && !narrow_ok ? (lone ? -1 : 0) : c;
 }
 
 // Configuration of a workload (of kTileConfigs, or a solo one): BF_TILE_ROWS, else
-// what bf_autotune measured fastest for it, else by the frames that share it
+// what bf_autotune measured fastest for it, else (by_rule) by the frames that share it
 // (bf_choice.h).
-static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w, bool narrow_ok)
+static int choose_cfg(const bf_handle *h, const PlanKey &key, const PlanWish &w, bool narrow_ok,
+                      bool *by_rule)
 {
+    *by_rule = false;
     const int forced = forced_cfg();
     if (forced >= 0)
         return forced;
-    auto it = h->tuned.find(key);
-    if (it != h->tuned.end())
-        return it->second;
+    const int tuned = tuned_cfg(h, key, w.alone && key.prec != kPrecIQ, narrow_ok);
+    if (tuned >= 0)
+        return tuned;
+    *by_rule = true;
     return rule_config(key.prec, key.ns, (int)key.angles.size(), image_tiles(h->g.nx, h->g.nz), h->sms,
                        w.alone, narrow_ok, w.peers);
 }
@@ -301,9 +310,9 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
     const bool narrow_ok = sharing_modes(flags);
     PlanKey key{ns, prec, std::vector<double>(angles, angles + na), 0};
     std::lock_guard<std::mutex> lk(h->mu);
-    key.cfg = (cfg >= 0 && cfg < kNumTileConfigs) ? cfg : choose_cfg(h, key, wish, narrow_ok);
-    const bool solo = key.cfg >= kSoloConfig;
-    if (!solo && kTileConfigs[key.cfg].rows == 2 && !narrow_ok) {
+    bool by_rule = false;
+    key.cfg = (cfg >= 0 && cfg < kNumConfigs) ? cfg : choose_cfg(h, key, wish, narrow_ok, &by_rule);
+    if (key.cfg < kSoloConfig && kTileConfigs[key.cfg].rows == 2 && !narrow_ok) {
         if (cfg >= 0)
             return fail(BF_EINVAL, "two-row tiles serve DAS / DMAS and IQ-DAS / BB-DMAS only");
         key.cfg = 0;
@@ -313,15 +322,28 @@ int handle_plan(bf_handle *h, int ns, const double *angles, int na, uint32_t fla
         *out = it->second.get();
         return BF_OK;
     }
-    // the default tiles' window bounds the pixel spacing, whichever tiles a rule chose
-    const TileConfig tc = kTileConfigs[solo ? 0 : key.cfg];
     int wmax = 0, box = 0, group = 0;
     auto fits = [&](const TileConfig &t) {
         tile_window(h->g, key.angles, prec, tile_rows(t.rows), 1, wmax, box);
         group = stage_channels(wmax, prec, t.rows, t.stage_bytes, h->g.ne);
         return beamform_smem_bytes(wmax, group, prec, 1, t.rows) <= (size_t)kMaxSmemPerCta;
     };
-    const bool by_rule = cfg < 0 && forced_cfg() < 0 && h->tuned.find(tuned_key(key)) == h->tuned.end();
+    // the default tiles' window bounds the pixel spacing, whichever tiles a rule chose; a
+    // workload that was tuned to smaller tiles keeps them where the default does not fit
+    if (by_rule && !fits(kTileConfigs[0])) {
+        const int tuned = tuned_cfg(h, key, false, narrow_ok);
+        if (tuned > 0) {
+            key.cfg = tuned;
+            by_rule = false;
+            it = h->plans.find(key);
+            if (it != h->plans.end()) {
+                *out = it->second.get();
+                return BF_OK;
+            }
+        }
+    }
+    const bool solo = key.cfg >= kSoloConfig;
+    const TileConfig tc = kTileConfigs[solo ? 0 : key.cfg];
     if ((by_rule && !fits(kTileConfigs[0])) || !fits(tc))
         return fail(BF_EINVAL,
                     "pixel spacing too coarse for the sample rate: one tile needs %d samples per channel",
@@ -1676,7 +1698,8 @@ BF_API int bf_plan_info(bf_handle *h, int32_t n_samples, const double *angles_ra
 // Autotuner: times the beamforming launches of `frames` copies of this
 // workload under every tile configuration (synthetic zero records: the work
 // does not depend on the data) and keeps the fastest for the handle's later
-// work on it.
+// work on it.  A lone frame, and frames whose combiners share no job, are also
+// timed on the solo tiles; what is fastest then serves the handle's lone frames.
 BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad,
                        int32_t n_angles, uint32_t flags, int32_t frames, int32_t *rows_out,
                        int32_t *stage_bytes_out, float *candidate_us, int32_t n_candidates)
@@ -1707,9 +1730,10 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
     if (e == cudaSuccess)
         e = cudaMemsetAsync(rf.p, 0, rf_bytes, st);
     std::vector<FrameScratch> scratch(frames);
-    std::vector<float> best_us(kNumTileConfigs, -1.f);
-    int best = -1;
-    for (int c = 0; c < kNumTileConfigs && e == cudaSuccess && !rc; ++c) {
+    const bool lone = frame_prec(flags) != kPrecIQ && (frames == 1 || !sharing_modes(flags));
+    std::vector<float> best_us(kNumConfigs, -1.f);
+    int best = -1, best_lone = -1;  // of the tile configurations; of these and the solo ones
+    for (int c = 0; c < (lone ? kNumConfigs : kNumTileConfigs) && e == cudaSuccess && !rc; ++c) {
         std::vector<FramePrep> fr(frames);
         int prc = BF_OK;
         for (int i = 0; i < frames && !prc; ++i)
@@ -1740,8 +1764,10 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
             break;
         std::sort(t.begin(), t.end());
         best_us[c] = t[t.size() / 2];
-        if (best < 0 || best_us[c] < best_us[best])
+        if (c < kNumTileConfigs && (best < 0 || best_us[c] < best_us[best]))
             best = c;
+        if (best_lone < 0 || best_us[c] < best_us[best_lone])
+            best_lone = c;
     }
     for (auto &m : marks)
         if (m)
@@ -1759,6 +1785,9 @@ BF_API int bf_autotune(bf_handle *h, int32_t n_samples, const double *angles_rad
         PlanKey key{n_samples, frame_prec(flags),
                     std::vector<double>(angles_rad, angles_rad + n_angles), 0};
         h->tuned[key] = best;
+        key.cfg = 1;  // see tuned_cfg
+        if (lone)
+            h->tuned[key] = best_lone;
     }
     h->call.clear();  // bf_beamform's last call may have used another configuration
     if (rows_out)

@@ -231,7 +231,8 @@ struct bf_handle {
     std::map<bfi::PlanKey, std::unique_ptr<bfi::Plan>> plans;
     // their angle tables (key prec = cfg = 0)
     std::map<bfi::PlanKey, std::shared_ptr<bfi::AngleTablesDev>> angle_tabs;
-    std::map<bfi::PlanKey, int> tuned;  // tile configuration bf_autotune chose (key cfg = 0)
+    // configurations bf_autotune chose (key cfg = 0; for lone frames 1)
+    std::map<bfi::PlanKey, int> tuned;
     bfi::FrameScratch scratch;     // bf_beamform
     bfi::DeviceLaunch launch;      // bf_beamform
     bfi::CallCache call;           // bf_beamform's last call

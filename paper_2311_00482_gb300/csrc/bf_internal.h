@@ -44,9 +44,9 @@ constexpr TileConfig kTileConfigs[] = {{4, 24 << 10}, {4, 16 << 10}, {4, 32 << 1
 __host__ __device__ constexpr int stages_for_rows(int rows) { return rows == 2 ? 2 : 3; }
 constexpr int kNumTileConfigs = 7;
 // Solo tiles (bf_solo.cu): frames that share their plan with no other frame.
-// Configuration kSoloConfig + k runs SPLIT = 2^k: tiles of 16 / SPLIT rows.  Not
-// among the autotuner's candidates; angles share a stage, at most kSoloAngles.
-constexpr int kSoloConfig = kNumTileConfigs, kSoloAngles = 4;
+// Configuration kSoloConfig + k runs SPLIT = 2^k: tiles of 16 / SPLIT rows; angles share a
+// stage, at most kSoloAngles.
+constexpr int kSoloConfig = kNumTileConfigs, kNumConfigs = kSoloConfig + 3, kSoloAngles = 4;
 constexpr int kSoloStages = 2, kSoloStageBytes = 33 << 10;
 // Record of one (step, tile): 8 masks of fully and 8 of partly counted channels,
 // then the window starts [angle][run of channels]; [step][tile] in the plan's table.
