@@ -407,12 +407,13 @@ BF_API int bf_selftest_wait(int64_t timeout_us);
  * magnitude along z, through the [f0, 3 f0] band-pass when bandpass != 0
  * (the DMAS image); z0_m, z1_m: the grid's depth range (sets the band).
  * Limits: nz a power of two <= 4096 and nx * nz <= 2^20; BF_EINVAL beyond.
- * Scratch: a fixed 4 MiB array inside the library (held by every GPU that
+ * Scratch: a fixed array of 4.4 MB inside the library (held by every GPU that
  * loads it until exit); no cudaMalloc, cudaFree or other allocating routine is
  * called.  Every call shares that array and leaves its contents behind, so
  * calls that overlap on the GPU (different streams, no ordering) race.  The
- * first call on a device looks up the array's device address; make that first
- * call before any stream capture.  Enqueued on cuda_stream (NULL: default
+ * first call on a device looks up the array's device address and sends 0.25 MB
+ * of constants ahead of its kernels on cuda_stream; make that first call before
+ * any stream capture.  Enqueued on cuda_stream (NULL: default
  * stream); returns after enqueueing. */
 BF_API int bf_logdb_static(const float *y_dev, int32_t nx, int32_t nz, double z0_m, double z1_m,
                            double f0_hz, double c_mps, int32_t bandpass, float *db_dev,

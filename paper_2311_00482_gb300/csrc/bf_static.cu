@@ -9,7 +9,7 @@
 // its -70 dB log-compressed envelope into the caller's output, and its only
 // scratch (the envelope image and its maxima) is a fixed array compiled
 // into this library.  Every GPU that loads the library holds that array
-// (kStaticPixels floats, 4 MiB) until the process exits.
+// (kStaticPixels floats, the maxima and the twiddles: 4.4 MB) until the process exits.
 //
 // The computation is the one of the BF_OUT_LOGDB stage of bf_beamform: the
 // analytic-signal magnitude along depth, optionally through the [f0, 3 f0]
@@ -135,8 +135,10 @@ __global__ void __launch_bounds__(256) static_envelope_kernel(const float *__res
     block_max(lmax, maxima + blockIdx.x);
 }
 
-// Sixteen pixels per thread; the image's maximum from the envelope CTAs' maxima.
-constexpr int kStaticLogPixels = 4096;
+// The image's maximum from the envelope CTAs' maxima.  Four pixels per thread: a logarithm
+// is about forty instructions, so a 512 x 512 image wants all SMs (whole pass 14.35 us at
+// sixteen pixels per thread, 13.5 at eight, 12.30 at four).
+constexpr int kStaticLogPixels = 1024;
 __global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict__ env, int n, int vec4,
                                                          const float *__restrict__ maxima, int nmax,
                                                          float *__restrict__ out, float dr)
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict
 #pragma unroll
     for (int w = 0; w < 8; ++w)
         peak = fmaxf(peak, red[w]);
-    // of the quotient, so that the image's scale cancels exactly and images of any scale
+    // 20 log10 of the quotient, so that the image's scale cancels exactly and images of any scale
     // lose nothing (a difference of two fast logarithms: 1e-5 dB at a scale of one, 1e-4 dB
     // at 2^-100)
     auto db = [&](float e) {
@@ -161,13 +163,10 @@ __global__ void __launch_bounds__(256) static_log_kernel(const float *__restrict
     };
     const int base = blockIdx.x * kStaticLogPixels;
     if (vec4) {
-#pragma unroll
-        for (int u = 0; u < kStaticLogPixels / 1024; ++u) {
-            const int p = base + 4 * (threadIdx.x + 256 * u);
-            if (p < n) {
-                const float4 e = __ldcg(reinterpret_cast<const float4 *>(env + p));
-                *reinterpret_cast<float4 *>(out + p) = make_float4(db(e.x), db(e.y), db(e.z), db(e.w));
-            }
+        const int p = base + 4 * threadIdx.x;
+        if (p < n) {
+            const float4 e = __ldcg(reinterpret_cast<const float4 *>(env + p));
+            *reinterpret_cast<float4 *>(out + p) = make_float4(db(e.x), db(e.y), db(e.z), db(e.w));
         }
         return;
     }
