@@ -184,6 +184,16 @@ struct PinnedBuf {
     }
 };
 
+// Device bytes of a slot's buffers, or of what a request needs.
+struct SlotSizes {
+    size_t rf = 0, out = 0, pairs = 0, y = 0, env = 0;
+    size_t total() const { return rf + out + pairs + y + env; }
+    bool holds(const SlotSizes &n) const
+    {
+        return rf >= n.rf && out >= n.out && pairs >= n.pairs && y >= n.y && env >= n.env;
+    }
+};
+
 struct Slot {
     DevMem rf, out;
     FrameScratch scratch;
@@ -194,11 +204,11 @@ struct Slot {
         if (h2d)
             cudaEventDestroy(h2d);
     }
-    size_t device_bytes() const
+    SlotSizes sizes() const
     {
-        return rf.bytes + out.bytes + scratch.pairs.bytes + scratch.y.bytes + scratch.env.bytes +
-               scratch.maxbits.bytes;
+        return {rf.bytes, out.bytes, scratch.pairs.bytes, scratch.y.bytes, scratch.env.bytes};
     }
+    size_t device_bytes() const { return sizes().total() + scratch.maxbits.bytes; }
 };
 
 // Device job lists, status word and events of one launched batch.
@@ -394,7 +404,7 @@ public:
 private:
     void loop();
     void launch(std::vector<std::shared_ptr<Request>> &reqs);
-    std::unique_ptr<Slot> take_slot(size_t need);
+    std::unique_ptr<Slot> take_slot(const SlotSizes *need);
     void put_free(std::unique_ptr<Slot> s);  // under mu_
 
     int device_;
@@ -403,7 +413,7 @@ private:
     std::deque<std::shared_ptr<Request>> pending_;
     std::deque<std::shared_ptr<Batch>> inflight_;
     std::vector<std::unique_ptr<Slot>> free_;
-    std::vector<size_t> free_bytes_;  // device bytes of free_[i]
+    std::vector<SlotSizes> free_sizes_;  // of free_[i]
     size_t used_ = 0, budget_ = 0;
     int live_ = 0;
     int max_batch_ = 64, max_inflight_ = 3, max_live_ = 512;
@@ -420,30 +430,36 @@ private:
     ResPool res_pool_;
 };
 
-std::unique_ptr<Slot> Engine::take_slot(size_t need)
+std::unique_ptr<Slot> Engine::take_slot(const SlotSizes *need)
 {
     if (free_.empty())
         return std::make_unique<Slot>();
-    // the smallest free slot of at least `need` bytes, else the largest (the least growth):
-    // frames with room for a whole job's pairs keep theirs; sizes kept beside the list so
-    // that the choice reads one contiguous array
-    size_t i = 0;
-    for (size_t k = 1; k < free_bytes_.size(); ++k) {
-        const bool fits = free_bytes_[k] >= need, had = free_bytes_[i] >= need;
-        if (fits != had ? fits : (free_bytes_[k] < free_bytes_[i]) == fits && free_bytes_[k] != free_bytes_[i])
+    // The largest free slot (the least growth: a trace of mixed sizes settles on slots that
+    // hold them all; by best fit 10 kHz went from 10,000 to 4,760 frames/s and the 20 kHz
+    // tail doubled).  need: a frame that leads no job; the smallest slot whose buffers all
+    // hold it, so that those with room for a job stay for the frames that lead one.
+    // Sizes kept beside the list so that the choice reads one contiguous array.
+    size_t i = free_.size(), largest = 0;
+    for (size_t k = 0; k < free_.size(); ++k) {
+        const size_t t = free_sizes_[k].total();
+        if (t > free_sizes_[largest].total())
+            largest = k;
+        if (need && free_sizes_[k].holds(*need) && (i == free_.size() || t < free_sizes_[i].total()))
             i = k;
     }
+    if (i == free_.size())
+        i = largest;
     std::unique_ptr<Slot> s = std::move(free_[i]);
     free_[i] = std::move(free_.back());
     free_.pop_back();
-    free_bytes_[i] = free_bytes_.back();
-    free_bytes_.pop_back();
+    free_sizes_[i] = free_sizes_.back();
+    free_sizes_.pop_back();
     return s;
 }
 
 void Engine::put_free(std::unique_ptr<Slot> s)
 {
-    free_bytes_.push_back(s->device_bytes());
+    free_sizes_.push_back(s->sizes());
     free_.push_back(std::move(s));
 }
 
@@ -485,17 +501,19 @@ int Engine::submit(bf_handle *h, const int16_t *rf, int ns, const double *angles
     // admission by device memory: a slot, which may have to grow.  Staged pairs: room for
     // the frames of a multi-frame job this frame may lead; a frame of a four leads a pair
     // where there is no memory for the four.
-    int room = pairs_room(job_frames_cap(plan, flags, kMaxFramesPerJob), index, peers, false);
-    size_t base = rf_bytes + out_bytes;
-    if ((flags & BF_OUT_MASK) != BF_OUT_RF)
-        base += out_bytes * ((flags & BF_OUT_MASK) == BF_OUT_LOGDB ? 2 : 1);
+    const int cap = job_frames_cap(plan, flags, kMaxFramesPerJob);
+    int room = pairs_room(cap, index, peers, false);
+    const uint32_t stage = flags & BF_OUT_MASK;
+    SlotSizes want{rf_bytes, out_bytes, 0, stage != BF_OUT_RF && prec != kPrecIQ ? out_bytes : 0,
+                   stage == BF_OUT_LOGDB ? out_bytes : 0};
     const size_t frame_pairs = (size_t)na * h->g.ne * plan->nsp * pair_bytes(prec);
     size_t before = 0, reserved = 0;
     {
         std::lock_guard<std::mutex> lk(mu_);
         for (;; room = 2) {
-            const size_t need = base + (size_t)room * frame_pairs;
-            req->slot = take_slot(need);
+            want.pairs = (size_t)room * frame_pairs;
+            const size_t need = want.total();
+            req->slot = take_slot(room < cap ? &want : nullptr);
             before = req->slot->device_bytes();
             reserved = need > before ? need - before : 0;
             int refused = BF_OK;
