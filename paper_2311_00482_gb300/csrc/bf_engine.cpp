@@ -413,7 +413,8 @@ private:
     std::deque<std::shared_ptr<Request>> pending_;
     std::deque<std::shared_ptr<Batch>> inflight_;
     std::vector<std::unique_ptr<Slot>> free_;
-    std::vector<SlotSizes> free_sizes_;  // of free_[i]
+    std::vector<size_t> free_bytes_;     // device bytes of free_[i]
+    std::vector<SlotSizes> free_sizes_;  // by buffer
     size_t used_ = 0, budget_ = 0;
     int live_ = 0;
     int max_batch_ = 64, max_inflight_ = 3, max_live_ = 512;
@@ -438,20 +439,21 @@ std::unique_ptr<Slot> Engine::take_slot(const SlotSizes *need)
     // hold them all; by best fit 10 kHz went from 10,000 to 4,760 frames/s and the 20 kHz
     // tail doubled).  need: a frame that leads no job; the smallest slot whose buffers all
     // hold it, so that those with room for a job stay for the frames that lead one.
-    // Sizes kept beside the list so that the choice reads one contiguous array.
-    size_t i = free_.size(), largest = 0;
-    for (size_t k = 0; k < free_.size(); ++k) {
-        const size_t t = free_sizes_[k].total();
-        if (t > free_sizes_[largest].total())
-            largest = k;
-        if (need && free_sizes_[k].holds(*need) && (i == free_.size() || t < free_sizes_[i].total()))
+    // Sizes kept beside the list so that the choice reads contiguous arrays.
+    size_t i = free_.size();
+    for (size_t k = 0; need && k < free_.size(); ++k)
+        if (free_sizes_[k].holds(*need) && (i == free_.size() || free_bytes_[k] < free_bytes_[i])) {
             i = k;
-    }
+            if (free_sizes_[k].total() == need->total())
+                break;  // none is smaller
+        }
     if (i == free_.size())
-        i = largest;
+        i = (size_t)(std::max_element(free_bytes_.begin(), free_bytes_.end()) - free_bytes_.begin());
     std::unique_ptr<Slot> s = std::move(free_[i]);
     free_[i] = std::move(free_.back());
     free_.pop_back();
+    free_bytes_[i] = free_bytes_.back();
+    free_bytes_.pop_back();
     free_sizes_[i] = free_sizes_.back();
     free_sizes_.pop_back();
     return s;
@@ -459,6 +461,7 @@ std::unique_ptr<Slot> Engine::take_slot(const SlotSizes *need)
 
 void Engine::put_free(std::unique_ptr<Slot> s)
 {
+    free_bytes_.push_back(s->device_bytes());
     free_sizes_.push_back(s->sizes());
     free_.push_back(std::move(s));
 }
