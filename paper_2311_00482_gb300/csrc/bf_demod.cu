@@ -107,7 +107,7 @@ __device__ __forceinline__ void demod_units(const DemodJob &J, int unit0, uint32
 }
 
 template <bool BIG>
-__global__ void __launch_bounds__(BIG ? kDemodBigThreads : kDemodThreads, BIG ? 1 : 2)
+__global__ void __launch_bounds__(BIG ? kDemodBigThreads : kDemodThreads, BIG ? 1 : 3)
     demod16_kernel(const DemodJob *__restrict__ jobs, const int *__restrict__ blk_prefix, int njobs)
 {
     constexpr int THREADS = BIG ? kDemodBigThreads : kDemodThreads;
