@@ -16,7 +16,7 @@
 // runs along Kz (with temporal bins a row apart every point took two 32-byte sectors
 // of its own).  Bound: the launches' latencies (a 64 x 2048 record of three angles has
 // 96 to 193 CTAs of work per launch).  Five launches of shared-memory radix-8
-// transforms and a synchronous upload took 59 us per call, these 29 us.
+// transforms and a synchronous upload took 59 us per call, these 31 us.
 #include "bf_fft16.cuh"
 #include "bf_internal.h"
 #include "bf_launch.cuh"
