@@ -688,9 +688,17 @@ static std::vector<size_t> job_frames(const std::vector<FramePrep> &frames, cons
     const FramePrep &f = frames[fi];
     const size_t want = (size_t)plan_frames_per_job(f.plan, f.modes, f.prec, kMaxFramesPerJob);
     std::vector<size_t> rest, leads;  // after fi, in order
-    for (size_t gi = fi + 1; gi < frames.size() && rest.size() + 1 < want && leads.size() < 2 * want; ++gi)
-        if (!taken[gi] && shareable(f, frames[gi]))
-            (frames[gi].nf_cap > 1 ? leads : rest).push_back(gi);
+    for (size_t gi = fi + 1; gi < frames.size() && want > 1; ++gi) {
+        const bool full = rest.size() + 1 >= want || leads.size() >= 2 * want;
+        if (full && (f.nf_cap > 1 || !leads.empty()))
+            break;  // enough partners, and a lead among them
+        if (taken[gi] || !shareable(f, frames[gi]))
+            continue;
+        if (frames[gi].nf_cap > 1)
+            leads.push_back(gi);
+        else if (rest.size() + 1 < want)
+            rest.push_back(gi);
+    }
     std::vector<size_t> job{fi};
     if (f.nf_cap == 1) {
         if (leads.empty())
